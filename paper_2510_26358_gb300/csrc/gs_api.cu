@@ -253,6 +253,8 @@ gs_status gs_workspace_create(const gs_camera *cams, int32_t n_views, const int6
     k.ext_abs_pad = cfg->ext_abs_pad;
     k.log2_alpha_min = (float)std::log2((double)cfg->alpha_min);
     k.ln_alpha_min = (float)std::log((double)cfg->alpha_min);
+    // (2^e by the approximate instruction is within 2^-22 of itself)
+    k.log2_alpha_noclamp = (float)(std::log2((double)cfg->alpha_max) - 1e-4);
     k.tile_w = cfg->tile_w;
     k.tile_h = cfg->tile_h;
 

@@ -19,12 +19,15 @@
 // thread's pixels and then over the warp with shuffles before one atomic per
 // component.
 //
-// In both passes each thread owns a few vertically adjacent pixels of one
-// column (PF forward, PPT backward): the shared memory loads, the loop
-// overhead, the column part of the exponent and (backward) the warp
-// reduction are paid once per column of pixels.  The backward runs its pixel
-// updates without branches: a pixel that a fragment does not reach takes
-// alpha = 0, for which each update is exactly the identity.
+// In both passes a tile is divided into quadrants of 8x8 pixels, two a lane,
+// and a warp holds one, two or four quadrants.  Of each entry it works only the
+// quadrants that the Gaussian's ellipse reaches and that still have a pixel to
+// blend: the passes are bound by instruction issue (FP32, selects and compares),
+// and of the pixel slots of a walk over whole 16x16 tiles only 43 % blend (4M
+// orchard, six 1920x1200 views; of the quadrants an entry meets 2.55 of 4
+// blend, 2.99 are reached).  Pixel updates run without branches: a pixel that a
+// fragment does not reach takes alpha = 0, for which each update is exactly the
+// identity.
 //
 // The VAR variants also render each pixel's depth distribution under the
 // weights w: its mean mu = sum w z / W and variance var = sum w (z - mu)^2 / W,
@@ -44,6 +47,45 @@
 
 namespace gs {
 namespace {
+
+// Paddings of the quadrant test (see quad_mask).
+constexpr float kQuadRelPad = 1e-3f, kQuadAbsPad = 1e-2f;
+
+// Entries staged at a time, at most (the configuration's batch depth below
+// it): with 64 the staged entries of 20 one-warp CTAs fit an SM.
+constexpr int kFwdDepth = 64, kBwdDepth = 64;
+
+// How many quadrants a warp takes, by the number of 16x16 tiles (or as many
+// pixels).  Whole tiles share the most work between quadrants but make the
+// fewest warps: with few tiles the time is the longest list's chain of
+// entries, which is shorter the less a warp does for each.  Measured (one,
+// two, four quadrants a warp, us), orchard of 200k: forward, 88 tiles (box of 3k)
+// 28, 41, -; 300 tiles 63, 58, 101; 3600 41, 38, 55; 7200 87, 64, 75; 1M, 24,480 tiles -, 391, 406; 4M,
+// 54,000 tiles -, 971, 936.  Backward, 300 tiles 93, 111, 186; 2400 95, 102,
+// 143; 3600 59, 59, 86; 7200 171, 130, 124.  With the variance (one, two; more
+// do not fit the registers) forward, 2400 tiles 73, 97; 7200 139, 107; backward
+// 104, 108; 186, 153.
+constexpr int kCoarseTiles = 152 * 24;     // backward, and forward with the variance
+constexpr int kFwdHalfTiles = 152, kFwdWholeTiles = 152 * 256;  // forward
+
+// Resident warps an SM that each variant's registers are bounded for, as CTAs
+// (forward, 4M orchard: 20 warps of whole tiles 0.94 ms, 24 0.99 ms with spills,
+// 16 1.23 ms; backward: 16 warps 1.61 ms, 12 1.95 ms).
+constexpr int fwd_blocks(int warps, int q, bool var) {
+    return (var ? (q == 4 ? 16 : 20) : (q == 4 ? 20 : q == 2 ? 28 : 40)) / warps;
+}
+
+constexpr int bwd_blocks(int warps, int q, bool var) { return (q == 1 ? 24 : 16) / warps; }
+
+// One step of the weighted Welford update (the VAR variants).
+__device__ __forceinline__ void welford(float w, float z, bool first, float &W, float &zc, float &m, float &M2) {
+    if (first) zc = z;
+    W = __fadd_rn(W, w);
+    const float y = z - zc;
+    const float d = y - m;
+    m = __fmaf_rn(d, __fdividef(w, W), m);
+    M2 = __fmaf_rn(__fmul_rn(w, d), y - m, M2);
+}
 
 struct RasterArgs {
     const ViewInfo *views;
@@ -66,15 +108,358 @@ struct RasterArgs {
     float *g2d;
 };
 
-// One CTA works a tile at a time (persistent, tiles taken in the work order);
-// a thread holds PF vertically adjacent pixels of one column, which share the
+// A tile is divided into quadrants of 8x8 pixels, two a lane: lane l holds
+// column l % 8 and rows l / 8 and l / 8 + 4 of each of its quadrants, packed
+// in one f32x2 pair.  A warp holds Q quadrants (4: a 16x16 tile; 2: a 16x8
+// half; 1), which share the row and the column terms of every exponent.
+template <int TW, int TH, int Q>
+struct Share {
+    static constexpr int QX = Q >= 2 ? 2 : 1, QY = Q == 4 ? 2 : 1;
+    static constexpr int NWX = TW / (8 * QX);            // warps across
+    static constexpr int NW = NWX * (TH / (8 * QY));     // warps a tile
+    static constexpr int NT = 32 * NW;
+    static_assert(TW % (8 * QX) == 0 && TH % (8 * QY) == 0 && NW * Q <= 16, "whole warps a tile");
+    // first pixel of warp w's share, relative to the tile
+    __device__ static constexpr int wx(int w) { return (w % NWX) * 8 * QX; }
+    __device__ static constexpr int wy(int w) { return (w / NWX) * 8 * QY; }
+};
+
+// Which quadrants a staged Gaussian can reach, bit w * Q + q for quadrant q
+// of warp w: the tile test of the binning on the quadrant's box of pixel
+// centres, with fixed paddings (0.1 % and 0.01 px) that exceed the rounding of
+// the exponents below, so an unset bit is a quadrant without a fragment to
+// keep.  kExactPath marks an entry whose fragments must take every branch:
+// one whose alpha may need the clamp at alpha_max, or with a value that is
+// not finite (0 x inf would leak into pixels that it does not reach).
+constexpr uint32_t kExactPath = 0x80000000u;
+template <int TW, int TH, int Q>
+__device__ __forceinline__ uint32_t quad_mask(const float4 r0, const float4 r1, const float4 r2, int x0, int y0,
+                                              const Consts &k) {
+    using S = Share<TW, TH, Q>;
+    float f = r0.x * 0.f + r0.y * 0.f + r0.z * 0.f + r0.w * 0.f;
+    f += r1.x * 0.f + r1.y * 0.f + r1.z * 0.f + r1.w * 0.f;
+    f += r2.x * 0.f + r2.y * 0.f + r2.z * 0.f + r2.w * 0.f;
+    if (!(f == 0.f)) return ~0u;
+    const float4 t = reach_terms(r1, k.log2_alpha_min, 1.f + kQuadRelPad);
+    uint32_t m = r1.w < k.log2_alpha_noclamp ? 0u : kExactPath;
+#pragma unroll
+    for (int w = 0; w < S::NW; ++w)
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            const int x = x0 + S::wx(w) + 8 * (q % S::QX), y = y0 + S::wy(w) + 8 * (q / S::QX);
+            if (tile_reached(r0, r1, t, x, x + 7, y, y + 7, kQuadAbsPad)) m |= 1u << (w * Q + q);
+        }
+    return m;
+}
+
+// One staged list entry of the forward: what the packed arithmetic multiplies
+// a pair of pixels by is stored twice, side by side, so that one 16-byte
+// shared load gives two packed operands (broadcasting a register into a pair
+// costs an instruction for every operand).
+struct FwdEntry {
+    float4 u;    // U, l11, k1
+    float4 row;  // V, V, k2, k2
+    float4 l;    // l12, l12, l22, l22
+    float4 or_;  // -log2 o twice, -r twice
+    float4 gb;   // -g twice, -b twice
+    float4 z;    // -z twice
+};
+struct F2x2 {
+    f2 a, b;
+};
+__device__ __forceinline__ F2x2 load_f2x2(const float4 &v) {
+    const ulonglong2 x = *reinterpret_cast<const ulonglong2 *>(&v);
+    return {{x.x}, {x.y}};
+}
+
+// One CTA works a tile at a time (persistent, tiles taken in the work order).
+// Each warp walks, of every 32 staged entries, those that reach one of its
+// quadrants that still has a live pixel (one ballot a quadrant), and of such an
+// entry only the quadrants it reaches: of the pixel slots of a 16x16 tile's
+// walk 45 % blend, of those worked here 60 %.  A pixel stops at the first
+// fragment that would take its transmittance below t_min (its threshold thr
+// then admits nothing), the warp when all of its pixels have, the CTA when all
+// warps have.
+//
+// Within a quadrant the two pixels of a lane are worked without branches: a
+// pixel that the fragment does not reach takes alpha = 0, for which T - T
+// alpha and C + T alpha c are exactly T and C.  alpha is carried negated, as
+// packed instructions cannot negate, and so is the staged colour.  Decisions
+// and sums round exactly as e = log2 o - t1^2 - t2^2, alpha = min(alpha_max,
+// 2^e), T' = fma(-T, alpha, T), C' = fma(T alpha, c, C) taken one by one.
+// (Against two warps a tile, four pixels a thread with a branch each: 4M
+// orchard, six 1920x1200 views, 1151 -> 936 us; three 1280x720 views of 500k
+// 194 -> 172; 161x119, 3k 52 -> 28.)
+template <int TW, int TH, int Q, bool VAR>
+__global__ void __launch_bounds__(Share<TW, TH, Q>::NT, fwd_blocks(Share<TW, TH, Q>::NW, Q, VAR))
+    k_raster_fwd(RasterArgs A) {
+    using S = Share<TW, TH, Q>;
+    constexpr int QX = S::QX, QY = S::QY, NW = S::NW, NT = S::NT;
+    extern __shared__ float4 smem[];
+    FwdEntry *sE = reinterpret_cast<FwdEntry *>(smem);
+    uint32_t *sM = reinterpret_cast<uint32_t *>(sE + A.depth);
+    __shared__ int s_tile;
+    const int tid = threadIdx.x, lane = tid & 31, wid = NW > 1 ? tid >> 5 : 0;
+    const float amax = A.c.alpha_max, tmin = A.c.t_min, l2amin = A.c.log2_alpha_min;
+    for (;;) {
+        __syncthreads();
+        if (tid == 0) {
+            const uint32_t w = atomicAdd(A.counter, 1u);
+            s_tile = w < (uint32_t)A.n_tiles ? (int)A.order[w] : -1;
+        }
+        __syncthreads();
+        const int tile = s_tile;
+        if (tile < 0) break;
+        const int v = view_of_tile(A.views, A.n_views, tile);
+        const ViewInfo vi = A.views[v];
+        const int lt = tile - vi.tile_off;
+        const int tx0 = (lt % vi.ntx) * TW, ty0 = (lt / vi.ntx) * TH;
+        const int px0 = tx0 + S::wx(wid) + (lane & 7), py0 = ty0 + S::wy(wid) + (lane >> 3);
+        const uint2 rg = A.ranges[tile];
+        f2 T[Q], Cr[Q], Cg[Q], Cb[Q], D[Q];
+        float thr[Q][2];  // -log2 alpha_min while the pixel lives, then -inf
+        uint32_t cnt[Q][2];
+        float Wsum[Q][2], zc[Q][2], mr[Q][2], M2[Q][2];
+        uint32_t live = 0;  // bit q: quadrant q has a live pixel
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            T[q] = f2_bcast(1.f);
+            Cr[q] = Cg[q] = Cb[q] = D[q] = f2_bcast(0.f);
+            const int px = px0 + 8 * (q % QX), py = py0 + 8 * (q / QX);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                Wsum[q][h] = zc[q][h] = mr[q][h] = M2[q][h] = 0.f;
+                cnt[q][h] = 0;
+                thr[q][h] = px < vi.W && py + 4 * h < vi.H ? -l2amin : -INFINITY;
+            }
+            if (__any_sync(0xffffffffu, fmaxf(thr[q][0], thr[q][1]) > -INFINITY)) live |= 1u << q;
+        }
+        for (uint32_t b0 = rg.x; b0 < rg.y; b0 += A.depth) {
+            if (__syncthreads_and(live == 0)) break;
+            const int nb = min((int)(rg.y - b0), A.depth);
+            for (int j = tid; j < nb; j += NT) {
+                const uint32_t pair = A.vals[b0 + j];
+                const float4 r0 = A.rec[3 * (size_t)pair], r1 = A.rec[3 * (size_t)pair + 1];
+                const float4 r2 = A.rec[3 * (size_t)pair + 2];
+                float4 a, b;
+                stage_record(r0, r1, a, b);
+                sE[j].u = make_float4(a.x, b.x, a.z, 0.f);
+                sE[j].row = make_float4(a.y, a.y, a.w, a.w);
+                sE[j].l = make_float4(b.y, b.y, b.z, b.z);
+                sE[j].or_ = make_float4(-b.w, -b.w, -r2.x, -r2.x);
+                sE[j].gb = make_float4(-r2.y, -r2.y, -r2.z, -r2.z);
+                sE[j].z = make_float4(-r2.w, -r2.w, 0.f, 0.f);
+                sM[j] = quad_mask<TW, TH, Q>(r0, r1, r2, tx0, ty0, A.c);
+            }
+            __syncthreads();
+            for (int jb = 0; jb < nb && live; jb += 32) {
+                const uint32_t mine = jb + lane < nb ? sM[jb + lane] : 0u;
+                uint32_t E[Q], todo = 0, all = ~0u;
+                const uint32_t exact = __ballot_sync(0xffffffffu, mine & kExactPath);
+#pragma unroll
+                for (int q = 0; q < Q; ++q) {
+                    E[q] = __ballot_sync(0xffffffffu, (mine >> (wid * Q + q)) & 1u);
+                    if (!(live >> q & 1u)) E[q] = 0;
+                    todo |= E[q];
+                    all &= E[q];
+                }
+                int since = 0;
+                while (todo) {
+                    const int j = __ffs(todo) - 1;
+                    todo &= todo - 1;
+                    const FwdEntry &e = sE[jb + j];
+                    const uint32_t j1 = b0 + jb + j - rg.x + 1;
+                    const float4 u = e.u;
+                    const F2x2 row = load_f2x2(e.row), l = load_f2x2(e.l), o = load_f2x2(e.or_);
+                    f2 U1[QX], DY[QY], IN[QY];
+#pragma unroll
+                    for (int x = 0; x < QX; ++x)
+                        U1[x] = f2_bcast(__fmaf_rn(u.y, __fsub_rn((float)(px0 + 8 * x), u.x), u.z));
+#pragma unroll
+                    for (int y = 0; y < QY; ++y) {
+                        DY[y] = f2_sub(f2_pack((float)(py0 + 8 * y), (float)(py0 + 8 * y + 4)), row.a);
+                        const f2 t2 = f2_fma(l.b, DY[y], row.b);
+                        IN[y] = f2_fma(t2, t2, o.a);
+                    }
+                    if (!(exact >> j & 1u)) {
+                        const F2x2 gb = load_f2x2(e.gb), z = load_f2x2(e.z);
+                        float al[Q][2], tn[Q][2];  // -alpha, the transmittance after
+                        bool in[Q][2];
+                        auto decide = [&](int q) {
+                            const f2 t1 = f2_fma(l.a, DY[q / QX], U1[q % QX]);
+                            float n[2];  // -e
+                            f2_unpack(f2_fma(t1, t1, IN[q / QX]), n[0], n[1]);
+#pragma unroll
+                            for (int h = 0; h < 2; ++h) {
+                                in[q][h] = n[h] <= thr[q][h];
+                                al[q][h] = in[q][h] ? -ex2_approx(-n[h]) : 0.f;
+                            }
+                            f2_unpack(f2_fma(T[q], f2_pack(al[q][0], al[q][1]), T[q]), tn[q][0], tn[q][1]);
+                        };
+                        auto stop = [&](int q) {
+#pragma unroll
+                            for (int h = 0; h < 2; ++h)
+                                if (tn[q][h] < tmin) {
+                                    thr[q][h] = -INFINITY;
+                                    al[q][h] = 0.f;
+                                    in[q][h] = false;
+                                }
+                        };
+                        auto blend = [&](int q) {
+                            const f2 nal = f2_pack(al[q][0], al[q][1]);
+                            const f2 nw = f2_mul(nal, T[q]);
+                            T[q] = f2_fma(T[q], nal, T[q]);
+                            Cr[q] = f2_fma(nw, o.b, Cr[q]);
+                            Cg[q] = f2_fma(nw, gb.a, Cg[q]);
+                            Cb[q] = f2_fma(nw, gb.b, Cb[q]);
+                            D[q] = f2_fma(nw, z.a, D[q]);
+                            if (VAR) {
+                                float w[2];
+                                f2_unpack(nw, w[0], w[1]);
+#pragma unroll
+                                for (int h = 0; h < 2; ++h)
+                                    if (in[q][h])
+                                        welford(-w[h], -f2_lo(z.a), cnt[q][h] == 0, Wsum[q][h], zc[q][h], mr[q][h],
+                                                M2[q][h]);
+                            }
+#pragma unroll
+                            for (int h = 0; h < 2; ++h)
+                                if (in[q][h]) cnt[q][h] = j1;
+                        };
+                        if (Q > 1 && (all >> j & 1u)) {
+                            // every quadrant, interleaved and with one test for
+                            // pixels that end (972 -> 936 us, 4M orchard)
+                            float low = 1.f;
+#pragma unroll
+                            for (int q = 0; q < Q; ++q) {
+                                decide(q);
+                                low = fminf(low, fminf(tn[q][0], tn[q][1]));
+                            }
+                            if (low < tmin) {
+#pragma unroll
+                                for (int q = 0; q < Q; ++q) stop(q);
+                            }
+#pragma unroll
+                            for (int q = 0; q < Q; ++q) blend(q);
+                        } else {
+#pragma unroll
+                            for (int q = 0; q < Q; ++q)
+                                if (E[q] >> j & 1u) {
+                                    decide(q);
+                                    if (fminf(tn[q][0], tn[q][1]) < tmin) stop(q);
+                                    blend(q);
+                                }
+                        }
+                    } else {
+                        const float cx = e.or_.z, cy = e.gb.x, cz = e.gb.z, cw = e.z.x;
+#pragma unroll
+                        for (int q = 0; q < Q; ++q) {
+                            if (!(E[q] >> j & 1u)) continue;
+                            const f2 t1 = f2_fma(l.a, DY[q / QX], U1[q % QX]);
+                            float n[2];
+                            f2_unpack(f2_fma(t1, t1, IN[q / QX]), n[0], n[1]);
+                            float t[2], cr[2], cg[2], cb[2], d[2];
+                            f2_unpack(T[q], t[0], t[1]);
+                            f2_unpack(Cr[q], cr[0], cr[1]);
+                            f2_unpack(Cg[q], cg[0], cg[1]);
+                            f2_unpack(Cb[q], cb[0], cb[1]);
+                            f2_unpack(D[q], d[0], d[1]);
+#pragma unroll
+                            for (int h = 0; h < 2; ++h) {
+                                // (an exponent that is not a number is not below the threshold)
+                                if (!(thr[q][h] > -INFINITY) || -n[h] < l2amin) continue;
+                                const float alpha = fminf(amax, ex2_approx(-n[h]));
+                                const float tn = __fmaf_rn(-t[h], alpha, t[h]);
+                                if (tn < tmin) {
+                                    thr[q][h] = -INFINITY;
+                                    continue;
+                                }
+                                const float w = __fmul_rn(alpha, t[h]);
+                                cr[h] = __fmaf_rn(w, -cx, cr[h]);
+                                cg[h] = __fmaf_rn(w, -cy, cg[h]);
+                                cb[h] = __fmaf_rn(w, -cz, cb[h]);
+                                d[h] = __fmaf_rn(w, -cw, d[h]);
+                                if (VAR) welford(w, -cw, cnt[q][h] == 0, Wsum[q][h], zc[q][h], mr[q][h], M2[q][h]);
+                                t[h] = tn;
+                                cnt[q][h] = j1;
+                            }
+                            T[q] = f2_pack(t[0], t[1]);
+                            Cr[q] = f2_pack(cr[0], cr[1]);
+                            Cg[q] = f2_pack(cg[0], cg[1]);
+                            Cb[q] = f2_pack(cb[0], cb[1]);
+                            D[q] = f2_pack(d[0], d[1]);
+                        }
+                    }
+                    // quadrants whose pixels have all ended leave the walk
+                    if (++since == 8) {
+                        since = 0;
+                        uint32_t left = 0;
+#pragma unroll
+                        for (int q = 0; q < Q; ++q) {
+                            if (!__any_sync(0xffffffffu, fmaxf(thr[q][0], thr[q][1]) > -INFINITY)) {
+                                E[q] = 0;
+                                live &= ~(1u << q);
+                            }
+                            left |= E[q];
+                            all &= E[q];
+                        }
+                        todo &= left;
+                    }
+                }
+            }
+        }
+        const int64_t hw = (int64_t)vi.W * vi.H;
+        float *rgb = A.rgb + 3 * (int64_t)vi.pix_off;
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            const int px = px0 + 8 * (q % QX);
+            float t[2], cr[2], cg[2], cb[2], d[2];
+            f2_unpack(T[q], t[0], t[1]);
+            f2_unpack(Cr[q], cr[0], cr[1]);
+            f2_unpack(Cg[q], cg[0], cg[1]);
+            f2_unpack(Cb[q], cb[0], cb[1]);
+            f2_unpack(D[q], d[0], d[1]);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int py = py0 + 8 * (q / QX) + 4 * h;
+                if (px >= vi.W || py >= vi.H) continue;
+                const int64_t pl = (int64_t)py * vi.W + px;
+                const int64_t pix = vi.pix_off + pl;
+                rgb[pl] = cr[h];
+                rgb[hw + pl] = cg[h];
+                rgb[2 * hw + pl] = cb[h];
+                A.depth_out[pix] = d[h];
+                // 1 - T loses the relative precision of a small alpha (T near 1);
+                // the variance variant has the direct sum of the weights at hand,
+                // which keeps it, as the normalised depth D / alpha needs
+                A.alpha_out[pix] = VAR ? Wsum[q][h] : 1.f - t[h];
+                A.last[pix] = cnt[q][h];
+                A.tfin[pix] = t[h];
+                if (VAR) {
+                    const float mean = zc[q][h] + mr[q][h];
+                    const float iw = Wsum[q][h] > 0.f ? 1.f / Wsum[q][h] : 0.f;
+                    const float var = M2[q][h] * iw;
+                    A.mean_out[pix] = mean;
+                    A.var_out[pix] = var;
+                    A.vstat[pix] = make_float4(mean, var, iw, 0.f);
+                }
+            }
+        }
+    }
+}
+
+// The forward of an 8x8 tile, which is one quadrant: its list holds what
+// reaches it already, so there is nothing to skip, and two pixels a lane
+// with a branch each are cheaper than the packed pairs of k_raster_fwd (three
+// 1280x720 views of a 500k orchard: 0.169 ms here, 0.217 there; with the
+// variance 0.266 and 0.332).  A thread holds PF vertically adjacent pixels of one column, which share the
 // shared-memory reads and the column part of every fragment's exponent.  A
 // pixel stops at the first fragment that would take its transmittance below
 // t_min, the thread when all of its pixels have, the CTA when all threads have.
 // The VAR variant holds four more values a pixel: at least 640 resident
 // threads an SM keeps it at 96 registers without spills (0: no minimum).
 template <int TW, int TH, int PF, bool VAR>
-__global__ void __launch_bounds__(TW * TH / PF, VAR ? 640 / (TW * TH / PF) : 0) k_raster_fwd(RasterArgs A) {
+__global__ void __launch_bounds__(TW * TH / PF, VAR ? 640 / (TW * TH / PF) : 0) k_raster_fwd_columns(RasterArgs A) {
     constexpr int NT = TW * TH / PF;
     static_assert(NT % 32 == 0, "the forward needs whole warps");
     extern __shared__ float4 smem[];
@@ -141,20 +526,13 @@ __global__ void __launch_bounds__(TW * TH / PF, VAR ? 640 / (TW * TH / PF) : 0) 
                         --nlive;
                         continue;
                     }
-                    const float wgt = al * T[i];
+                    const float wgt = __fmul_rn(al, T[i]);
                     const float4 c = sC[j];
                     Cr[i] = __fmaf_rn(wgt, c.x, Cr[i]);
                     Cg[i] = __fmaf_rn(wgt, c.y, Cg[i]);
                     Cb[i] = __fmaf_rn(wgt, c.z, Cb[i]);
                     D[i] = __fmaf_rn(wgt, c.w, D[i]);
-                    if (VAR) {
-                        if (cnt[i] == 0) zc[i] = c.w;
-                        Wsum[i] += wgt;
-                        const float y = c.w - zc[i];
-                        const float d = y - mr[i];
-                        mr[i] = __fmaf_rn(d, __fdividef(wgt, Wsum[i]), mr[i]);
-                        M2[i] = __fmaf_rn(wgt * d, y - mr[i], M2[i]);
-                    }
+                    if (VAR) welford(wgt, c.w, cnt[i] == 0, Wsum[i], zc[i], mr[i], M2[i]);
                     T[i] = Tn;
                     cnt[i] = b0 + j - rg.x + 1;
                 }
@@ -190,87 +568,103 @@ __global__ void __launch_bounds__(TW * TH / PF, VAR ? 640 / (TW * TH / PF) : 0) 
     }
 }
 
-// Sums ten per-lane values over the warp by recursive halving: at each of the
-// five butterfly levels a lane keeps half of its remaining components and
-// sends the other half to its partner, so 12 shuffles replace 50.  Afterwards
-// lane l holds the warp total of component
-//   comp(l) = 5*b4 + 3*b3 + 2*b2 + b1      (bK = bit K of l),
-// valid when (b3 == 0 and not (b2 and b1)) or (b3 == 1 and b2 == 0); lanes l
-// and l^1 hold the same total.  reduce10_component gives comp(l) or -1.
-__device__ __forceinline__ float warp_reduce_scatter10(const float v[10], int lane) {
-    const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4, b1 = lane & 2;
-    float a[5];
-#pragma unroll
-    for (int i = 0; i < 5; ++i) {
-        float send = b4 ? v[i] : v[i + 5];
-        float keep = b4 ? v[i + 5] : v[i];
-        a[i] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
-    }
-    float c[3];
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-        float hiv = i + 3 < 5 ? a[i + 3] : 0.f;
-        float send = b3 ? a[i] : hiv;
-        float keep = b3 ? hiv : a[i];
-        c[i] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
-    }
-    float d[2];
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-        float hiv = i + 2 < 3 ? c[i + 2] : 0.f;
-        float send = b2 ? c[i] : hiv;
-        float keep = b2 ? hiv : c[i];
-        d[i] = keep + __shfl_xor_sync(0xffffffffu, send, 4);
-    }
-    float send = b1 ? d[0] : d[1];
-    float keep = b1 ? d[1] : d[0];
-    float e = keep + __shfl_xor_sync(0xffffffffu, send, 2);
-    return e + __shfl_xor_sync(0xffffffffu, e, 1);
+// One staged list entry of the backward (see FwdEntry).
+struct BwdEntry {
+    float4 u;    // U, l11, k1, hx
+    float4 row;  // V, V, k2, k2
+    float4 l;    // l12, l12, l22, l22
+    float4 or_;  // -log2 o twice, r twice
+    float4 gb;   // g twice, b twice
+    float4 z;    // z twice, hy, pair (bits)
+};
+
+// Warp sums of the ten image-space components go through shared memory: each
+// lane stores its ten values of an entry as one row of kSumRow floats, and
+// once kSumSlots entries are pending the warp sums them together, a lane adding
+// one 16-byte column over half of the rows.  (Against a butterfly of
+// shuffles an entry at a time, 12 shuffles and some 35 selects and adds, an
+// entry takes 3 shared stores, 4 loads and 8 packed adds.)  The row stride of
+// 12 floats and the rotated row order below keep stores and loads free of
+// bank conflicts.
+constexpr int kSumSlots = 4, kSumRow = 12;
+constexpr int kSumBytes = kSumSlots * 32 * kSumRow * (int)sizeof(float);
+
+__device__ __forceinline__ void red_add2(float *p, float a, float b) {
+    asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" ::"l"(p), "f"(a), "f"(b) : "memory");
 }
 
-__device__ __forceinline__ int reduce10_component(int lane) {
-    const int b4 = (lane >> 4) & 1, b3 = (lane >> 3) & 1, b2 = (lane >> 2) & 1, b1 = (lane >> 1) & 1;
-    const bool ok = b3 == 0 ? !(b2 && b1) : b2 == 0;
-    return ok ? 5 * b4 + 3 * b3 + 2 * b2 + b1 : -1;
+// Adds the n pending entries' sums to their pairs' gradient rows; byte k of
+// `which` is the staged index of slot k.
+__device__ __forceinline__ void flush_sums(const float *sum, const BwdEntry *sE, int n, uint32_t which, int lane,
+                                           float *g2d) {
+    __syncwarp();
+    // lane = 8 f + 2 slot + half: column f (components 4f .. 4f + 3) of a slot's rows 16 half .. 16 half + 15
+    const int f = lane >> 3, turn = lane & 7, slot = turn >> 1, half = lane & 1;
+    const bool active = f < 3 && slot < n;
+    f2 v[4][2];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k][0] = v[k][1] = f2_bcast(0.f);
+    if (active) {
+        const float *col = sum + (slot * 32 + 16 * half) * kSumRow + 4 * f;
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            const F2x2 x = load_f2x2(*reinterpret_cast<const float4 *>(col + ((i + turn) & 15) * kSumRow));
+            v[i & 3][0] = i < 4 ? x.a : f2_add(v[i & 3][0], x.a);
+            v[i & 3][1] = i < 4 ? x.b : f2_add(v[i & 3][1], x.b);
+        }
+    }
+    float4 t;
+    f2_unpack(f2_add(f2_add(v[0][0], v[1][0]), f2_add(v[2][0], v[3][0])), t.x, t.y);
+    f2_unpack(f2_add(f2_add(v[0][1], v[1][1]), f2_add(v[2][1], v[3][1])), t.z, t.w);
+    t.x += __shfl_xor_sync(0xffffffffu, t.x, 1);
+    t.y += __shfl_xor_sync(0xffffffffu, t.y, 1);
+    t.z += __shfl_xor_sync(0xffffffffu, t.z, 1);
+    t.w += __shfl_xor_sync(0xffffffffu, t.w, 1);
+    if (active) {
+        // the raw sums are negated (dpw and the weights are carried negated);
+        // dL/dQ = -1/2 sum gpw d d^T; dpw/du = (Q d)_x = l11 t1 / s^2,
+        // dpw/dv = (l12 t1 + l22 t2) / s^2 with 1/s^2 = 2 ln 2
+        const BwdEntry &e = sE[which >> (8 * slot) & 255u];
+        float *gp = g2d + (size_t)__float_as_uint(e.z.w) * kGrad + 4 * f;
+        if (f == 0) {
+            if (half == 0) red_add2(gp, -kTwoLn2 * (e.u.y * t.x), -kTwoLn2 * __fmaf_rn(e.l.x, t.x, e.l.z * t.y));
+            else red_add2(gp + 2, 0.5f * t.z, t.w);
+        } else if (f == 1) {
+            if (half == 0) red_add2(gp, 0.5f * t.x, -t.y);
+            else red_add2(gp + 2, -t.z, -t.w);
+        } else if (half == 0) {
+            red_add2(gp, -t.x, -t.y);
+        }
+    }
+    __syncwarp();
 }
 
-// At least 512 resident threads per SM (16 warps, 128 registers a thread):
-// with eight pixels a thread, measured best on the 500k orchard (16 one-warp
-// blocks: 0.435 ms; 14: 0.441 ms).
-//
-// A thread's PPT pixels are worked in Q = PPT/2 packed pairs (pixel p in the
-// low half, pixel p + Q in the high half), so that one f32x2 instruction does
-// the arithmetic of two pixels.  The alpha decision is taken on
+// Back to front over each tile's list, with the forward's division of a tile
+// into quadrants and its masks; a quadrant joins the walk at the last entry
+// that one of its pixels blended.  A pixel that a fragment does not reach
+// takes alpha = 0 and runs the same instructions, which are then exactly the
+// identity (T * 1, acc + 0 * h, sums + 0; the reciprocal approximation
+// returns 1 for 1 on sm_103, measured).  The alpha decision is taken on
 // -e = fma(t1, t1, fma(t2, t2, -log2 o)), which is exactly the negation of
-// the forward's e = fma(-t1, t1, fma(-t2, t2, log2 o)) (round to nearest is
-// symmetric), so both passes take the same decisions bit for bit.
-template <int TW, int TH, int PPT, bool VAR>
-__global__ void __launch_bounds__(TW * TH / PPT, 512 / (TW * TH / PPT)) k_raster_bwd(RasterArgs A) {
-    constexpr int NT = TW * TH / PPT;
-    static_assert(NT % 32 == 0, "the backward needs whole warps");
-    static_assert(PPT % 2 == 0, "the backward works pixels in pairs");
-    constexpr int NW = (NT + 31) / 32;
-    constexpr int Q = PPT / 2;
+// e = fma(-t1, t1, fma(-t2, t2, log2 o)) (round to nearest is symmetric), so
+// both passes take the same decisions bit for bit.
+// (Against one warp a tile, a thread a column of eight pixels and a butterfly
+// of shuffles an entry: 4M orchard, six 1920x1200 views, 1841 -> 1606 us; three
+// 1280x720 views of 500k 322 -> 281; 320x240, 10k 213 -> 99.)
+template <int TW, int TH, int Q, bool VAR>
+__global__ void __launch_bounds__(Share<TW, TH, Q>::NT, bwd_blocks(Share<TW, TH, Q>::NW, Q, VAR))
+    k_raster_bwd(RasterArgs A) {
+    using S = Share<TW, TH, Q>;
+    constexpr int QX = S::QX, QY = S::QY, NW = S::NW, NT = S::NT;
     extern __shared__ float4 smem[];
-    float4 *sA = smem, *sB = smem + A.depth, *sC = smem + 2 * A.depth;
-    float2 *sH = reinterpret_cast<float2 *>(smem + 3 * A.depth);
-    uint32_t *sP = reinterpret_cast<uint32_t *>(sH + A.depth);
+    BwdEntry *sE = reinterpret_cast<BwdEntry *>(smem);
+    uint32_t *sM = reinterpret_cast<uint32_t *>(sE + A.depth);
+    float *sums = reinterpret_cast<float *>(sM + A.depth) + (NW > 1 ? (threadIdx.x >> 5) * (kSumBytes / 4) : 0);
     __shared__ int s_tile;
     __shared__ uint32_t s_max[NW];
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int tid = threadIdx.x, lane = tid & 31, wid = NW > 1 ? tid >> 5 : 0;
     const float amax = A.c.alpha_max, nl2amin = -A.c.log2_alpha_min;
-    const f2 ONE = f2_bcast(1.f);
-    // component this lane adds after the reduction (even lanes only), and the
-    // factors c0 + c11 l11 + c22 l22 that turn its raw sum into the gradient
-    // (the colour and depth sums come out negated, see below)
-    const int my_comp = (lane & 1) ? -1 : reduce10_component(lane);
-    const float sc0 = my_comp == G_QA || my_comp == G_QC ? -0.5f
-                      : my_comp == G_QB                  ? -1.f
-                      : my_comp == G_U || my_comp == G_V ? 0.f
-                      : my_comp == G_LNO                 ? 1.f
-                                                         : -1.f;
-    const float sc11 = my_comp == G_U ? kTwoLn2 : 0.f;
-    const float sc22 = my_comp == G_V ? kTwoLn2 : 0.f;
+    const f2 ONE = f2_bcast(1.f), ZERO = f2_bcast(0.f);
     for (;;) {
         __syncthreads();
         if (tid == 0) {
@@ -283,29 +677,28 @@ __global__ void __launch_bounds__(TW * TH / PPT, 512 / (TW * TH / PPT)) k_raster
         const int v = view_of_tile(A.views, A.n_views, tile);
         const ViewInfo vi = A.views[v];
         const int lt = tile - vi.tile_off;
-        const int px = (lt % vi.ntx) * TW + tid % TW;
-        const int py0 = (lt / vi.ntx) * TH + (tid / TW) * PPT;
-        const float pxf = (float)px;
-        const f2 PY0 = f2_pack((float)py0, (float)(py0 + Q));
+        const int tx0 = (lt % vi.ntx) * TW, ty0 = (lt / vi.ntx) * TH;
+        const int px0 = tx0 + S::wx(wid) + (lane & 7), py0 = ty0 + S::wy(wid) + (lane >> 3);
         const uint2 rg = A.ranges[tile];
         const int64_t hw = (int64_t)vi.W * vi.H;
         const float *grgb = A.dL_drgb + 3 * (int64_t)vi.pix_off;
-        uint32_t cnt[PPT], mycnt = 0;
+        uint32_t cnt[Q][2], qmax[Q], wmax = 0;
         f2 T[Q], gR[Q], gG[Q], gB[Q], gD[Q], gA[Q], nacc[Q];  // nacc = -acc
         f2 zmu[Q], ga[Q], gb[Q];
 #pragma unroll
-        for (int p = 0; p < Q; ++p) {
+        for (int q = 0; q < Q; ++q) {
             float t_[2], r_[2], g_[2], b_[2], d_[2], a_[2], z_[2], ma_[2], mb_[2];
+            const int px = px0 + 8 * (q % QX);
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
-                const int i = p + h * Q, py = py0 + i;
-                cnt[i] = 0;
+                const int py = py0 + 8 * (q / QX) + 4 * h;
+                cnt[q][h] = 0;
                 t_[h] = 1.f;
                 r_[h] = g_[h] = b_[h] = d_[h] = a_[h] = z_[h] = ma_[h] = mb_[h] = 0.f;
                 if (px < vi.W && py < vi.H) {
                     const int64_t pl = (int64_t)py * vi.W + px;
                     const int64_t pix = vi.pix_off + pl;
-                    cnt[i] = A.last[pix];
+                    cnt[q][h] = A.last[pix];
                     t_[h] = A.tfin[pix];
                     r_[h] = grgb[pl];
                     g_[h] = grgb[hw + pl];
@@ -320,177 +713,186 @@ __global__ void __launch_bounds__(TW * TH / PPT, 512 / (TW * TH / PPT)) k_raster
                         a_[h] = __fmaf_rn(-mb_[h], vs.y, a_[h]);  // the -b var part of every h
                     }
                 }
-                mycnt = max(mycnt, cnt[i]);
             }
-            T[p] = f2_pack(t_[0], t_[1]);
-            gR[p] = f2_pack(r_[0], r_[1]);
-            gG[p] = f2_pack(g_[0], g_[1]);
-            gB[p] = f2_pack(b_[0], b_[1]);
-            gD[p] = f2_pack(d_[0], d_[1]);
-            gA[p] = f2_pack(a_[0], a_[1]);
-            nacc[p] = f2_bcast(0.f);
+            qmax[q] = __reduce_max_sync(0xffffffffu, max(cnt[q][0], cnt[q][1]));
+            wmax = max(wmax, qmax[q]);
+            T[q] = f2_pack(t_[0], t_[1]);
+            gR[q] = f2_pack(r_[0], r_[1]);
+            gG[q] = f2_pack(g_[0], g_[1]);
+            gB[q] = f2_pack(b_[0], b_[1]);
+            gD[q] = f2_pack(d_[0], d_[1]);
+            gA[q] = f2_pack(a_[0], a_[1]);
+            nacc[q] = ZERO;
             if (VAR) {
-                zmu[p] = f2_pack(z_[0], z_[1]);
-                ga[p] = f2_pack(ma_[0], ma_[1]);
-                gb[p] = f2_pack(mb_[0], mb_[1]);
+                zmu[q] = f2_pack(z_[0], z_[1]);
+                ga[q] = f2_pack(ma_[0], ma_[1]);
+                gb[q] = f2_pack(mb_[0], mb_[1]);
             }
         }
-        uint32_t wmax = mycnt;
+        uint32_t maxcnt = wmax;
+        if constexpr (NW > 1) {
+            if (lane == 0) s_max[wid] = wmax;
+            __syncthreads();
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) wmax = max(wmax, __shfl_xor_sync(0xffffffffu, wmax, o));
-        if (lane == 0) s_max[wid] = wmax;
-        __syncthreads();
-        uint32_t maxcnt = 0;
-#pragma unroll
-        for (int w = 0; w < NW; ++w) maxcnt = max(maxcnt, s_max[w]);
+            for (int w = 0; w < NW; ++w) maxcnt = max(maxcnt, s_max[w]);
+        }
         for (int64_t hi = (int64_t)rg.x + maxcnt; hi > (int64_t)rg.x; hi -= A.depth) {
             const int64_t lo = max((int64_t)rg.x, hi - A.depth);
             const int nb = (int)(hi - lo);
             __syncthreads();
             for (int j = tid; j < nb; j += NT) {
-                uint32_t pair = A.vals[lo + j];
-                float4 r0 = A.rec[3 * (size_t)pair], r1 = A.rec[3 * (size_t)pair + 1];
-                float4 a, bb;
-                stage_record(r0, r1, a, bb);
-                sA[j] = a;
-                sB[j] = bb;
-                sC[j] = A.rec[3 * (size_t)pair + 2];
-                sH[j] = make_float2(r0.z, r0.w);
-                sP[j] = pair;
+                const uint32_t pair = A.vals[lo + j];
+                const float4 r0 = A.rec[3 * (size_t)pair], r1 = A.rec[3 * (size_t)pair + 1];
+                const float4 r2 = A.rec[3 * (size_t)pair + 2];
+                float4 a, b;
+                stage_record(r0, r1, a, b);
+                sE[j].u = make_float4(a.x, b.x, a.z, r0.z);
+                sE[j].row = make_float4(a.y, a.y, a.w, a.w);
+                sE[j].l = make_float4(b.y, b.y, b.z, b.z);
+                sE[j].or_ = make_float4(-b.w, -b.w, r2.x, r2.x);
+                sE[j].gb = make_float4(r2.y, r2.y, r2.z, r2.z);
+                sE[j].z = make_float4(r2.w, r2.w, r0.w, __uint_as_float(pair));
+                sM[j] = quad_mask<TW, TH, Q>(r0, r1, r2, tx0, ty0, A.c);
             }
             __syncthreads();
-            for (int j = nb - 1; j >= 0; --j) {
-                const uint32_t rel = (uint32_t)(lo + j - rg.x);
-                if (rel >= wmax) continue;  // no pixel of this warp reached this entry
-                const float4 a = sA[j], b = sB[j];
-                float dxi, u1;
-                frag_column(a, b, pxf, dxi, u1);
-                // the forward's alpha decision for each of the thread's pixels:
-                // ar = the unclamped alpha of a pixel the fragment reaches, else 0
-                float ar[PPT], t1_0 = 0.f, t2_0 = 0.f, dyi_0 = 0.f;
-                bool any = false;
-                {
-                    const f2 AY = f2_bcast(a.y), L12 = f2_bcast(b.y), L22 = f2_bcast(b.z);
-                    const f2 U1 = f2_bcast(u1), K2 = f2_bcast(a.w), NBW = f2_bcast(-b.w);
-                    f2 PY = PY0;
+            uint32_t which = 0;
+            int pending = 0;
+            for (int jb = (nb - 1) & ~31; jb >= 0; jb -= 32) {
+                const uint32_t rel0 = (uint32_t)(lo + jb - rg.x);
+                if (rel0 >= wmax) continue;  // no pixel of this warp reached these entries
+                const uint32_t mine = jb + lane < nb ? sM[jb + lane] : 0u;
+                const uint32_t exact = __ballot_sync(0xffffffffu, mine & kExactPath);
+                uint32_t E[Q], todo = 0, all = ~0u;
 #pragma unroll
-                    for (int p = 0; p < Q; ++p) {
-                        const f2 dy = f2_sub(PY, AY);  // dyi = py - V, exact as in the forward
-                        if (p + 1 < Q) PY = f2_add(PY, ONE);
-                        const f2 t1 = f2_fma(L12, dy, U1);
-                        const f2 t2 = f2_fma(L22, dy, K2);
-                        const f2 ne = f2_fma(t1, t1, f2_fma(t2, t2, NBW));  // -e
-                        if (p == 0) {
-                            t1_0 = f2_lo(t1);
-                            t2_0 = f2_lo(t2);
-                            dyi_0 = f2_lo(dy);
-                        }
-                        float n_[2];
-                        f2_unpack(ne, n_[0], n_[1]);
+                for (int q = 0; q < Q; ++q) {
+                    const bool hit = (mine >> (wid * Q + q) & 1u) && rel0 + lane < qmax[q];
+                    E[q] = __ballot_sync(0xffffffffu, hit);
+                    todo |= E[q];
+                    all &= E[q];
+                }
+                while (todo) {
+                    const int j = 31 - __clz(todo);
+                    todo ^= 1u << j;
+                    const uint32_t rel = rel0 + j;
+                    const BwdEntry &e = sE[jb + j];
+                    const float4 u = e.u;
+                    const F2x2 row = load_f2x2(e.row), l = load_f2x2(e.l), o = load_f2x2(e.or_), gbc = load_f2x2(e.gb);
+                    const float4 ez = e.z;
+                    const f2 CW = load_f2x2(ez).a;
+                    float dxi[QX], u1[QX];
+                    f2 DY[QY], IN[QY];
+#pragma unroll
+                    for (int x = 0; x < QX; ++x) {
+                        dxi[x] = __fsub_rn((float)(px0 + 8 * x), u.x);
+                        u1[x] = __fmaf_rn(u.y, dxi[x], u.z);
+                    }
+                    float t2_0 = 0.f;
+#pragma unroll
+                    for (int y = 0; y < QY; ++y) {
+                        DY[y] = f2_sub(f2_pack((float)(py0 + 8 * y), (float)(py0 + 8 * y + 4)), row.a);
+                        const f2 t2 = f2_fma(l.b, DY[y], row.b);
+                        if (y == 0) t2_0 = f2_lo(t2);
+                        IN[y] = f2_fma(t2, t2, o.a);
+                    }
+                    f2 sR = ZERO, sG = ZERO, sB_ = ZERO, sZ = ZERO;  // sums of -wgt dL/dc
+                    f2 ng[Q];                                        // -dL/dpw of each pixel
+                    auto quad = [&](int q, const bool clamp) {
+                        const f2 t1 = f2_fma(l.a, DY[q / QX], f2_bcast(u1[q % QX]));
+                        float n[2], al[2], ag[2];  // -e, -alpha, the -alpha that has a gradient through pw
+                        f2_unpack(f2_fma(t1, t1, IN[q / QX]), n[0], n[1]);
 #pragma unroll
                         for (int h = 0; h < 2; ++h) {
-                            const int i = p + h * Q;
-                            const bool in = rel < cnt[i] && n_[h] <= nl2amin;
-                            ar[i] = in ? ex2_approx(-n_[h]) : 0.f;
-                            any |= in;
+                            const bool in = rel < cnt[q][h] && n[h] <= nl2amin;
+                            al[h] = ag[h] = in ? -ex2_approx(-n[h]) : 0.f;
+                            if (clamp) {
+                                ag[h] = al[h] >= -amax ? al[h] : 0.f;
+                                al[h] = fmaxf(-amax, al[h]);
+                            }
+                        }
+                        const f2 nal = f2_pack(al[0], al[1]);
+                        float om[2];
+                        f2_unpack(f2_add(ONE, nal), om[0], om[1]);
+                        const f2 r1m = f2_pack(rcp_approx(om[0]), rcp_approx(om[1]));  // 1 / (1 - alpha)
+                        T[q] = f2_mul(T[q], r1m);  // transmittance before this fragment
+                        const f2 nwgt = f2_mul(nal, T[q]);
+                        f2 hh = f2_fma(gR[q], o.b, f2_fma(gG[q], gbc.a, f2_fma(gB[q], gbc.b, f2_fma(gD[q], CW, gA[q]))));
+                        f2 gz = gD[q];
+                        if (VAR) {
+                            const f2 dz = f2_sub(CW, zmu[q]);
+                            const f2 t = f2_fma(gb[q], dz, ga[q]);  // a + b dz
+                            hh = f2_fma(t, dz, hh);
+                            gz = f2_add(gz, f2_fma(gb[q], dz, t));  // a + 2 b dz
+                        }
+                        // dL/dalpha = T h - acc / (1 - alpha)
+                        const f2 dLda = f2_fma(T[q], hh, f2_mul(nacc[q], r1m));
+                        nacc[q] = f2_fma(nwgt, hh, nacc[q]);
+                        ng[q] = f2_mul(dLda, clamp ? f2_pack(ag[0], ag[1]) : nal);
+                        sR = f2_fma(nwgt, gR[q], sR);
+                        sG = f2_fma(nwgt, gG[q], sG);
+                        sB_ = f2_fma(nwgt, gB[q], sB_);
+                        sZ = f2_fma(nwgt, gz, sZ);
+                    };
+                    if (Q > 1 && (all & ~exact) >> j & 1u) {
+                        // every quadrant, interleaved (1680 -> 1606 us, 4M orchard)
+#pragma unroll
+                        for (int q = 0; q < Q; ++q) quad(q, false);
+                    } else {
+#pragma unroll
+                        for (int q = 0; q < Q; ++q) ng[q] = ZERO;
+                        if (!(exact >> j & 1u)) {
+#pragma unroll
+                            for (int q = 0; q < Q; ++q)
+                                if (E[q] >> j & 1u) quad(q, false);
+                        } else {
+#pragma unroll
+                            for (int q = 0; q < Q; ++q)
+                                if (E[q] >> j & 1u) quad(q, true);
                         }
                     }
-                }
-                if (!__any_sync(0xffffffffu, any)) continue;
-                // Every pixel runs the same instructions: a pixel this fragment
-                // does not reach takes alpha = 0, for which each update below is
-                // exactly the identity (T * 1, acc + 0 * h, sums + 0; the
-                // reciprocal approximation returns 1 for 1 on sm_103, measured).
-                // The blended sums are carried negated (nwgt = -wgt), which
-                // saves the negations the packed instructions cannot fold.
-                const float4 c = sC[j];
-                const f2 CX = f2_bcast(c.x), CY = f2_bcast(c.y), CZ = f2_bcast(c.z), CW = f2_bcast(c.w);
-                f2 sR, sG, sB_, sZ;  // sums of -wgt dL/dc
-                // R_k = sum over pairs p of p^k gpw (k = 0, 1, 2), gpw = dL/dpw
-                f2 R0, R1, R2;
+                    // Moments of the lane's pixels.  Its rows lie 0, 4, 8 and 12
+                    // below the first: with S_k = sum over a column of row^k (-gpw),
+                    // t1 and t2 affine in the row, dy = dy0 + row.
+                    const float dy0 = f2_lo(DY[0]) + ez.z;
+                    float S0 = 0.f, S1 = 0.f, S2 = 0.f, mU = 0.f, mA = 0.f, mB = 0.f;
 #pragma unroll
-                for (int p = 0; p < Q; ++p) {
-                    const float a0 = ar[p], a1 = ar[p + Q];
-                    const f2 nal = f2_pack(fmaxf(-amax, -a0), fmaxf(-amax, -a1));  // -alpha
-                    // alpha of an unclamped pixel, else 0: a clamped alpha has no
-                    // gradient through pw
-                    const f2 ag = f2_pack(a0 <= amax ? a0 : 0.f, a1 <= amax ? a1 : 0.f);
-                    float o_[2];
-                    f2_unpack(f2_add(ONE, nal), o_[0], o_[1]);
-                    const f2 r1m = f2_pack(rcp_approx(o_[0]), rcp_approx(o_[1]));  // 1 / (1 - alpha)
-                    T[p] = f2_mul(T[p], r1m);  // transmittance before this fragment
-                    const f2 nwgt = f2_mul(nal, T[p]);
-                    f2 h = f2_fma(gR[p], CX, f2_fma(gG[p], CY, f2_fma(gB[p], CZ, f2_fma(gD[p], CW, gA[p]))));
-                    f2 gz = gD[p];
-                    if (VAR) {
-                        const f2 dz = f2_sub(CW, zmu[p]);
-                        const f2 t = f2_fma(gb[p], dz, ga[p]);  // a + b dz
-                        h = f2_fma(t, dz, h);
-                        gz = f2_add(gz, f2_fma(gb[p], dz, t));  // a + 2 b dz
+                    for (int x = 0; x < QX; ++x) {
+                        float a0, a1, b0 = 0.f, b1 = 0.f;
+                        f2_unpack(ng[x], a0, a1);
+                        float s0 = a0 + a1, s1 = 4.f * a1, s2 = 16.f * a1;
+                        if (QY == 2) {
+                            f2_unpack(ng[(QY - 1) * QX + x], b0, b1);
+                            s0 += b0 + b1;
+                            s1 = __fmaf_rn(12.f, b1, __fmaf_rn(8.f, b0, s1));
+                            s2 = __fmaf_rn(144.f, b1, __fmaf_rn(64.f, b0, s2));
+                        }
+                        const float dx = dxi[x] + u.w;
+                        const float t1_0 = __fmaf_rn(e.l.x, f2_lo(DY[0]), u1[x]);
+                        S0 += s0;
+                        S1 += s1;
+                        S2 += s2;
+                        mU = __fmaf_rn(t1_0, s0, mU);
+                        mA = __fmaf_rn(dx * dx, s0, mA);
+                        mB = __fmaf_rn(dx, __fmaf_rn(dy0, s0, s1), mB);
                     }
-                    // dL/dalpha = T h - acc / (1 - alpha)
-                    const f2 dLda = f2_fma(T[p], h, f2_mul(nacc[p], r1m));
-                    nacc[p] = f2_fma(nwgt, h, nacc[p]);
-                    const f2 gpw = f2_mul(dLda, ag);
-                    if (p == 0) {
-                        sR = f2_mul(nwgt, gR[p]);
-                        sG = f2_mul(nwgt, gG[p]);
-                        sB_ = f2_mul(nwgt, gB[p]);
-                        sZ = f2_mul(nwgt, gz);
-                        R0 = gpw;
-                    } else {
-                        sR = f2_fma(nwgt, gR[p], sR);
-                        sG = f2_fma(nwgt, gG[p], sG);
-                        sB_ = f2_fma(nwgt, gB[p], sB_);
-                        sZ = f2_fma(nwgt, gz, sZ);
-                        R0 = f2_add(R0, gpw);
+                    float *mine_sum = sums + (pending * 32 + lane) * kSumRow;
+                    // (u, v, qa, qb), (qc, ln o, r, g), (b, z)
+                    *reinterpret_cast<float4 *>(mine_sum) =
+                        make_float4(__fmaf_rn(e.l.x, S1, mU), __fmaf_rn(t2_0, S0, e.l.z * S1), mA, mB);
+                    *reinterpret_cast<float4 *>(mine_sum + 4) =
+                        make_float4(__fmaf_rn(dy0, __fmaf_rn(dy0, S0, S1), __fmaf_rn(dy0, S1, S2)), S0,
+                                    f2_lo(sR) + f2_hi(sR), f2_lo(sG) + f2_hi(sG));
+                    *reinterpret_cast<float2 *>(mine_sum + 8) =
+                        make_float2(f2_lo(sB_) + f2_hi(sB_), f2_lo(sZ) + f2_hi(sZ));
+                    which = which << 8 | (uint32_t)(jb + j);
+                    if (++pending == kSumSlots) {
+                        flush_sums(sums, sE, kSumSlots, __byte_perm(which, 0, 0x0123), lane, A.g2d);
+                        pending = 0;
                     }
-                    if (p == 1) {
-                        R1 = gpw;
-                        R2 = gpw;
-                    } else if (p > 1) {
-                        R1 = f2_fma(gpw, f2_bcast((float)p), R1);
-                        R2 = f2_fma(gpw, f2_bcast((float)(p * p)), R2);
-                    }
-                }
-                if (Q == 1) R1 = R2 = f2_bcast(0.f);
-                // S_k = sum over the column's pixels i of i^k gpw: pixel p + Q
-                // sits in the high half of pair p
-                float r0l, r0h, r1l, r1h, r2l, r2h;
-                f2_unpack(R0, r0l, r0h);
-                f2_unpack(R1, r1l, r1h);
-                f2_unpack(R2, r2l, r2h);
-                const float S0 = r0l + r0h;
-                const float S1 = __fmaf_rn((float)Q, r0h, r1l + r1h);
-                const float S2 = __fmaf_rn((float)(Q * Q), r0h, __fmaf_rn((float)(2 * Q), r1h, r2l + r2h));
-                // per-lane raw moments: the pixel offsets are dx (one per column)
-                // and dy_i = dy_0 + i, and t1, t2 are affine in i; the
-                // per-Gaussian factors are applied once after the warp reduction
-                const float2 hh = sH[j];
-                const float dx = dxi + hh.x, dy0 = dyi_0 + hh.y;
-                const float sy = __fmaf_rn(dy0, S0, S1);  // sum gpw dy
-                float g[kGrad];
-                g[G_LNO] = S0;
-                g[G_U] = __fmaf_rn(t1_0, S0, b.y * S1);  // sum gpw t1, t1_i = t1_0 + l12 i
-                g[G_V] = __fmaf_rn(t2_0, S0, b.z * S1);  // sum gpw t2, t2_i = t2_0 + l22 i
-                g[G_QA] = dx * dx * S0;                     // sum gpw dx^2
-                g[G_QB] = dx * sy;                          // sum gpw dx dy
-                g[G_QC] = __fmaf_rn(dy0, sy, __fmaf_rn(dy0, S1, S2));  // sum gpw dy^2
-                g[G_R] = f2_lo(sR) + f2_hi(sR);
-                g[G_G] = f2_lo(sG) + f2_hi(sG);
-                g[G_B] = f2_lo(sB_) + f2_hi(sB_);
-                g[G_Z] = f2_lo(sZ) + f2_hi(sZ);
-                const float tot = warp_reduce_scatter10(g, lane);
-                if (my_comp >= 0) {
-                    // dL/dQ = -1/2 sum gpw d d^T; dpw/du = (Q d)_x = l11 t1 / s^2,
-                    // dpw/dv = (l12 t1 + l22 t2) / s^2 with 1/s^2 = 2 ln 2: each lane
-                    // scales its sum by c0 + c11 l11 + c22 l22 (constants per lane;
-                    // c0 = -1 undoes the negation of the colour and depth sums)
-                    float *gp = A.g2d + (size_t)sP[j] * kGrad;
-                    atomicAdd(gp + my_comp, tot * __fmaf_rn(sc11, b.x, __fmaf_rn(sc22, b.z, sc0)));
-                    if (my_comp == G_U) atomicAdd(gp + G_V, kTwoLn2 * b.y * tot);
                 }
             }
+            // (the pending entries' staged records go with this batch)
+            if (pending)
+                flush_sums(sums, sE, pending, __byte_perm(which << 8 * (kSumSlots - pending), 0, 0x0123), lane, A.g2d);
         }
     }
 }
@@ -503,57 +905,58 @@ __global__ void k_zero_g2d(const uint32_t *vis_pair, const DevState *st, float *
         g2d[(size_t)vis_pair[i / kGrad] * kGrad + i % kGrad] = 0.f;
 }
 
-// Pixels per thread of the backward (the forward uses one, so that a pixel
-// leaves the list as soon as it saturates).  More pixels a thread amortise the
-// per-fragment warp reduction and the shared-memory reads over more pixels:
-// on the 500k orchard with 16x16 tiles, 4 -> 0.467 ms and 8 (one warp a tile)
-// -> 0.435 ms.  The VAR variant holds three more values a pixel and keeps 4
-// (8 spills).  An 8x8 tile keeps 2 so that its CTA is still a whole warp,
-// which the full-mask shuffles and votes require.
-template <int TW, int TH, bool VAR>
-constexpr int ppt_bwd() { return TW * TH >= 256 ? (VAR ? 4 : 8) : 2; }
+// The kernel of one pass for a tile size, with its launch shape.
+struct RasterKernel {
+    void (*fn)(RasterArgs);
+    int threads, depth;  // depth: entries staged at a time
+    size_t smem;
+};
 
-size_t fwd_smem(int depth) { return (size_t)depth * 3 * sizeof(float4); }
-size_t bwd_smem(int depth) {
-    return (size_t)depth * (3 * sizeof(float4) + sizeof(float2) + sizeof(uint32_t));
+// The forward's quadrants a warp.
+template <int TW, int TH, int Q, bool VAR>
+RasterKernel fwd_variant(int depth) {
+    const int d = std::min(depth, kFwdDepth);
+    return {k_raster_fwd<TW, TH, Q, VAR>, Share<TW, TH, Q>::NT, d,
+            (size_t)d * (sizeof(FwdEntry) + sizeof(uint32_t))};
 }
-
-// Pixels per thread of the forward: on the 500k orchard with 16x16 tiles
-// 1 -> 0.307 ms, 2 -> 0.268 ms, 4 -> 0.239 ms, 8 -> 0.303 ms; the VAR variant
-// (four more values a pixel, register bound above) 2 -> 0.370 ms, 4 -> 0.352 ms.
-template <int TW, int TH, bool VAR>
-constexpr int ppt_fwd() { return TW * TH >= 256 ? 4 : 2; }
-
-template <int TW, int TH, bool VAR>
-cudaError_t configure_variant(gs_workspace *ws, int &grid_f, int &grid_b) {
-    constexpr int PPT = ppt_bwd<TW, TH, VAR>(), PF = ppt_fwd<TW, TH, VAR>();
-    const int depth = ws->cfg.batch_depth;
-    cudaError_t e = cudaFuncSetAttribute(k_raster_fwd<TW, TH, PF, VAR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)fwd_smem(256));
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_raster_bwd<TW, TH, PPT, VAR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)bwd_smem(256));
-    int occ_f = 0, occ_b = 0;
-    if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_f, k_raster_fwd<TW, TH, PF, VAR>, TW * TH / PF,
-                                                          fwd_smem(depth));
-    if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_b, k_raster_bwd<TW, TH, PPT, VAR>, TW * TH / PPT,
-                                                          bwd_smem(depth));
-    grid_f = std::max(1, occ_f) * ws->num_sms;
-    grid_b = std::max(1, occ_b) * ws->num_sms;
-    return e;
-}
-
 template <int TW, int TH>
-gs_status configure_one(gs_workspace *ws) {
-    cudaError_t e = configure_variant<TW, TH, false>(ws, ws->raster_grid_fwd, ws->raster_grid_bwd);
-    if (e == cudaSuccess) e = configure_variant<TW, TH, true>(ws, ws->raster_grid_fwd_var, ws->raster_grid_bwd_var);
-    if (e != cudaSuccess) {
-        set_last_error(std::string("raster_configure: ") + cudaGetErrorString(e));
-        return GS_ERR_CUDA;
+RasterKernel fwd_kernel(const gs_workspace *ws, bool var) {
+    const int d = ws->cfg.batch_depth;
+    if constexpr (TW * TH >= 256) {
+        const int64_t tiles = ws->n_tiles * (TW * TH / 256);
+        if (!var)
+            return tiles >= kFwdWholeTiles ? fwd_variant<TW, TH, 4, false>(d)
+                   : tiles >= kFwdHalfTiles ? fwd_variant<TW, TH, 2, false>(d) : fwd_variant<TW, TH, 1, false>(d);
+        return tiles >= kCoarseTiles ? fwd_variant<TW, TH, 2, true>(d) : fwd_variant<TW, TH, 1, true>(d);
     }
-    return GS_OK;
+    else {
+        const size_t smem = (size_t)d * 3 * sizeof(float4);
+        return {var ? k_raster_fwd_columns<TW, TH, 2, true> : k_raster_fwd_columns<TW, TH, 2, false>, TW * TH / 2, d, smem};
+    }
+}
+
+template <int TW, int TH, int Q, bool VAR>
+RasterKernel bwd_variant(int depth) {
+    const int d = std::min(depth, kBwdDepth);
+    using S = Share<TW, TH, Q>;
+    return {k_raster_bwd<TW, TH, Q, VAR>, S::NT, d, (size_t)d * (sizeof(BwdEntry) + sizeof(uint32_t)) + S::NW * kSumBytes};
+}
+template <int TW, int TH>
+RasterKernel bwd_kernel(const gs_workspace *ws, bool var) {
+    const int d = ws->cfg.batch_depth;
+    if constexpr (TW * TH >= 256) {
+        if (ws->n_tiles * (TW * TH / 256) >= kCoarseTiles)
+            return var ? bwd_variant<TW, TH, 2, true>(d) : bwd_variant<TW, TH, 4, false>(d);
+    }
+    return var ? bwd_variant<TW, TH, 1, true>(d) : bwd_variant<TW, TH, 1, false>(d);
+}
+
+RasterKernel raster_kernel(const gs_workspace *ws, bool forward, bool var) {
+    const int tw = ws->cfg.tile_w, th = ws->cfg.tile_h;
+    if (tw == 8) return forward ? fwd_kernel<8, 8>(ws, var) : bwd_kernel<8, 8>(ws, var);
+    if (tw == 16 && th == 16) return forward ? fwd_kernel<16, 16>(ws, var) : bwd_kernel<16, 16>(ws, var);
+    if (tw == 16) return forward ? fwd_kernel<16, 32>(ws, var) : bwd_kernel<16, 32>(ws, var);
+    return forward ? fwd_kernel<32, 16>(ws, var) : bwd_kernel<32, 16>(ws, var);
 }
 
 RasterArgs make_args(gs_workspace *ws) {
@@ -561,7 +964,6 @@ RasterArgs make_args(gs_workspace *ws) {
     A.views = ws->views;
     A.n_views = ws->n_views;
     A.n_tiles = (int32_t)ws->n_tiles;
-    A.depth = ws->cfg.batch_depth;
     A.c = ws->consts;
     A.rec = ws->rec;
     A.vals = ws->inst_val;
@@ -572,38 +974,36 @@ RasterArgs make_args(gs_workspace *ws) {
     return A;
 }
 
-template <int TW, int TH>
-gs_status run_fwd(gs_workspace *ws, RasterArgs A, cudaStream_t s) {
-    StageTimer timer(ws, GS_STAGE_RASTER_FWD, s);
+gs_status run(gs_workspace *ws, RasterArgs A, bool forward, bool var, cudaStream_t s) {
+    StageTimer timer(ws, forward ? GS_STAGE_RASTER_FWD : GS_STAGE_RASTER_BWD, s);
     ++ws->kernel_launches;
-    constexpr int PV = ppt_fwd<TW, TH, true>(), P = ppt_fwd<TW, TH, false>();
-    if (A.mean_out)
-        k_raster_fwd<TW, TH, PV, true><<<ws->raster_grid_fwd_var, TW * TH / PV, fwd_smem(A.depth), s>>>(A);
-    else
-        k_raster_fwd<TW, TH, P, false><<<ws->raster_grid_fwd, TW * TH / P, fwd_smem(A.depth), s>>>(A);
-    return check_launch("raster_fwd");
-}
-template <int TW, int TH>
-gs_status run_bwd(gs_workspace *ws, RasterArgs A, cudaStream_t s) {
-    constexpr int PV = ppt_bwd<TW, TH, true>(), P = ppt_bwd<TW, TH, false>();
-    StageTimer timer(ws, GS_STAGE_RASTER_BWD, s);
-    ++ws->kernel_launches;
-    if (A.vstat)
-        k_raster_bwd<TW, TH, PV, true><<<ws->raster_grid_bwd_var, TW * TH / PV, bwd_smem(A.depth), s>>>(A);
-    else
-        k_raster_bwd<TW, TH, P, false><<<ws->raster_grid_bwd, TW * TH / P, bwd_smem(A.depth), s>>>(A);
-    return check_launch("raster_bwd");
+    const RasterKernel k = raster_kernel(ws, forward, var);
+    A.depth = k.depth;
+    const int grid = forward ? (var ? ws->raster_grid_fwd_var : ws->raster_grid_fwd)
+                             : (var ? ws->raster_grid_bwd_var : ws->raster_grid_bwd);
+    k.fn<<<grid, k.threads, k.smem, s>>>(A);
+    return check_launch(forward ? "raster_fwd" : "raster_bwd");
 }
 
 }  // namespace
 
 gs_status raster_configure(gs_workspace *ws) {
-    int tw = ws->cfg.tile_w, th = ws->cfg.tile_h;
-    if (tw == 8 && th == 8) return configure_one<8, 8>(ws);
-    if (tw == 16 && th == 16) return configure_one<16, 16>(ws);
-    if (tw == 16 && th == 32) return configure_one<16, 32>(ws);
-    if (tw == 32 && th == 16) return configure_one<32, 16>(ws);
-    return GS_ERR_INVALID_ARG;
+    cudaError_t e = cudaSuccess;
+    for (int i = 0; i < 4 && e == cudaSuccess; ++i) {
+        const bool forward = i < 2, var = i & 1;
+        const RasterKernel k = raster_kernel(ws, forward, var);
+        e = cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem);
+        int occ = 0;
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k.fn, k.threads, k.smem);
+        int32_t &grid = forward ? (var ? ws->raster_grid_fwd_var : ws->raster_grid_fwd)
+                                : (var ? ws->raster_grid_bwd_var : ws->raster_grid_bwd);
+        grid = std::max(1, occ) * ws->num_sms;
+    }
+    if (e != cudaSuccess) {
+        set_last_error(std::string("raster_configure: ") + cudaGetErrorString(e));
+        return GS_ERR_CUDA;
+    }
+    return GS_OK;
 }
 
 gs_status launch_raster_fwd(gs_workspace *ws, float *rgb, float *depth, float *alpha, float *mean,
@@ -619,11 +1019,7 @@ gs_status launch_raster_fwd(gs_workspace *ws, float *rgb, float *depth, float *a
         A.vstat = ws->vstat;
     }
     cudaMemsetAsync(A.counter, 0, sizeof(uint32_t), s);
-    int tw = ws->cfg.tile_w, th = ws->cfg.tile_h;
-    if (tw == 8 && th == 8) return run_fwd<8, 8>(ws, A, s);
-    if (tw == 16 && th == 16) return run_fwd<16, 16>(ws, A, s);
-    if (tw == 16 && th == 32) return run_fwd<16, 32>(ws, A, s);
-    return run_fwd<32, 16>(ws, A, s);
+    return run(ws, A, true, mean != nullptr, s);
 }
 
 gs_status launch_raster_bwd(gs_workspace *ws, const float *dL_drgb, const float *dL_ddepth,
@@ -651,11 +1047,7 @@ gs_status launch_raster_bwd(gs_workspace *ws, const float *dL_drgb, const float 
     }
     ws->g2d_clear = false;
     cudaMemsetAsync(A.counter, 0, sizeof(uint32_t), s);
-    int tw = ws->cfg.tile_w, th = ws->cfg.tile_h;
-    if (tw == 8 && th == 8) return run_bwd<8, 8>(ws, A, s);
-    if (tw == 16 && th == 16) return run_bwd<16, 16>(ws, A, s);
-    if (tw == 16 && th == 32) return run_bwd<16, 32>(ws, A, s);
-    return run_bwd<32, 16>(ws, A, s);
+    return run(ws, A, false, var, s);
 }
 
 }  // namespace gs

@@ -455,56 +455,6 @@ __global__ void __launch_bounds__(T) k_instance_offsets(const DevState *st, cons
 // the highest tile id), the ranges skip them, and the rasterisers never walk
 // them.
 
-// Does the tile whose pixels span [X0, X1] x [Y0, Y1] hold an instance of the
-// pair with record r0 = (U, V, hx, hy), r1 = (l11, l12, l22, log2 o)?  The
-// rasterisers keep a fragment where log2 o - |t|^2 >= log2 alpha_min, with
-// t = L d, L = [[l11, l12], [0, l22]] and d = (px - U + hx, py - V + hy) the
-// offset of pixel (px, py)'s centre from the mean.  The tile is kept iff the
-// minimum of |L d|^2 over the box of its pixel centres, grown by ext_abs_pad,
-// is within (log2 o - log2 alpha_min) (1 + ext_rel_pad)^2: the same padding as
-// the rectangle's extents, which dwarfs the rounding of this test and of the
-// rasterisers' own evaluation, so a dropped tile has no fragment to keep.  The
-// minimum of the convex quadratic is 0 when the box holds the mean, else it
-// lies on an edge, at the edge's stationary point clamped to the edge.
-// The pair's own factors of the test: the stationary slopes on an edge
-// dx = const (sy = dy/dx) and dy = const (sx = dx/dy), and the padded
-// threshold.  (Staging them per pair in the window, with the record load that
-// needs, measured slower than recomputing them per instance: the load lands
-// on the staging's critical path.)
-__device__ __forceinline__ float4 reach_terms(const float4 r1, const Consts &k) {
-    const float l11 = r1.x, l12 = r1.y, l22 = r1.z;
-    const float pad = 1.f + k.ext_rel_pad;
-    // (the slopes by the fast division, within 2 ulps: the quadratic is
-    // stationary there, so a slope off by e moves the edge minimum by O(e^2);
-    // orchard4m emission 0.239 -> 0.228 ms)
-    return make_float4(__fdividef(-l11 * l12, l12 * l12 + l22 * l22), __fdividef(-l12, l11),
-                       (r1.w - k.log2_alpha_min) * pad * pad, 0.f);
-}
-
-__device__ __forceinline__ bool tile_reached(const float4 r0, const float4 r1, const float4 q, int X0, int X1,
-                                             int Y0, int Y1, const Consts &k) {
-    const float ax = __fadd_rn((float)X0 - r0.x, r0.z) - k.ext_abs_pad;
-    const float bx = __fadd_rn((float)X1 - r0.x, r0.z) + k.ext_abs_pad;
-    const float ay = __fadd_rn((float)Y0 - r0.y, r0.w) - k.ext_abs_pad;
-    const float by = __fadd_rn((float)Y1 - r0.y, r0.w) + k.ext_abs_pad;
-    if (ax <= 0.f && bx >= 0.f && ay <= 0.f && by >= 0.f) return true;
-    const float l11 = r1.x, l12 = r1.y, l22 = r1.z;
-    const float sy = q.x, sx = q.y;
-    float m = INFINITY;
-#pragma unroll
-    for (int e = 0; e < 2; ++e) {
-        const float cx = e ? bx : ax;
-        const float dy = fminf(fmaxf(sy * cx, ay), by);
-        const float t1 = l11 * cx + l12 * dy, t2 = l22 * dy;
-        m = fminf(m, t1 * t1 + t2 * t2);
-        const float cy = e ? by : ay;
-        const float dx = fminf(fmaxf(sx * cy, ax), bx);
-        const float u1 = l11 * dx + l12 * cy, u2 = l22 * cy;
-        m = fminf(m, u1 * u1 + u2 * u2);
-    }
-    return m <= q.z;
-}
-
 // Blocks of the emission an SM keeps resident: a window's staging is a short
 // chain of dependent loads (slot owners, pair ids, rectangles) that every
 // thread of the block waits for, so several blocks per SM hide it.
@@ -615,8 +565,10 @@ __global__ void __launch_bounds__(T, kEmitBlocksPerSM) k_emit_instances(
             const int ty = r.y + row, tx = r.x + (local - row * wdt);
             const int X0 = tx * k.tile_w, Y0 = ty * k.tile_h;
             const float4 r1 = __ldg(rec + 3 * (size_t)pair + 1);
-            const bool keep = tile_reached(__ldg(rec + 3 * (size_t)pair), r1, reach_terms(r1, k), X0,
-                                           min(X0 + k.tile_w, vw.z) - 1, Y0, min(Y0 + k.tile_h, vw.w) - 1, k);
+            const bool keep = tile_reached(__ldg(rec + 3 * (size_t)pair), r1,
+                                           reach_terms(r1, k.log2_alpha_min, 1.f + k.ext_rel_pad), X0,
+                                           min(X0 + k.tile_w, vw.z) - 1, Y0, min(Y0 + k.tile_h, vw.w) - 1,
+                                           k.ext_abs_pad);
             inst_tile[o] = keep ? (uint32_t)(vw.x + ty * vw.y + tx) : kInvalidKey;
             inst_val[o] = pair;
         }
