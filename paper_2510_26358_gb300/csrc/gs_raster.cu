@@ -59,14 +59,15 @@ constexpr int kFwdDepth = 64, kBwdDepth = 64;
 // pixels).  Whole tiles share the most work between quadrants but make the
 // fewest warps: with few tiles the time is the longest list's chain of
 // entries, which is shorter the less a warp does for each.  Measured (one,
-// two, four quadrants a warp, us), orchard of 200k: forward, 88 tiles (box of 3k)
-// 28, 41, -; 300 tiles 63, 58, 101; 3600 41, 38, 55; 7200 87, 64, 75; 1M, 24,480 tiles -, 391, 406; 4M,
-// 54,000 tiles -, 971, 936.  Backward, 300 tiles 93, 111, 186; 2400 95, 102,
-// 143; 3600 59, 59, 86; 7200 171, 130, 124.  With the variance (one, two; more
-// do not fit the registers) forward, 2400 tiles 73, 97; 7200 139, 107; backward
-// 104, 108; 186, 153.
+// two, four quadrants a warp, us).  Forward, the whole step: 300 tiles (320x240,
+// box of 10k) 288, 298, -; 1200 (orchard of 200k, as below) 247, 258, -; 2400
+// 318, 319, -; 3600 249, 247, -; the kernel: 7200 87, 64, 75; 24,480 (1M) -, 391,
+// 406; 54,000 (4M) -, 971, 936.  Backward, the kernel: 300 tiles 93, 111, 186;
+// 2400 95, 102, 143; 3600 59, 59, 86; 7200 171, 130, 124.  With the variance (one,
+// two; more do not fit the registers) forward, 2400 tiles 73, 97; 7200 139, 107;
+// backward 104, 108; 186, 153.
 constexpr int kCoarseTiles = 152 * 24;     // backward, and forward with the variance
-constexpr int kFwdHalfTiles = 152, kFwdWholeTiles = 152 * 256;  // forward
+constexpr int kFwdHalfTiles = 152 * 16, kFwdWholeTiles = 152 * 256;  // forward
 
 // Resident warps an SM that each variant's registers are bounded for, as CTAs
 // (forward, 4M orchard: 20 warps of whole tiles 0.94 ms, 24 0.99 ms with spills,
