@@ -14,10 +14,10 @@
 //
 // Three kernels: classify (action and output count per splat, block sums),
 // scan (block offsets, total, capacity check, new submap offsets), scatter
-// (block-local scan, then the rows; SH rows copied warp-cooperatively so the
-// writes coalesce).  A total above the output capacity writes nothing and
+// (block-local scan, then the rows array by array, see gs_rows.cuh).  A total above the output capacity writes nothing and
 // sets the flag gs_lifecycle_status reports.
 #include "gs_internal.cuh"
+#include "gs_rows.cuh"
 #include "gs_scan.cuh"
 
 #include <cmath>
@@ -36,7 +36,7 @@ namespace gs {
 namespace {
 
 constexpr int LT = 256;            // threads per block
-constexpr int LCHUNK = 8 * LT;     // splats per block
+constexpr int LCHUNK = kRowChunk;  // splats per block
 enum : uint8_t { A_PRUNE = 0, A_KEEP = 1, A_CLONE = 2, A_SPLIT = 3 };
 __host__ __device__ constexpr uint32_t out_count(uint8_t a) { return a == A_PRUNE ? 0u : (a == A_KEEP ? 1u : 2u); }
 
@@ -88,25 +88,32 @@ __global__ void __launch_bounds__(LT) k_lc_classify(Thresholds t, Arrays in, con
     if (threadIdx.x == 0) block_sum[blockIdx.x] = tot;
 }
 
-// One block: exclusive scan of the block sums, the total and the capacity
-// check, then the new submap offsets (output position of each submap's first
-// splat: the offset of its chunk plus the counts before it in the chunk).
-__global__ void __launch_bounds__(LT) k_lc_scan(const uint32_t *block_sum, int nblocks, const uint8_t *action,
-                                                int64_t n, const int64_t *offs_in, int n_submaps, int64_t capacity,
-                                                uint32_t *block_off, int64_t *offs_out, int64_t *state, int64_t *n_out) {
-    __shared__ uint32_t sm[LT / 32];
-    __shared__ uint32_t carry;
-    if (threadIdx.x == 0) carry = 0;
-    __syncthreads();
-    for (int b0 = 0; b0 < nblocks; b0 += LT) {
-        const int b = b0 + threadIdx.x;
-        const uint32_t v = b < nblocks ? block_sum[b] : 0u;
-        uint32_t tot;
-        const uint32_t ex = block_scan_u32(v, sm, tot);
-        if (b < nblocks) block_off[b] = carry + ex;
-        __syncthreads();
-        if (threadIdx.x == 0) carry += tot;
-        __syncthreads();
+// One block: exclusive scan of the block sums (four a thread at a time), the
+// total and the capacity check, then the new submap offsets, a warp a submap
+// (output position of each submap's first splat: the offset of its chunk plus
+// the counts before it in the chunk).
+constexpr int kScanThreads = 1024;
+__global__ void __launch_bounds__(kScanThreads) k_lc_scan(const uint32_t *block_sum, int nblocks, const uint8_t *action,
+                                                          int64_t n, const int64_t *offs_in, int n_submaps,
+                                                          int64_t capacity, uint32_t *block_off, int64_t *offs_out,
+                                                          int64_t *state, int64_t *n_out) {
+    __shared__ uint32_t sm[kScanThreads / 32];
+    uint32_t carry = 0;
+    for (int b0 = 0; b0 < nblocks; b0 += 4 * kScanThreads) {
+        const int b = b0 + 4 * threadIdx.x;
+        uint32_t v[4], sum = 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            v[k] = b + k < nblocks ? block_sum[b + k] : 0u;
+            sum += v[k];
+        }
+        uint32_t tot, ex = carry + gs::block_scan_u32<kScanThreads>(sum, sm, tot);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            if (b + k < nblocks) block_off[b + k] = ex;
+            ex += v[k];
+        }
+        carry += tot;
     }
     const int64_t total = carry;
     const bool fits = total <= capacity;
@@ -116,20 +123,18 @@ __global__ void __launch_bounds__(LT) k_lc_scan(const uint32_t *block_sum, int n
         if (n_out) *n_out = total;
     }
     if (!fits || !offs_out) return;
-    for (int s = 0; s <= n_submaps; ++s) {
+    __syncthreads();  // the offsets written above
+    for (int s = threadIdx.x >> 5; s <= n_submaps; s += kScanThreads / 32) {
+        const int lane = threadIdx.x & 31;
         const int64_t j = offs_in[s];
-        uint32_t c = 0;
-        int64_t pos;
-        if (j >= n) {
-            pos = total;
-        } else {
+        int64_t pos = total;
+        if (j < n) {
             const int64_t cb = j / LCHUNK;
-            for (int64_t i = cb * LCHUNK + threadIdx.x; i < j; i += LT) c += out_count(action[i] & 0x7f);
-            const uint32_t t = block_sum_u32(c, sm);
-            pos = (int64_t)block_off[cb] + t;
+            uint32_t c = 0;
+            for (int64_t i = cb * LCHUNK + lane; i < j; i += 32) c += out_count(action[i] & 0x7f);
+            pos = (int64_t)block_off[cb] + __reduce_add_sync(0xffffffffu, c);
         }
-        if (threadIdx.x == 0) offs_out[s] = pos;
-        __syncthreads();
+        if (lane == 0) offs_out[s] = pos;
     }
 }
 
@@ -150,95 +155,70 @@ struct ScatterArgs {
     const uint32_t *block_off;
     const int64_t *state;
     int64_t n;
-    int32_t nsh;  // SH floats per splat
     bool moments;
 };
 
-// Optimiser moments of one output row (small fields): the source's, or zero
-// for a new splat.
-__device__ __forceinline__ void copy_moment_row(const Arrays src, const OutArrays dst, int64_t j, int64_t o,
-                                                bool fresh) {
-#pragma unroll
-    for (int r = 0; r < 3; ++r) {
-        dst.means[3 * o + r] = fresh ? 0.f : src.means[3 * j + r];
-        dst.log_scales[3 * o + r] = fresh ? 0.f : src.log_scales[3 * j + r];
-    }
-#pragma unroll
-    for (int r = 0; r < 4; ++r) dst.quats[4 * o + r] = fresh ? 0.f : src.quats[4 * j + r];
-    dst.omega[o] = fresh ? 0.f : src.omega[j];
+// The moments of a block's output rows: the source's, or zero for a new splat.
+template <int NSH>
+__device__ __forceinline__ void copy_moments(const Arrays &in, const OutArrays &out, int64_t j0, int64_t o0,
+                                             const uint16_t *rows, int n) {
+    copy_rows<LT, NSH, ROWS_ZERO_FRESH>(in.sh + j0 * NSH, out.sh + o0 * NSH, rows, n);
+    copy_rows<LT, 3, ROWS_ZERO_FRESH>(in.means + 3 * j0, out.means + 3 * o0, rows, n);
+    copy_rows<LT, 3, ROWS_ZERO_FRESH>(in.log_scales + 3 * j0, out.log_scales + 3 * o0, rows, n);
+    copy_rows<LT, 4, ROWS_ZERO_FRESH>(in.quats + 4 * j0, out.quats + 4 * o0, rows, n);
+    copy_rows<LT, 1, ROWS_ZERO_FRESH>(in.omega + j0, out.omega + o0, rows, n);
 }
 
-// Writes one output row of the small fields (the SH rows are copied apart).
-__device__ __forceinline__ void write_row(const ScatterArgs &A, int64_t j, int64_t o, uint8_t a, int k,
-                                          bool reset) {
-    float mean[3] = {A.in.means[3 * j], A.in.means[3 * j + 1], A.in.means[3 * j + 2]};
-    float ls[3] = {A.in.log_scales[3 * j], A.in.log_scales[3 * j + 1], A.in.log_scales[3 * j + 2]};
-    const float *q = A.in.quats + 4 * j;
-    if (a == A_SPLIT) {
-        float R[9];
-        quat_rot(q, R);
-        const float *z = A.normals + 6 * j + 3 * k;
-        const float v0 = expf(ls[0]) * z[0], v1 = expf(ls[1]) * z[1], v2 = expf(ls[2]) * z[2];
-#pragma unroll
-        for (int r = 0; r < 3; ++r) mean[r] += R[3 * r] * v0 + R[3 * r + 1] * v1 + R[3 * r + 2] * v2;
-#pragma unroll
-        for (int r = 0; r < 3; ++r) ls[r] -= A.t.shrink;
-    }
-#pragma unroll
-    for (int r = 0; r < 3; ++r) {
-        A.out.means[3 * o + r] = mean[r];
-        A.out.log_scales[3 * o + r] = ls[r];
-    }
-#pragma unroll
-    for (int r = 0; r < 4; ++r) A.out.quats[4 * o + r] = q[r];
-    A.out.omega[o] = reset ? A.t.reset : A.in.omega[j];
-    if (A.moments) {
-        const bool fresh = a == A_SPLIT || (a == A_CLONE && k == 1);
-        copy_moment_row(A.in_m, A.out_m, j, o, fresh);
-        copy_moment_row(A.in_v, A.out_v, j, o, fresh);
-    }
-}
-
+template <int NSH>
 __global__ void __launch_bounds__(LT) k_lc_scatter(ScatterArgs A) {
     __shared__ uint32_t sm[LT / 32];
-    __shared__ uint32_t s_carry;
+    __shared__ uint16_t rows[2 * LCHUNK];
+    static_assert(LCHUNK == 2 * LT, "two splats a thread");
     if (A.state[1]) return;  // over capacity: nothing is written
-    const int64_t base = (int64_t)blockIdx.x * LCHUNK;
-    const int lane = threadIdx.x & 31;
-    if (threadIdx.x == 0) s_carry = A.block_off[blockIdx.x];
+    const int64_t j0 = (int64_t)blockIdx.x * LCHUNK, o0 = A.block_off[blockIdx.x];
+    uint8_t code[2];
+    uint32_t c = 0;
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const int64_t j = j0 + 2 * threadIdx.x + i;
+        code[i] = j < A.n ? A.action[j] : (uint8_t)A_PRUNE;
+        c += out_count(code[i] & 0x7f);
+    }
+    uint32_t tot;
+    uint32_t o = block_scan_u32(c, sm, tot);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const uint8_t a = code[i] & 0x7f;
+        const uint32_t r = (2 * threadIdx.x + i) | (a == A_SPLIT ? kRowSplit | kRowFresh : 0u) |
+                           (code[i] & 0x80 ? kRowReset : 0u);
+        if (a != A_PRUNE) rows[o++] = (uint16_t)r;
+        if (out_count(a) == 2) rows[o++] = (uint16_t)(r | kRowChild | kRowFresh);
+    }
     __syncthreads();
-    for (int i0 = 0; i0 < LCHUNK; i0 += LT) {
-        const int64_t j = base + i0 + threadIdx.x;
-        const uint8_t code = j < A.n ? A.action[j] : (uint8_t)A_PRUNE;
-        const uint8_t a = code & 0x7f;
-        const bool reset = code & 0x80;
-        const uint32_t c = out_count(a);
-        uint32_t tot;
-        const uint32_t ex = block_scan_u32(c, sm, tot);
-        const int64_t o = (int64_t)s_carry + ex;
-        for (uint32_t k = 0; k < c; ++k) write_row(A, j, o + k, a, (int)k, reset);
-        // SH rows: each warp copies the rows of its 32 splats, lanes along the row
-        for (int src = 0; src < 32; ++src) {
-            const uint32_t cs = __shfl_sync(0xffffffffu, c, src);
-            if (cs == 0) continue;
-            const int64_t js = __shfl_sync(0xffffffffu, j, src);
-            const int64_t os = __shfl_sync(0xffffffffu, o, src);
-            const uint8_t as = (uint8_t)__shfl_sync(0xffffffffu, (uint32_t)a, src);
-            for (uint32_t k = 0; k < cs; ++k) {
-                const bool fresh = as == A_SPLIT || (as == A_CLONE && k == 1);
-                for (int e = lane; e < A.nsh; e += 32) {
-                    A.out.sh[(os + k) * A.nsh + e] = A.in.sh[js * A.nsh + e];
-                    if (A.moments) {
-                        A.out_m.sh[(os + k) * A.nsh + e] = fresh ? 0.f : A.in_m.sh[js * A.nsh + e];
-                        A.out_v.sh[(os + k) * A.nsh + e] = fresh ? 0.f : A.in_v.sh[js * A.nsh + e];
-                    }
-                }
-            }
+    const int n = (int)tot;
+    copy_rows<LT, NSH, ROWS_COPY>(A.in.sh + j0 * NSH, A.out.sh + o0 * NSH, rows, n);
+    copy_rows<LT, 4, ROWS_COPY>(A.in.quats + 4 * j0, A.out.quats + 4 * o0, rows, n);
+    copy_rows<LT, 3, ROWS_SKIP_SPLIT>(A.in.means + 3 * j0, A.out.means + 3 * o0, rows, n);
+    copy_rows<LT, 3, ROWS_SKIP_SPLIT>(A.in.log_scales + 3 * j0, A.out.log_scales + 3 * o0, rows, n);
+    for (int r = threadIdx.x; r < n; r += LT) {
+        const uint32_t row = rows[r];
+        const int64_t j = j0 + (row & kRowIndex), out = o0 + r;
+        A.out.omega[out] = row & kRowReset ? A.t.reset : A.in.omega[j];
+        if (!(row & kRowSplit)) continue;
+        const float *ls = A.in.log_scales + 3 * j;
+        float R[9];
+        quat_rot(A.in.quats + 4 * j, R);
+        const float *z = A.normals + 6 * j + (row & kRowChild ? 3 : 0);
+        const float v0 = expf(ls[0]) * z[0], v1 = expf(ls[1]) * z[1], v2 = expf(ls[2]) * z[2];
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            A.out.means[3 * out + i] = A.in.means[3 * j + i] + (R[3 * i] * v0 + R[3 * i + 1] * v1 + R[3 * i + 2] * v2);
+            A.out.log_scales[3 * out + i] = ls[i] - A.t.shrink;
         }
-        __syncthreads();
-        if (threadIdx.x == 0) s_carry += tot;
-        __syncthreads();
-        if (base + i0 + LT >= A.n) break;
+    }
+    if (A.moments) {
+        copy_moments<NSH>(A.in_m, A.out_m, j0, o0, rows, n);
+        copy_moments<NSH>(A.in_v, A.out_v, j0, o0, rows, n);
     }
 }
 
@@ -445,7 +425,7 @@ gs_status gs_lifecycle_run(gs_lifecycle *lc, const gs_lifecycle_params *p, int32
         cudaMemsetAsync(lc->block_sum, 0, sizeof(uint32_t), s);
     }
     ++lc->kernel_launches;
-    k_lc_scan<<<1, LT, 0, s>>>(lc->block_sum, n_in > 0 ? nblocks : 0, lc->action, n_in, submap_offsets_in, n_submaps,
+    k_lc_scan<<<1, kScanThreads, 0, s>>>(lc->block_sum, n_in > 0 ? nblocks : 0, lc->action, n_in, submap_offsets_in, n_submaps,
                                out_capacity, lc->block_off, submap_offsets_out, lc->state, n_out);
     gs_status r = check_launch("lifecycle");
     if (r != GS_OK || n_in == 0) return r;
@@ -462,10 +442,14 @@ gs_status gs_lifecycle_run(gs_lifecycle *lc, const gs_lifecycle_params *p, int32
     A.block_off = lc->block_off;
     A.state = lc->state;
     A.n = n_in;
-    A.nsh = 3 * (sh_degree + 1) * (sh_degree + 1);
     A.moments = moments;
     ++lc->kernel_launches;
-    k_lc_scatter<<<nblocks, LT, 0, s>>>(A);
+    switch (sh_degree) {
+        case 0: k_lc_scatter<3><<<nblocks, LT, 0, s>>>(A); break;
+        case 1: k_lc_scatter<12><<<nblocks, LT, 0, s>>>(A); break;
+        case 2: k_lc_scatter<27><<<nblocks, LT, 0, s>>>(A); break;
+        default: k_lc_scatter<48><<<nblocks, LT, 0, s>>>(A);
+    }
     return check_launch("lifecycle_scatter");
 }
 

@@ -22,12 +22,14 @@
 // Partition: a stable split of the splat rows by a flag array into a kept and
 // a moved set; either side may live in host-mapped memory (offload, reload).
 #include "gs_internal.cuh"
+#include "gs_rows.cuh"
 #include "gs_scan.cuh"
 
 #include <cmath>
 
 namespace {
 constexpr unsigned long long kEmpty = ~0ull;
+constexpr int kSelBins = 2048;  // 11-bit digits: three passes over the 32 bits
 }
 
 struct gs_voxel {
@@ -39,8 +41,8 @@ struct gs_voxel {
     int32_t *tknown = nullptr;           // [cap]
     uint32_t *pslot = nullptr;           // [max_points]
     uint32_t *block_sum = nullptr, *block_off = nullptr;  // [nblocks]
-    uint32_t *hist = nullptr;            // [256]
-    uint32_t *sel = nullptr;             // [4] prefix, mask, remaining rank
+    uint32_t *hist = nullptr;            // [kSelBins]
+    uint32_t *sel = nullptr;             // [4] prefix, mask, remaining rank, finished blocks
     int64_t *state = nullptr;            // [0] new splats needed, [1] capacity flag, [2] kept, [3] moved
     int64_t kernel_launches = 0;
 };
@@ -49,7 +51,8 @@ namespace gs {
 namespace {
 
 constexpr int VT = 256;
-constexpr int VCHUNK = 8 * VT;
+constexpr int VCHUNK = kRowChunk;  // items of a block of the ordered kernels
+static_assert(VCHUNK == 2 * VT, "two items a thread");
 constexpr unsigned long long kP1 = 73856093ull, kP2 = 19349663ull, kP3 = 83492791ull;
 constexpr float kY00 = 0.28209479177387814f;
 
@@ -95,14 +98,31 @@ __global__ void __launch_bounds__(VT) k_table_insert(const float *pts, int64_t n
     }
 }
 
-// Probes keys[j] in the table: found -> out[j] = value (or leaves it when
-// `only_found`), and marks the voxel known; not found -> out[j] = miss.
-__global__ void __launch_bounds__(VT) k_table_probe(const unsigned long long *keys, int64_t n,
-                                                    const unsigned long long *tkey, int32_t *tknown, int bits,
-                                                    int32_t *out, int32_t value, bool only_found, int32_t miss) {
+// Empties the table: keys all ones, smallest point index at its largest, no
+// voxel known (one launch, 16-byte stores; the capacity is a multiple of 16).
+__global__ void __launch_bounds__(VT) k_table_clear(unsigned long long *tkey, int32_t *tmin, int32_t *tknown,
+                                                    int64_t cap) {
+    const int64_t stride = (int64_t)gridDim.x * VT;
+    const uint4 ones = make_uint4(~0u, ~0u, ~0u, ~0u), zero = make_uint4(0u, 0u, 0u, 0u);
+    const uint4 large = make_uint4(0x7F7F7F7Fu, 0x7F7F7F7Fu, 0x7F7F7F7Fu, 0x7F7F7F7Fu);
+    for (int64_t i = (int64_t)blockIdx.x * VT + threadIdx.x; i < cap / 4; i += stride) {
+        reinterpret_cast<uint4 *>(tkey)[2 * i] = ones;
+        reinterpret_cast<uint4 *>(tkey)[2 * i + 1] = ones;
+        reinterpret_cast<uint4 *>(tmin)[i] = large;
+        reinterpret_cast<uint4 *>(tknown)[i] = zero;
+    }
+}
+
+// Probes the keys of the device splats (found -> last_used = frame) and of the
+// host-resident ones (reload = found) in one launch, and marks their voxels known.
+__global__ void __launch_bounds__(VT) k_table_probe(const unsigned long long *splat_keys, int64_t n_splats,
+                                                    int32_t *last_used, int32_t frame,
+                                                    const unsigned long long *host_keys, int64_t n_host, int32_t *reload,
+                                                    const unsigned long long *tkey, int32_t *tknown, int bits) {
     const uint32_t mask = (1u << bits) - 1u;
-    for (int64_t j = (int64_t)blockIdx.x * VT + threadIdx.x; j < n; j += (int64_t)gridDim.x * VT) {
-        unsigned long long k = keys[j];
+    for (int64_t j = (int64_t)blockIdx.x * VT + threadIdx.x; j < n_splats + n_host; j += (int64_t)gridDim.x * VT) {
+        const bool host = j >= n_splats;
+        unsigned long long k = host ? host_keys[j - n_splats] : splat_keys[j];
         if (k == kEmpty) k = kEmpty - 1;
         uint32_t s = slot_of(k, bits);
         bool found = false;
@@ -116,8 +136,8 @@ __global__ void __launch_bounds__(VT) k_table_probe(const unsigned long long *ke
             }
             s = (s + 1u) & mask;
         }
-        if (found) out[j] = value;
-        else if (!only_found) out[j] = miss;
+        if (host) reload[j - n_splats] = found ? 1 : 0;
+        else if (found) last_used[j] = frame;
     }
 }
 
@@ -128,39 +148,70 @@ __device__ __forceinline__ uint32_t is_creator(int64_t i, int64_t n, const uint3
     return (tknown[s] == 0 && tmin[s] == (int32_t)i) ? 1u : 0u;
 }
 
-__global__ void __launch_bounds__(VT) k_creator_count(int64_t n, const uint32_t *pslot, const int32_t *tmin,
-                                                      const int32_t *tknown, uint32_t *block_sum) {
-    __shared__ uint32_t sm[VT / 32];
-    const int64_t base = (int64_t)blockIdx.x * VCHUNK;
-    uint32_t c = 0;
-    for (int i = threadIdx.x; i < VCHUNK; i += VT) c += is_creator(base + i, n, pslot, tmin, tknown);
-    const uint32_t t = block_sum_u32<VT>(c, sm);
-    if (threadIdx.x == 0) block_sum[blockIdx.x] = t;
+// Called by every thread after the block's results are written: true in the
+// one block that finishes last, which then sees the others' (and puts the
+// counter back to 0).
+__device__ __forceinline__ bool last_block(uint32_t *done) {
+    __shared__ bool s_last;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        s_last = atomicAdd(done, 1u) == gridDim.x - 1;
+        if (s_last) *done = 0u;
+    }
+    __syncthreads();
+    if (s_last) __threadfence();
+    return s_last;
 }
 
-// One block: exclusive scan of the block sums; total -> state[0] (and *total_out),
-// total > capacity -> state[1].
-__global__ void __launch_bounds__(VT) k_scan_blocks(const uint32_t *block_sum, int nblocks, uint32_t *block_off,
-                                                    int64_t capacity, int64_t *state, int64_t *total_out) {
+// Where a chunk count's exclusive scan goes: total -> state[0] (and *total),
+// total > capacity -> state[1], (items - total, total) -> split[0, 1].
+struct ScanOut {
+    uint32_t *block_sum, *block_off, *done;
+    int64_t capacity;
+    int64_t *state, *total, *split;
+};
+
+// Writes the block's count; the last block scans all of them (eight a thread
+// at a time: a scan of its own cost a launch of 2-4 us).
+__device__ __forceinline__ void count_and_scan(uint32_t c, const ScanOut &S, int64_t items) {
     __shared__ uint32_t sm[VT / 32];
-    __shared__ uint32_t carry;
-    if (threadIdx.x == 0) carry = 0;
-    __syncthreads();
-    for (int b0 = 0; b0 < nblocks; b0 += VT) {
-        const int b = b0 + threadIdx.x;
-        const uint32_t v = b < nblocks ? block_sum[b] : 0u;
-        uint32_t tot;
-        const uint32_t ex = block_scan_u32<VT>(v, sm, tot);
-        if (b < nblocks) block_off[b] = carry + ex;
-        __syncthreads();
-        if (threadIdx.x == 0) carry += tot;
-        __syncthreads();
+    const uint32_t t = block_sum_u32<VT>(c, sm);
+    if (threadIdx.x == 0) S.block_sum[blockIdx.x] = t;
+    if (!last_block(S.done)) return;
+    const int nblocks = (int)gridDim.x;
+    uint32_t carry = 0;
+    for (int b0 = 0; b0 < nblocks; b0 += 8 * VT) {
+        const int b = b0 + 8 * threadIdx.x;
+        uint32_t v[8], sum = 0;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            v[k] = b + k < nblocks ? __ldcg(S.block_sum + b + k) : 0u;
+            sum += v[k];
+        }
+        uint32_t tot, ex = carry + block_scan_u32<VT>(sum, sm, tot);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            if (b + k < nblocks) S.block_off[b + k] = ex;
+            ex += v[k];
+        }
+        carry += tot;
     }
     if (threadIdx.x == 0) {
-        state[0] = carry;
-        state[1] = (int64_t)carry > capacity ? 1 : 0;
-        if (total_out) *total_out = carry;
+        S.state[0] = carry;
+        S.state[1] = (int64_t)carry > S.capacity ? 1 : 0;
+        if (S.total) *S.total = carry;
+        if (S.split) {
+            S.split[0] = items - carry;
+            S.split[1] = carry;
+        }
     }
+}
+
+__global__ void __launch_bounds__(VT) k_creator_count(int64_t n, const uint32_t *pslot, const int32_t *tmin,
+                                                      const int32_t *tknown, ScanOut S) {
+    const int64_t i = (int64_t)blockIdx.x * VCHUNK + threadIdx.x;
+    count_and_scan(is_creator(i, n, pslot, tmin, tknown) + is_creator(i + VT, n, pslot, tmin, tknown), S, n);
 }
 
 struct EmitArgs {
@@ -173,42 +224,52 @@ struct EmitArgs {
     const int64_t *state;
     float *means, *log_scales, *quats, *opacity, *sh;
     unsigned long long *keys;
-    int32_t nsh;
 };
 
+// The new splats of a chunk of points are consecutive: their rows are written
+// element by element, neighbouring threads on neighbouring words (a thread a
+// row, 48 words apart, took 47 us for 0.2M splats of SH degree 3, 11 us).
+template <int NSH>
 __global__ void __launch_bounds__(VT) k_creator_emit(EmitArgs A) {
     __shared__ uint32_t sm[VT / 32];
-    __shared__ uint32_t carry;
+    __shared__ uint16_t rows[VCHUNK];
     if (A.state[1]) return;
-    const int64_t base = (int64_t)blockIdx.x * VCHUNK;
-    if (threadIdx.x == 0) carry = A.block_off[blockIdx.x];
+    const int64_t i0 = (int64_t)blockIdx.x * VCHUNK, o0 = A.block_off[blockIdx.x];
+    const int64_t i = i0 + 2 * threadIdx.x;
+    const uint32_t c0 = is_creator(i, A.n, A.pslot, A.tmin, A.tknown);
+    const uint32_t c1 = is_creator(i + 1, A.n, A.pslot, A.tmin, A.tknown);
+    uint32_t tot;
+    uint32_t o = block_scan_u32<VT>(c0 + c1, sm, tot);
+    if (c0) rows[o++] = (uint16_t)(2 * threadIdx.x);
+    if (c1) rows[o] = (uint16_t)(2 * threadIdx.x + 1);
     __syncthreads();
-    for (int i0 = 0; i0 < VCHUNK; i0 += VT) {
-        const int64_t i = base + i0 + threadIdx.x;
-        const uint32_t c = is_creator(i, A.n, A.pslot, A.tmin, A.tknown);
-        uint32_t tot;
-        const uint32_t ex = block_scan_u32<VT>(c, sm, tot);
-        if (c) {
-            const int64_t o = (int64_t)carry + ex;
-            const float *p = A.pts + 6 * i;
-#pragma unroll
-            for (int r = 0; r < 3; ++r) {
-                A.means[3 * o + r] = p[r];
-                A.log_scales[3 * o + r] = A.log_s;
-            }
-            A.quats[4 * o] = 1.f;
-            A.quats[4 * o + 1] = A.quats[4 * o + 2] = A.quats[4 * o + 3] = 0.f;
-            A.opacity[o] = A.omega;
-            float *sh = A.sh + o * A.nsh;
-#pragma unroll
-            for (int ch = 0; ch < 3; ++ch) sh[ch] = (p[3 + ch] - 0.5f) / kY00;
-            for (int e = 3; e < A.nsh; ++e) sh[e] = 0.f;
-            A.keys[o] = voxel_key(p[0], p[1], p[2], A.v);
+    const int n = (int)tot;
+    const float *pts = A.pts + 6 * i0;
+    for (int e = threadIdx.x; e < 3 * n; e += VT) {
+        const int r = e / 3, ch = e - 3 * r;
+        A.means[3 * o0 + e] = pts[6 * rows[r] + ch];
+        A.log_scales[3 * o0 + e] = A.log_s;
+    }
+    for (int e = threadIdx.x; e < 4 * n; e += VT) A.quats[4 * o0 + e] = (e & 3) == 0 ? 1.f : 0.f;
+    for (int r = threadIdx.x; r < n; r += VT) {
+        const float *p = pts + 6 * rows[r];
+        A.opacity[o0 + r] = A.omega;
+        A.keys[o0 + r] = voxel_key(p[0], p[1], p[2], A.v);
+    }
+    float *sh = A.sh + o0 * NSH;
+    auto dc = [&](int r, int ch) { return (pts[6 * rows[r] + 3 + ch] - 0.5f) / kY00; };
+    if (NSH % 4 == 0 && ((uintptr_t)sh & 15) == 0) {
+        constexpr int W = NSH / 4 > 0 ? NSH / 4 : 1;
+        for (int e = threadIdx.x; e < W * n; e += VT) {
+            const int r = e / W;
+            reinterpret_cast<float4 *>(sh)[e] =
+                e - r * W == 0 ? make_float4(dc(r, 0), dc(r, 1), dc(r, 2), 0.f) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
-        __syncthreads();
-        if (threadIdx.x == 0) carry += tot;
-        __syncthreads();
-        if (base + i0 + VT >= A.n) break;
+    } else {
+        for (int e = threadIdx.x; e < NSH * n; e += VT) {
+            const int r = e / NSH, k = e - r * NSH;
+            sh[e] = k < 3 ? dc(r, k) : 0.f;
+        }
     }
 }
 
@@ -218,77 +279,92 @@ __global__ void __launch_bounds__(VT) k_creator_emit(EmitArgs A) {
 
 __device__ __forceinline__ uint32_t lru_bits(int32_t v) { return (uint32_t)v ^ 0x80000000u; }
 
-__global__ void __launch_bounds__(VT) k_sel_hist(const int32_t *lu, int64_t n, const uint32_t *sel, int shift,
-                                                 uint32_t *hist) {
-    __shared__ uint32_t h[256];
-    h[threadIdx.x] = 0;
-    __syncthreads();
-    const uint32_t prefix = sel[0], mask = sel[1];
-    for (int64_t i = (int64_t)blockIdx.x * VT + threadIdx.x; i < n; i += (int64_t)gridDim.x * VT) {
-        const uint32_t u = lru_bits(lu[i]);
-        if ((u & mask) == prefix) atomicAdd(h + ((u >> shift) & 255u), 1u);
-    }
-    __syncthreads();
-    if (h[threadIdx.x]) atomicAdd(hist + threadIdx.x, h[threadIdx.x]);
-}
-
-// one block of 256: the digit where the remaining rank falls
-__global__ void __launch_bounds__(256) k_sel_pick(uint32_t *hist, uint32_t *sel, int shift) {
-    __shared__ uint32_t sm[8];
-    const uint32_t c = hist[threadIdx.x];
-    uint32_t tot;
-    const uint32_t before = block_scan_u32<256>(c, sm, tot);
-    const uint32_t r = sel[2];
-    __syncthreads();
-    if (before < r && before + c >= r) {
-        sel[0] |= threadIdx.x << shift;
-        sel[1] |= 255u << shift;
-        sel[2] = r - before;
-    }
-    hist[threadIdx.x] = 0;
-}
-
-__global__ void __launch_bounds__(VT) k_sel_eqcount(const int32_t *lu, int64_t n, const uint32_t *sel,
-                                                    uint32_t *block_sum) {
+// One pass of the radix select over an 11-bit digit (the first: prefix and
+// mask 0, rank `rank`): the last block to finish takes the digit in which the
+// remaining rank falls and clears the histogram for the next pass.  (A
+// launch each for the start, every pass and every choice of a digit took 12
+// launches a selection of 2-5 us each; this takes five.)  Values are mostly
+// alike (recent frames), so a warp that agrees on its digit adds once.
+__global__ void __launch_bounds__(VT) k_sel_pass(const int32_t *lu, int64_t n, uint32_t *sel, int shift, int bits,
+                                                 bool first, uint32_t rank, uint32_t *hist) {
+    __shared__ uint32_t h[kSelBins];
     __shared__ uint32_t sm[VT / 32];
-    const int64_t base = (int64_t)blockIdx.x * VCHUNK;
+    for (int i = threadIdx.x; i < kSelBins; i += VT) h[i] = 0;
+    __syncthreads();
+    const uint32_t prefix = first ? 0u : sel[0], mask = first ? 0u : sel[1], left = first ? rank : sel[2];
+    const uint32_t dmask = (1u << bits) - 1u;
+    const int64_t stride = (int64_t)gridDim.x * VT;
+    const int64_t whole = n / VT * VT;  // whole warps take part in the vote
+    for (int64_t i0 = (int64_t)blockIdx.x * VT + threadIdx.x; i0 < whole; i0 += 4 * stride) {
+        uint32_t u[4];  // four loads in flight; the strides past the end are warp-uniform
+#pragma unroll
+        for (int k = 0; k < 4; ++k) u[k] = i0 + k * stride < whole ? lru_bits(lu[i0 + k * stride]) : 0u;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            if (i0 + k * stride >= whole) break;
+            const uint32_t d = (u[k] & mask) == prefix ? (u[k] >> shift) & dmask : ~0u;
+            if (__all_sync(0xffffffffu, d == __shfl_sync(0xffffffffu, d, 0))) {
+                if ((threadIdx.x & 31) == 0 && d != ~0u) atomicAdd(h + d, 32u);
+            } else if (d != ~0u) {
+                atomicAdd(h + d, 1u);
+            }
+        }
+    }
+    if (blockIdx.x == 0 && whole + threadIdx.x < n) {
+        const uint32_t u = lru_bits(lu[whole + threadIdx.x]);
+        if ((u & mask) == prefix) atomicAdd(h + ((u >> shift) & dmask), 1u);
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < kSelBins; i += VT)
+        if (h[i]) atomicAdd(hist + i, h[i]);
+    if (!last_block(sel + 3)) return;
+    constexpr int PER = kSelBins / VT;
+    uint32_t c[PER], sum = 0;
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        c[k] = __ldcg(hist + PER * threadIdx.x + k);
+        sum += c[k];
+    }
+    uint32_t tot, before = block_scan_u32<VT>(sum, sm, tot);
+#pragma unroll
+    for (int k = 0; k < PER; ++k) {
+        if (before < left && before + c[k] >= left) {
+            sel[0] = prefix | (uint32_t)(PER * threadIdx.x + k) << shift;
+            sel[1] = mask | dmask << shift;
+            sel[2] = left - before;
+        }
+        before += c[k];
+        hist[PER * threadIdx.x + k] = 0;
+    }
+}
+
+__global__ void __launch_bounds__(VT) k_sel_eqcount(const int32_t *lu, int64_t n, const uint32_t *sel, ScanOut S) {
+    const int64_t j = (int64_t)blockIdx.x * VCHUNK + threadIdx.x;
     const uint32_t f = sel[0];
     uint32_t c = 0;
-    for (int i = threadIdx.x; i < VCHUNK; i += VT) {
-        const int64_t j = base + i;
-        if (j < n && lru_bits(lu[j]) == f) ++c;
-    }
-    const uint32_t t = block_sum_u32<VT>(c, sm);
-    if (threadIdx.x == 0) block_sum[blockIdx.x] = t;
+#pragma unroll
+    for (int i = 0; i < 2; ++i) c += j + i * VT < n && lru_bits(lu[j + i * VT]) == f;
+    count_and_scan(c, S, n);
 }
 
 __global__ void __launch_bounds__(VT) k_sel_mark(const int32_t *lu, int64_t n, const uint32_t *sel,
                                                  const uint32_t *block_off, int32_t *flags) {
     __shared__ uint32_t sm[VT / 32];
-    __shared__ uint32_t carry;
-    const int64_t base = (int64_t)blockIdx.x * VCHUNK;
+    const int64_t j = (int64_t)blockIdx.x * VCHUNK + 2 * threadIdx.x;
     const uint32_t f = sel[0], r = sel[2];
-    if (threadIdx.x == 0) carry = block_off[blockIdx.x];
-    __syncthreads();
-    for (int i0 = 0; i0 < VCHUNK; i0 += VT) {
-        const int64_t j = base + i0 + threadIdx.x;
-        const uint32_t u = j < n ? lru_bits(lu[j]) : 0xFFFFFFFFu;
-        const uint32_t eq = (j < n && u == f) ? 1u : 0u;
-        uint32_t tot;
-        const uint32_t ex = block_scan_u32<VT>(eq, sm, tot);
-        if (j < n) flags[j] = (u < f || (eq && carry + ex < r)) ? 1 : 0;
-        __syncthreads();
-        if (threadIdx.x == 0) carry += tot;
-        __syncthreads();
-        if (base + i0 + VT >= n) break;
+    uint32_t u[2], eq[2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        u[i] = j + i < n ? lru_bits(lu[j + i]) : 0xFFFFFFFFu;
+        eq[i] = j + i < n && u[i] == f;
     }
-}
-
-__global__ void k_sel_init(uint32_t *sel, uint32_t m) {
-    sel[0] = 0u;
-    sel[1] = 0u;
-    sel[2] = m;
-    sel[3] = 0u;
+    uint32_t tot;
+    uint32_t rank = block_off[blockIdx.x] + block_scan_u32<VT>(eq[0] + eq[1], sm, tot);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        if (j + i < n) flags[j + i] = (u[i] < f || (eq[i] && rank < r)) ? 1 : 0;
+        rank += eq[i];
+    }
 }
 
 __global__ void k_fill_i32(int32_t *p, int64_t n, int32_t v) {
@@ -300,16 +376,12 @@ __global__ void k_fill_i32(int32_t *p, int64_t n, int32_t v) {
 // stable partition
 // ---------------------------------------------------------------------------
 
-__global__ void __launch_bounds__(VT) k_flag_count(const int32_t *flags, int64_t n, uint32_t *block_sum) {
-    __shared__ uint32_t sm[VT / 32];
-    const int64_t base = (int64_t)blockIdx.x * VCHUNK;
+__global__ void __launch_bounds__(VT) k_flag_count(const int32_t *flags, int64_t n, ScanOut S) {
+    const int64_t j = (int64_t)blockIdx.x * VCHUNK + threadIdx.x;
     uint32_t c = 0;
-    for (int i = threadIdx.x; i < VCHUNK; i += VT) {
-        const int64_t j = base + i;
-        if (j < n && flags[j]) ++c;
-    }
-    const uint32_t t = block_sum_u32<VT>(c, sm);
-    if (threadIdx.x == 0) block_sum[blockIdx.x] = t;
+#pragma unroll
+    for (int i = 0; i < 2; ++i) c += j + i * VT < n && flags[j + i * VT] != 0;
+    count_and_scan(c, S, n);
 }
 
 struct PartArgs {
@@ -322,63 +394,49 @@ struct PartArgs {
     unsigned long long *kept_keys, *moved_keys;
     const int32_t *in_lu;
     int32_t *kept_lu, *moved_lu;
-    int32_t nsh;
 };
 
-__device__ __forceinline__ void copy_small(const PartArgs &A, int64_t j, int64_t o, bool mv) {
-    float *const *dst = mv ? A.moved : A.kept;
-#pragma unroll
-    for (int r = 0; r < 3; ++r) {
-        dst[0][3 * o + r] = A.in[0][3 * j + r];
-        dst[1][3 * o + r] = A.in[1][3 * j + r];
-    }
-#pragma unroll
-    for (int r = 0; r < 4; ++r) dst[2][4 * o + r] = A.in[2][4 * j + r];
-    dst[3][o] = A.in[3][j];
-    if (A.in_keys) (mv ? A.moved_keys : A.kept_keys)[o] = A.in_keys[j];
-    if (A.in_lu) (mv ? A.moved_lu : A.kept_lu)[o] = A.in_lu[j];
+// One side's rows of a block's chunk (consecutive there): the arrays one
+// after the other, neighbouring threads on neighbouring words, which also
+// makes whole-line writes of the rows that go to host memory.
+template <int NSH>
+__device__ __forceinline__ void copy_side(const PartArgs &A, int64_t j0, int64_t o0, const uint16_t *rows, int n,
+                                          float *const dst[5], unsigned long long *keys, int32_t *lu) {
+    copy_rows<VT, NSH, ROWS_COPY>(A.in[4] + j0 * NSH, dst[4] + o0 * NSH, rows, n);
+    copy_rows<VT, 3, ROWS_COPY>(A.in[0] + 3 * j0, dst[0] + 3 * o0, rows, n);
+    copy_rows<VT, 3, ROWS_COPY>(A.in[1] + 3 * j0, dst[1] + 3 * o0, rows, n);
+    copy_rows<VT, 4, ROWS_COPY>(A.in[2] + 4 * j0, dst[2] + 4 * o0, rows, n);
+    copy_rows<VT, 1, ROWS_COPY>(A.in[3] + j0, dst[3] + o0, rows, n);
+    if (A.in_keys) copy_elements<VT, 1, ROWS_COPY>(A.in_keys + j0, keys + o0, rows, n);
+    if (A.in_lu) copy_elements<VT, 1, ROWS_COPY>(A.in_lu + j0, lu + o0, rows, n);
 }
 
+template <int NSH>
 __global__ void __launch_bounds__(VT) k_partition(PartArgs A) {
     __shared__ uint32_t sm[VT / 32];
-    __shared__ uint32_t carry;
-    const int64_t base = (int64_t)blockIdx.x * VCHUNK;
-    const int lane = threadIdx.x & 31;
-    if (threadIdx.x == 0) carry = A.block_off[blockIdx.x];
+    __shared__ uint16_t rows[VCHUNK];  // kept rows from the front, moved rows after them
+    const int64_t j0 = (int64_t)blockIdx.x * VCHUNK;
+    const int64_t moved0 = A.block_off[blockIdx.x], kept0 = j0 - moved0;
+    const int n = (int)(A.n - j0 < VCHUNK ? A.n - j0 : VCHUNK);
+    const int i = 2 * threadIdx.x;
+    const uint32_t f0 = i < n && A.flags[j0 + i], f1 = i + 1 < n && A.flags[j0 + i + 1];
+    uint32_t moved;
+    uint32_t m = block_scan_u32<VT>(f0 + f1, sm, moved);  // moved rows before this thread's
+    const int kept = n - (int)moved;
+    if (i < n) rows[f0 ? kept + m : i - m] = (uint16_t)i;
+    m += f0;
+    if (i + 1 < n) rows[f1 ? kept + m : i + 1 - m] = (uint16_t)(i + 1);
     __syncthreads();
-    for (int i0 = 0; i0 < VCHUNK; i0 += VT) {
-        const int64_t j = base + i0 + threadIdx.x;
-        const bool valid = j < A.n;
-        const uint32_t f = valid && A.flags[j] ? 1u : 0u;
-        uint32_t tot;
-        const uint32_t ex = block_scan_u32<VT>(f, sm, tot);
-        const int64_t moved_before = (int64_t)carry + ex;
-        const int64_t o = f ? moved_before : j - moved_before;
-        if (valid) copy_small(A, j, o, f);
-        // SH rows: each warp copies the rows of its 32 splats, lanes along the row
-        for (int src = 0; src < 32; ++src) {
-            const bool vs = __shfl_sync(0xffffffffu, valid, src);
-            if (!vs) continue;
-            const int64_t js = __shfl_sync(0xffffffffu, j, src);
-            const int64_t os = __shfl_sync(0xffffffffu, o, src);
-            const bool fs = __shfl_sync(0xffffffffu, f, src);
-            float *dst = fs ? A.moved[4] : A.kept[4];
-            for (int e = lane; e < A.nsh; e += 32) dst[os * A.nsh + e] = A.in[4][js * A.nsh + e];
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) carry += tot;
-        __syncthreads();
-        if (base + i0 + VT >= A.n) break;
-    }
-}
-
-__global__ void k_partition_counts(const int64_t *state, int64_t n, int64_t *out) {
-    out[0] = n - state[0];
-    out[1] = state[0];
+    copy_side<NSH>(A, j0, moved0, rows + kept, (int)moved, A.moved, A.moved_keys, A.moved_lu);
+    copy_side<NSH>(A, j0, kept0, rows, kept, A.kept, A.kept_keys, A.kept_lu);
 }
 
 int grid_for(int64_t n) { return (int)std::max<int64_t>(1, std::min<int64_t>((n + VT - 1) / VT, 152 * 16)); }
 int nblocks_for(int64_t n) { return (int)std::max<int64_t>(1, (n + VCHUNK - 1) / VCHUNK); }
+
+ScanOut scan_out(gs_voxel *vx, int64_t capacity, int64_t *state, int64_t *total, int64_t *split) {
+    return {vx->block_sum, vx->block_off, vx->sel + 3, capacity, state, total, split};
+}
 
 bool params_set(const gs_param_arrays *a) {
     return a && a->means && a->log_scales && a->quats && a->opacity_logits && a->sh;
@@ -420,11 +478,12 @@ gs_status gs_voxel_create(int64_t max_points, int64_t max_items, gs_voxel **out)
     if (e == cudaSuccess) e = cudaMalloc(&vx->pslot, sizeof(uint32_t) * std::max<int64_t>(1, max_points));
     if (e == cudaSuccess) e = cudaMalloc(&vx->block_sum, sizeof(uint32_t) * nb);
     if (e == cudaSuccess) e = cudaMalloc(&vx->block_off, sizeof(uint32_t) * nb);
-    if (e == cudaSuccess) e = cudaMalloc(&vx->hist, sizeof(uint32_t) * 256);
+    if (e == cudaSuccess) e = cudaMalloc(&vx->hist, sizeof(uint32_t) * kSelBins);
     if (e == cudaSuccess) e = cudaMalloc(&vx->sel, sizeof(uint32_t) * 4);
     if (e == cudaSuccess) e = cudaMalloc(&vx->state, sizeof(int64_t) * 4);
     if (e == cudaSuccess) e = cudaMemset(vx->state, 0, sizeof(int64_t) * 4);
-    if (e == cudaSuccess) e = cudaMemset(vx->hist, 0, sizeof(uint32_t) * 256);
+    if (e == cudaSuccess) e = cudaMemset(vx->hist, 0, sizeof(uint32_t) * kSelBins);
+    if (e == cudaSuccess) e = cudaMemset(vx->sel, 0, sizeof(uint32_t) * 4);
     if (e != cudaSuccess) {
         set_last_error(std::string("gs_voxel_create: ") + cudaGetErrorString(e));
         gs_voxel_destroy(vx);
@@ -461,34 +520,22 @@ gs_status gs_voxel_insert(gs_voxel *vx, const gs_insert_params *p, const float *
     cudaStream_t s = (cudaStream_t)stream;
     const unsigned long long *sk = reinterpret_cast<const unsigned long long *>(splat_keys);
     const unsigned long long *hk = reinterpret_cast<const unsigned long long *>(host_keys);
-    cudaMemsetAsync(vx->tkey, 0xFF, sizeof(unsigned long long) * vx->cap, s);
-    cudaMemsetAsync(vx->tmin, 0x7F, sizeof(int32_t) * vx->cap, s);
-    cudaMemsetAsync(vx->tknown, 0, sizeof(int32_t) * vx->cap, s);
+    ++vx->kernel_launches;
+    k_table_clear<<<grid_for((int64_t)vx->cap / 4), VT, 0, s>>>(vx->tkey, vx->tmin, vx->tknown, (int64_t)vx->cap);
     if (n_points > 0) {
         ++vx->kernel_launches;
         k_table_insert<<<grid_for(n_points), VT, 0, s>>>(points, n_points, p->voxel, vx->tkey, vx->tmin, vx->pslot,
                                                          vx->cap_bits);
     }
-    if (n_splats > 0) {
+    if (n_splats + n_host > 0) {
         ++vx->kernel_launches;
-        k_table_probe<<<grid_for(n_splats), VT, 0, s>>>(sk, n_splats, vx->tkey, vx->tknown, vx->cap_bits, last_used,
-                                                        p->frame, true, 0);
-    }
-    if (n_host > 0) {
-        ++vx->kernel_launches;
-        k_table_probe<<<grid_for(n_host), VT, 0, s>>>(hk, n_host, vx->tkey, vx->tknown, vx->cap_bits, reload, 1, false,
-                                                      0);
+        k_table_probe<<<grid_for(n_splats + n_host), VT, 0, s>>>(sk, n_splats, last_used, p->frame, hk, n_host, reload,
+                                                                 vx->tkey, vx->tknown, vx->cap_bits);
     }
     const int nb = nblocks_for(n_points);
-    if (n_points > 0) {
-        ++vx->kernel_launches;
-        k_creator_count<<<nb, VT, 0, s>>>(n_points, vx->pslot, vx->tmin, vx->tknown, vx->block_sum);
-    } else {
-        cudaMemsetAsync(vx->block_sum, 0, sizeof(uint32_t), s);
-    }
     ++vx->kernel_launches;
-    k_scan_blocks<<<1, VT, 0, s>>>(vx->block_sum, n_points > 0 ? nb : 0, vx->block_off, new_capacity, vx->state,
-                                   n_new);
+    k_creator_count<<<nb, VT, 0, s>>>(n_points, vx->pslot, vx->tmin, vx->tknown,
+                                      scan_out(vx, new_capacity, vx->state, n_new, nullptr));
     gs_status r = check_launch("voxel_insert");
     if (r != GS_OK || n_points == 0) return r;
     EmitArgs A{};
@@ -510,10 +557,14 @@ gs_status gs_voxel_insert(gs_voxel *vx, const gs_insert_params *p, const float *
         A.sh = new_splats->sh;
         A.keys = reinterpret_cast<unsigned long long *>(new_keys);
     }
-    A.nsh = 3 * (sh_degree + 1) * (sh_degree + 1);
     if (new_capacity > 0) {
         ++vx->kernel_launches;
-        k_creator_emit<<<nb, VT, 0, s>>>(A);
+        switch (sh_degree) {
+            case 0: k_creator_emit<3><<<nb, VT, 0, s>>>(A); break;
+            case 1: k_creator_emit<12><<<nb, VT, 0, s>>>(A); break;
+            case 2: k_creator_emit<27><<<nb, VT, 0, s>>>(A); break;
+            default: k_creator_emit<48><<<nb, VT, 0, s>>>(A);
+        }
     }
     return check_launch("voxel_emit");
 }
@@ -548,17 +599,12 @@ gs_status gs_active_select(gs_voxel *vx, const int32_t *last_used, int64_t n, in
         k_fill_i32<<<grid_for(n), VT, 0, s>>>(flags, n, m <= 0 ? 0 : 1);
         return check_launch("active_select");
     }
-    ++vx->kernel_launches;
-    k_sel_init<<<1, 1, 0, s>>>(vx->sel, (uint32_t)m);
-    for (int shift = 24; shift >= 0; shift -= 8) {
-        vx->kernel_launches += 2;
-        k_sel_hist<<<grid_for(n), VT, 0, s>>>(last_used, n, vx->sel, shift, vx->hist);
-        k_sel_pick<<<1, 256, 0, s>>>(vx->hist, vx->sel, shift);
-    }
+    vx->kernel_launches += 5;
+    const int shift[3] = {21, 10, 0}, bits[3] = {11, 11, 10};
+    for (int p = 0; p < 3; ++p)
+        k_sel_pass<<<grid_for(n / 4), VT, 0, s>>>(last_used, n, vx->sel, shift[p], bits[p], p == 0, (uint32_t)m, vx->hist);
     const int nb = nblocks_for(n);
-    vx->kernel_launches += 3;
-    k_sel_eqcount<<<nb, VT, 0, s>>>(last_used, n, vx->sel, vx->block_sum);
-    k_scan_blocks<<<1, VT, 0, s>>>(vx->block_sum, nb, vx->block_off, INT64_MAX, vx->state + 2, nullptr);
+    k_sel_eqcount<<<nb, VT, 0, s>>>(last_used, n, vx->sel, scan_out(vx, INT64_MAX, vx->state + 2, nullptr, nullptr));
     k_sel_mark<<<nb, VT, 0, s>>>(last_used, n, vx->sel, vx->block_off, flags);
     return check_launch("active_select");
 }
@@ -575,18 +621,8 @@ gs_status gs_partition(gs_voxel *vx, const int32_t *flags, int64_t n, int32_t sh
     }
     cudaStream_t s = (cudaStream_t)stream;
     const int nb = nblocks_for(n);
-    if (n > 0) {
-        ++vx->kernel_launches;
-        k_flag_count<<<nb, VT, 0, s>>>(flags, n, vx->block_sum);
-    } else {
-        cudaMemsetAsync(vx->block_sum, 0, sizeof(uint32_t), s);
-    }
-    vx->kernel_launches += 1;
-    k_scan_blocks<<<1, VT, 0, s>>>(vx->block_sum, n > 0 ? nb : 0, vx->block_off, INT64_MAX, vx->state + 2, nullptr);
-    if (counts) {
-        ++vx->kernel_launches;
-        k_partition_counts<<<1, 1, 0, s>>>(vx->state + 2, n, counts);
-    }
+    ++vx->kernel_launches;
+    k_flag_count<<<nb, VT, 0, s>>>(flags, n, scan_out(vx, INT64_MAX, vx->state + 2, nullptr, counts));
     if (n == 0) return check_launch("partition");
     PartArgs A{};
     A.flags = flags;
@@ -606,9 +642,13 @@ gs_status gs_partition(gs_voxel *vx, const int32_t *flags, int64_t n, int32_t sh
     A.in_lu = in_last_used;
     A.kept_lu = kept_last_used;
     A.moved_lu = moved_last_used;
-    A.nsh = 3 * (sh_degree + 1) * (sh_degree + 1);
     ++vx->kernel_launches;
-    k_partition<<<nb, VT, 0, s>>>(A);
+    switch (sh_degree) {
+        case 0: k_partition<3><<<nb, VT, 0, s>>>(A); break;
+        case 1: k_partition<12><<<nb, VT, 0, s>>>(A); break;
+        case 2: k_partition<27><<<nb, VT, 0, s>>>(A); break;
+        default: k_partition<48><<<nb, VT, 0, s>>>(A);
+    }
     return check_launch("partition");
 }
 
