@@ -787,12 +787,10 @@ __global__ void __launch_bounds__(Share<TW, TH, Q>::NT, bwd_blocks(Share<TW, TH,
                         dxi[x] = __fsub_rn((float)(px0 + 8 * x), u.x);
                         u1[x] = __fmaf_rn(u.y, dxi[x], u.z);
                     }
-                    float t2_0 = 0.f;
 #pragma unroll
                     for (int y = 0; y < QY; ++y) {
                         DY[y] = f2_sub(f2_pack((float)(py0 + 8 * y), (float)(py0 + 8 * y + 4)), row.a);
                         const f2 t2 = f2_fma(l.b, DY[y], row.b);
-                        if (y == 0) t2_0 = f2_lo(t2);
                         IN[y] = f2_fma(t2, t2, o.a);
                     }
                     f2 sR = ZERO, sG = ZERO, sB_ = ZERO, sZ = ZERO;  // sums of -wgt dL/dc
@@ -850,37 +848,46 @@ __global__ void __launch_bounds__(Share<TW, TH, Q>::NT, bwd_blocks(Share<TW, TH,
                                 if (E[q] >> j & 1u) quad(q, true);
                         }
                     }
-                    // Moments of the lane's pixels.  Its rows lie 0, 4, 8 and 12
-                    // below the first: with S_k = sum over a column of row^k (-gpw),
-                    // t1 and t2 affine in the row, dy = dy0 + row.
-                    const float dy0 = f2_lo(DY[0]) + ez.z;
+                    // Moments of the lane's pixels about the middle of its rows,
+                    // which lie at -6, -2, 2 and 6 (-2, 2) from there: with S_k = sum
+                    // over a column of row^k (-gpw), t1 and t2 affine in the row,
+                    // dy = dym + row.  (About the first row the terms are up to
+                    // twice as large and cancel.)
+                    constexpr float MID = QY == 2 ? 6.f : 2.f;
+                    const float dyi = f2_lo(DY[0]) + MID, dym = dyi + ez.z;
+                    const float t2_m = __fmaf_rn(e.l.z, dyi, e.row.z);
                     float S0 = 0.f, S1 = 0.f, S2 = 0.f, mU = 0.f, mA = 0.f, mB = 0.f;
 #pragma unroll
                     for (int x = 0; x < QX; ++x) {
-                        float a0, a1, b0 = 0.f, b1 = 0.f;
+                        float a0, a1, s0, s1, s2;
                         f2_unpack(ng[x], a0, a1);
-                        float s0 = a0 + a1, s1 = 4.f * a1, s2 = 16.f * a1;
                         if (QY == 2) {
+                            float b0, b1;
                             f2_unpack(ng[(QY - 1) * QX + x], b0, b1);
-                            s0 += b0 + b1;
-                            s1 = __fmaf_rn(12.f, b1, __fmaf_rn(8.f, b0, s1));
-                            s2 = __fmaf_rn(144.f, b1, __fmaf_rn(64.f, b0, s2));
+                            const float outer = a0 + b1, inner = a1 + b0;
+                            s0 = outer + inner;
+                            s1 = __fmaf_rn(6.f, b1 - a0, 2.f * (b0 - a1));
+                            s2 = __fmaf_rn(36.f, outer, 4.f * inner);
+                        } else {
+                            s0 = a0 + a1;
+                            s1 = 2.f * (a1 - a0);
+                            s2 = 4.f * s0;
                         }
                         const float dx = dxi[x] + u.w;
-                        const float t1_0 = __fmaf_rn(e.l.x, f2_lo(DY[0]), u1[x]);
+                        const float t1_m = __fmaf_rn(e.l.x, dyi, u1[x]);
                         S0 += s0;
                         S1 += s1;
                         S2 += s2;
-                        mU = __fmaf_rn(t1_0, s0, mU);
+                        mU = __fmaf_rn(t1_m, s0, mU);
                         mA = __fmaf_rn(dx * dx, s0, mA);
-                        mB = __fmaf_rn(dx, __fmaf_rn(dy0, s0, s1), mB);
+                        mB = __fmaf_rn(dx, __fmaf_rn(dym, s0, s1), mB);
                     }
                     float *mine_sum = sums + (pending * 32 + lane) * kSumRow;
                     // (u, v, qa, qb), (qc, ln o, r, g), (b, z)
                     *reinterpret_cast<float4 *>(mine_sum) =
-                        make_float4(__fmaf_rn(e.l.x, S1, mU), __fmaf_rn(t2_0, S0, e.l.z * S1), mA, mB);
+                        make_float4(__fmaf_rn(e.l.x, S1, mU), __fmaf_rn(t2_m, S0, e.l.z * S1), mA, mB);
                     *reinterpret_cast<float4 *>(mine_sum + 4) =
-                        make_float4(__fmaf_rn(dy0, __fmaf_rn(dy0, S0, S1), __fmaf_rn(dy0, S1, S2)), S0,
+                        make_float4(__fmaf_rn(dym, __fmaf_rn(dym, S0, S1), __fmaf_rn(dym, S1, S2)), S0,
                                     f2_lo(sR) + f2_hi(sR), f2_lo(sG) + f2_hi(sG));
                     *reinterpret_cast<float2 *>(mine_sum + 8) =
                         make_float2(f2_lo(sB_) + f2_hi(sB_), f2_lo(sZ) + f2_hi(sZ));
