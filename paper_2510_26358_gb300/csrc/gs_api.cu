@@ -139,7 +139,7 @@ void gs_workspace_destroy(gs_workspace *ws) {
                     ws->inst_tile, ws->inst_val, ws->inst_tile_alt, ws->inst_val_alt, ws->ranges,
                     ws->tile_order, ws->order_tot, ws->order_base,
                     ws->last, ws->tfin, ws->vstat, ws->hist, ws->part, ws->digit_tot, ws->pose_part, ws->red_part, ws->ssim_d, ws->ssim_part,
-                    ws->st};
+                    ws->ssim_tile, ws->st};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     for (cudaEvent_t e : ws->ev)
@@ -295,9 +295,11 @@ gs_status gs_workspace_create(const gs_camera *cams, int32_t n_views, const int6
     GS_ALLOC(ws->digit_tot, (size_t)256);
     GS_ALLOC(ws->pose_part, (size_t)std::max(1, blocks) * maxv * 6);
     GS_ALLOC(ws->red_part, (size_t)2 * ws->sort_blocks);
-    ws->n_ssim_tiles = ssim_tiles(ws->views_h);
+    const std::vector<int4> tiles = ssim_tiles(ws->views_h);
+    ws->n_ssim_tiles = (int64_t)tiles.size();
+    GS_ALLOC(ws->ssim_tile, tiles.size());
     GS_ALLOC(ws->ssim_d, (size_t)9 * ws->n_pix);
-    GS_ALLOC(ws->ssim_part, (size_t)std::max<int64_t>(1, ws->n_ssim_tiles));
+    GS_ALLOC(ws->ssim_part, (size_t)2 * std::max<int64_t>(1, ws->n_ssim_tiles));
     GS_ALLOC(ws->st, 1);
 #undef GS_ALLOC
     if (r == GS_OK) {
@@ -308,6 +310,8 @@ gs_status gs_workspace_create(const gs_camera *cams, int32_t n_views, const int6
         if (e == cudaSuccess)
             e = cudaMemcpy(ws->sub_views, ws->sub_views_h.data(), sizeof(int32_t) * ws->sub_views_h.size(),
                            cudaMemcpyHostToDevice);
+        if (e == cudaSuccess)
+            e = cudaMemcpy(ws->ssim_tile, tiles.data(), sizeof(int4) * tiles.size(), cudaMemcpyHostToDevice);
         if (e == cudaSuccess) e = cudaMemset(ws->st, 0, sizeof(DevState));
         if (e == cudaSuccess) e = cudaMemset(ws->ranges, 0, sizeof(uint2) * std::max<int64_t>(1, ws->n_tiles));
         if (e == cudaSuccess) e = cudaMemset(ws->last, 0, sizeof(uint32_t) * std::max<int64_t>(1, ws->n_pix));

@@ -91,9 +91,10 @@ struct gs_workspace {
     uint32_t *digit_tot = nullptr; // [256] digit totals of the current radix pass
     float *pose_part = nullptr;    // [proj_blocks][max_views_per_submap][6]
     double *red_part = nullptr;    // [2][sort_blocks] loss partials
-    int64_t n_ssim_tiles = 0;      // 32x16 SSIM tiles over all channel planes
+    int64_t n_ssim_tiles = 0;      // 32x32 SSIM tiles over all channel planes
+    int4 *ssim_tile = nullptr;     // [n_ssim_tiles] where each lies
     float *ssim_d = nullptr;       // [3][3 n_pix] SSIM partials for the backward
-    double *ssim_part = nullptr;   // [n_ssim_tiles] per-tile sums of the SSIM map
+    double *ssim_part = nullptr;   // [2][n_ssim_tiles] per-tile sums of 1 - SSIM and of |x - y|
     gs::DevState *st = nullptr;
     // host-side order checks
     bool projected = false, binned = false, rendered = false, rendered_var = false;
@@ -156,10 +157,11 @@ gs_status launch_image_l1(gs_workspace *ws, const float *rgb, const float *targe
 // Eq. (6): (1 - lambda) L1 + lambda (1 - SSIM); loss[0..2] = total, L1, 1 - SSIM
 gs_status launch_image_loss(gs_workspace *ws, const float *rgb, const float *target, float lambda,
                             float *loss, float *dL_drgb, cudaStream_t s);
-// SSIM map sums into ws->ssim_part; with dL_drgb, adds grad_scale * dSSIM/dx
-gs_status launch_ssim(gs_workspace *ws, const float *rgb, const float *target, float grad_scale,
-                      float *dL_drgb, cudaStream_t s);
-int64_t ssim_tiles(const std::vector<ViewInfo> &views);
+// SSIM and L1 sums into ws->ssim_part; with dL_drgb and lambda != 0, adds the
+// gradient of both terms
+gs_status launch_ssim(gs_workspace *ws, const float *rgb, const float *target, float lambda, float *dL_drgb,
+                      cudaStream_t s);
+std::vector<int4> ssim_tiles(const std::vector<ViewInfo> &views);  // one entry a CTA of the SSIM kernels
 // occupancy-derived persistent grid sizes for the rasterisers
 gs_status raster_configure(gs_workspace *ws);
 gs_status sort_configure();

@@ -22,6 +22,8 @@
 // them in block order.
 #include "gs_internal.cuh"
 
+#include <algorithm>
+
 namespace gs {
 namespace {
 
@@ -301,19 +303,52 @@ __global__ void __launch_bounds__(LT) k_l1_partial(const float *rgb, const TT *t
 }
 
 // loss[0] = (1 - lambda) L1 + lambda (1 - SSIM), loss[1] = L1, loss[2] = 1 - SSIM
-__global__ void __launch_bounds__(LT) k_image_loss_final(const double *l1part, int nb, const double *spart,
-                                                        int64_t ns, int64_t n, float lambda, float *loss) {
-    __shared__ double sm[32];
-    double a = 0.0, b = 0.0;
-    for (int i = threadIdx.x; i < nb; i += LT) a += l1part[i];
-    for (int64_t i = threadIdx.x; i < ns; i += LT) b += spart[i];
-    const double l1 = block_sum_d(a, sm) / (double)n;
-    const double dssim = block_sum_d(b, sm) / (double)n;  // the SSIM partials hold sums of 1 - S
-    if (threadIdx.x == 0) {
-        loss[0] = (float)((1.0 - (double)lambda) * l1 + (double)lambda * dssim);
-        loss[1] = (float)l1;
-        loss[2] = (float)dssim;
+// from nl partial sums of |x - y| and ns of 1 - S: each block adds a slice of
+// both, the last block the blocks' sums, all in a fixed order.  (Bound by the
+// FP64 adds, two a clock an SM: one block for the 2 x 8280 partials of three
+// 1280x720 views took 10 us, 7 this way.  The last CTA of the SSIM kernel doing
+// it instead cost every CTA a fence and an atomic: 100 -> 124 us.)
+constexpr int kFinalBlocks = 32;
+__global__ void __launch_bounds__(LT) k_image_loss_final(const double *l1part, int64_t nl, const double *spart,
+                                                        int64_t ns, int64_t n, float lambda, double *slice,
+                                                        uint32_t *done, float *loss) {
+    __shared__ double sm[2][LT / 32];
+    static_assert(kFinalBlocks == 32, "a warp adds the slices");
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    auto slice_sum = [&](const double *p, int64_t m) {
+        const int64_t per = (m + kFinalBlocks - 1) / kFinalBlocks, lo = blockIdx.x * per, hi = min(m, lo + per);
+        double v = 0.0;
+        for (int64_t i = lo + threadIdx.x; i < hi; i += LT) v += p[i];
+        return v;
+    };
+    auto warp_sum = [](double v) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        return v;
+    };
+    const double a = warp_sum(slice_sum(l1part, nl)), b = warp_sum(slice_sum(spart, ns));
+    if (lane == 0) {
+        sm[0][w] = a;
+        sm[1][w] = b;
     }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double s = 0.0, t = 0.0;
+        for (int i = 0; i < LT / 32; ++i) {
+            s += sm[0][i];
+            t += sm[1][i];
+        }
+        slice[blockIdx.x] = s;
+        slice[kFinalBlocks + blockIdx.x] = t;
+    }
+    if (!last_block(done) || w != 0) return;
+    const double l1 = warp_sum(__ldcg(slice + lane)) / (double)n;
+    const double dssim = warp_sum(__ldcg(slice + kFinalBlocks + lane)) / (double)n;
+    if (lane != 0) return;
+    loss[0] = (float)((1.0 - (double)lambda) * l1 + (double)lambda * dssim);
+    loss[1] = (float)l1;
+    loss[2] = (float)dssim;
+    *done = 0u;
 }
 
 }  // namespace
@@ -375,20 +410,30 @@ gs_status launch_image_l1_u8(gs_workspace *ws, const float *rgb, const uint8_t *
 
 gs_status launch_image_loss(gs_workspace *ws, const float *rgb, const float *target, float lambda, float *loss,
                             float *dL_drgb, cudaStream_t s) {
-    const int64_t n = 3 * ws->n_pix;
-    const int nb = ws->sort_blocks;
-    {
+    const int64_t n = 3 * ws->n_pix, ns = ws->n_ssim_tiles;
+    // the SSIM kernels take the L1 term along (its sum where x and y are
+    // staged, its gradient in the same read and write); without SSIM in the
+    // gradient the L1 kernel gives gs_image_l1's value and gradient, and SSIM
+    // is only reported
+    const bool fused = (float)((double)lambda / (double)std::max<int64_t>(1, n)) != 0.f;
+    const double *l1part = ws->ssim_part + ns;
+    int64_t nl = ns;
+    gs_status r = GS_OK;
+    if (!fused) {
         StageTimer timer(ws, GS_STAGE_IMAGE_L1, s);
         ++ws->kernel_launches;
-        k_l1_partial<float><<<nb, LT, 0, s>>>(rgb, target, n, dL_drgb, ws->red_part,
-                                       (float)((1.0 - (double)lambda) / (double)n), nullptr, nullptr);
+        l1part = ws->red_part;
+        nl = ws->sort_blocks;
+        k_l1_partial<float><<<(int)nl, LT, 0, s>>>(rgb, target, n, dL_drgb, ws->red_part,
+                                                   (float)((1.0 - (double)lambda) / (double)n), nullptr, nullptr);
+        r = check_launch("image_loss");
     }
-    gs_status r = check_launch("image_loss");
-    if (r != GS_OK) return r;
-    r = launch_ssim(ws, rgb, target, (float)(-(double)lambda / (double)n), dL_drgb, s);
+    if (r == GS_OK) r = launch_ssim(ws, rgb, target, lambda, fused ? dL_drgb : nullptr, s);
     if (r != GS_OK) return r;
     ++ws->kernel_launches;
-    k_image_loss_final<<<1, LT, 0, s>>>(ws->red_part, nb, ws->ssim_part, ws->n_ssim_tiles, n, lambda, loss);
+    // (the slices' sums after the L1 kernel's partials: 2 sort_blocks doubles)
+    k_image_loss_final<<<kFinalBlocks, LT, 0, s>>>(l1part, nl, ws->ssim_part, ns, n, lambda,
+                                                   ws->red_part + ws->sort_blocks, &ws->st->done_l1, loss);
     return check_launch("image_loss");
 }
 

@@ -7,7 +7,7 @@
 //   S = (2 mu_x mu_y + C1)(2 s_xy + C2) / ((mu_x^2 + mu_y^2 + C1)(s_xx + s_yy + C2)).
 //
 // Forward: one CTA per 32x16 output tile of one channel plane stages the tile
-// and its 5-pixel halo of x and y in shared memory, filters the five products
+// and its 5-pixel halo of x and y in shared memory, filters x, y, x^2 + y^2 and xy
 // horizontally, then vertically, and writes S's partial derivatives w.r.t.
 // the three window sums that depend on x,
 //   d1 = dS/dE[x],  d2 = dS/dE[x^2],  d12 = dS/dE[xy],
@@ -47,8 +47,9 @@ namespace {
 
 constexpr int TX = 32, TY = 32, R = 5, K = 2 * R + 1;
 constexpr int IW = TX + 2 * R, IH = TY + 2 * R;
-constexpr int SW = IW + 1;  // staged row stride: odd, so the blocked row reads hit distinct banks
-constexpr int HW = TX + 1;  // filtered row stride
+constexpr int BW = IW + 6;    // staged row: columns x0 - 8 .. x0 + 39 of the plane
+constexpr int BOFF = 3;       // halo column c lives at staged column c + BOFF
+constexpr int HW = TX + 4;    // filtered row stride (16-byte pieces)
 constexpr int NT = 256;
 constexpr int HB = 4;                     // horizontal outputs per thread
 constexpr int HITEMS = IH * (TX / HB);    // 208 row segments per tile
@@ -59,14 +60,14 @@ static_assert(HITEMS <= 2 * NT, "two horizontal passes cover the tile");
 constexpr float C1 = 0.01f * 0.01f, C2 = 0.03f * 0.03f;
 
 struct SsimArgs {
-    const ViewInfo *views;
-    int32_t n_views;
+    const int4 *tiles;   // one a CTA, see locate
     const float *x, *y;  // planar images (rendered, target)
     float *dmap;         // [3][n_elem] partials, nullptr: no backward
     float *grad;         // dL/dx, accumulated
-    double *part;        // [grid] per-CTA sums of 1 - S
+    double *part;        // [2][grid] per-CTA sums of 1 - S and of |x - y|
     int64_t n_elem;
     float scale;         // gradient scale of S (backward)
+    float l1_step;       // gradient scale of |x - y| (backward)
     float gsum;          // sum of the 11 weights (the in-image weight of an interior axis)
     float g[K];          // window weights
     uint32_t *flags;     // workspace state flags (TMA wait time-out)
@@ -82,34 +83,25 @@ struct PlaneTile {
 // TMA path: per view, 3-D maps (x, y, channel) of the two images and a 4-D map
 // (x, y, channel, partial) of the backward's three partial maps.
 constexpr int kTmaViews = 8;
-constexpr int BW = IW + 6;    // box width: columns x0 - 8 .. x0 + 39
-constexpr int BOFF = 3;       // halo column c lives at box column c + BOFF
 struct SsimTma {
     CUtensorMap x[kTmaViews], y[kTmaViews], d[kTmaViews];
 };
 constexpr uint64_t kTmaWaitNs = 1000000000ull;  // 1 s for a tile's copies
 
-// CTA b -> (view, channel, tile); views in order, channels in order, tiles
-// row-major.  The grid holds exactly sum_v 3 ntx(v) nty(v) CTAs.
+// CTA b's tile, from the table made with the workspace: (x0 | y0 << 16,
+// view | channel << 8, W | H << 16, element offset of the plane).  (Worked out
+// from the views by every thread it took some 150 instructions of integer
+// division, 37 a pixel: forward 90 -> 85 us.)
 __device__ __forceinline__ PlaneTile locate(const SsimArgs &A, int b) {
-    PlaneTile p{0, 0, 0, 0, 0, 0, 0};
-    for (int v = 0; v < A.n_views; ++v) {
-        const ViewInfo vi = A.views[v];
-        const int ntx = (vi.W + TX - 1) / TX, nty = (vi.H + TY - 1) / TY;
-        const int per_plane = ntx * nty;
-        if (b < 3 * per_plane) {
-            const int ch = b / per_plane, t = b % per_plane;
-            p.base = 3 * (int64_t)vi.pix_off + (int64_t)ch * vi.W * vi.H;
-            p.W = vi.W;
-            p.H = vi.H;
-            p.x0 = (t % ntx) * TX;
-            p.y0 = (t / ntx) * TY;
-            p.v = v;
-            p.ch = ch;
-            return p;
-        }
-        b -= 3 * per_plane;
-    }
+    const int4 t = __ldg(A.tiles + b);
+    PlaneTile p;
+    p.base = t.w;
+    p.W = t.z & 0xFFFF;
+    p.H = (int)((uint32_t)t.z >> 16);
+    p.x0 = t.x & 0xFFFF;
+    p.y0 = (int)((uint32_t)t.x >> 16);
+    p.v = t.y & 0xFF;
+    p.ch = t.y >> 8;
     return p;
 }
 
@@ -125,71 +117,94 @@ __device__ __forceinline__ float inside_weight(const SsimArgs &A, int i, int n) 
     return w;
 }
 
+// The passes are bound by instruction issue (forward 80 %), so they are laid
+// out for few instructions: staged rows are read and filtered rows written in
+// 16-byte pieces, and x'^2 and y'^2 are filtered as their sum, which is all that
+// S takes of them (three 1280x720 views: forward 99 -> 90 us, 85 with the table
+// of tiles, 75 with five CTAs an SM; the whole loss, whose L1 term and last sum
+// were kernels of their own, 203 -> 164 us).  (Packed f32x2 multiply-adds do not help: the weights are
+// constant-bank operands of the scalar ones, but would need register pairs.)
+using Box = float[IH][BW];
+using Rows = float[IH][HW];
+
+// The HB + 2R staged values behind row segment c0 (a multiple of 4).
+__device__ __forceinline__ void load_segment(const float *row, int c0, float v[HB + 2 * R]) {
+    static_assert(HB == 4 && R == 5 && BOFF == 3, "columns c0 + 3 .. c0 + 16 of the staged row");
+    float t[17];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const float4 x = *reinterpret_cast<const float4 *>(row + c0 + 4 * q);
+        t[4 * q] = x.x;
+        t[4 * q + 1] = x.y;
+        t[4 * q + 2] = x.z;
+        t[4 * q + 3] = x.w;
+    }
+    t[16] = row[c0 + 16];
+#pragma unroll
+    for (int j = 0; j < HB + 2 * R; ++j) v[j] = t[j + BOFF];
+}
+
+__device__ __forceinline__ void filter_segment(const SsimArgs &A, const float v[HB + 2 * R], float *dst) {
+    float o[HB];
+#pragma unroll
+    for (int i = 0; i < HB; ++i) {
+        o[i] = 0.f;
+#pragma unroll
+        for (int k = 0; k < K; ++k) o[i] = __fmaf_rn(A.g[k], v[i + k], o[i]);
+    }
+    *reinterpret_cast<float4 *>(dst) = make_float4(o[0], o[1], o[2], o[3]);
+}
+
 // Horizontal pass of the forward: row segment `item` (row r, columns
-// c0..c0+HB-1) of x', y', x'^2, y'^2 and x'y' from HB + 2R staged x', y'.
-__device__ __forceinline__ void horizontal_fwd(const SsimArgs &A, const float (*src)[IH][SW],
-                                               float (*dst)[IH][HW], int item) {
+// c0..c0+HB-1) of x', y', x'^2 + y'^2 and x'y'.  The staged values are shifted
+// by (cx, cy) here; EDGE: except the zeros outside the image.
+template <bool EDGE>
+__device__ __forceinline__ void horizontal_fwd(const SsimArgs &A, const PlaneTile &P, const Box &bx, const Box &by,
+                                               float cx, float cy, Rows *dst, int item) {
     const int r = item / (TX / HB), c0 = (item % (TX / HB)) * HB;
-    float u[HB + 2 * R], w[HB + 2 * R], uu[HB + 2 * R], ww[HB + 2 * R], uw[HB + 2 * R];
+    float u[HB + 2 * R], w[HB + 2 * R], q[HB + 2 * R], p[HB + 2 * R];
+    load_segment(bx[r], c0, u);
+    load_segment(by[r], c0, w);
+    const bool row_in = P.y0 - R + r >= 0 && P.y0 - R + r < P.H;
 #pragma unroll
     for (int j = 0; j < HB + 2 * R; ++j) {
-        u[j] = src[0][r][c0 + j];
-        w[j] = src[1][r][c0 + j];
-        uu[j] = u[j] * u[j];
-        ww[j] = w[j] * w[j];
-        uw[j] = u[j] * w[j];
+        const int gx = P.x0 - R + c0 + j;
+        const bool in = !EDGE || (row_in && gx >= 0 && gx < P.W);
+        u[j] = in ? u[j] - cx : 0.f;
+        w[j] = in ? w[j] - cy : 0.f;
+        q[j] = __fmaf_rn(u[j], u[j], w[j] * w[j]);
+        p[j] = u[j] * w[j];
     }
-#pragma unroll
-    for (int o = 0; o < HB; ++o) {
-        float a = 0.f, b = 0.f, aa = 0.f, bb = 0.f, ab = 0.f;
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-            a = __fmaf_rn(A.g[k], u[o + k], a);
-            b = __fmaf_rn(A.g[k], w[o + k], b);
-            aa = __fmaf_rn(A.g[k], uu[o + k], aa);
-            bb = __fmaf_rn(A.g[k], ww[o + k], bb);
-            ab = __fmaf_rn(A.g[k], uw[o + k], ab);
-        }
-        dst[0][r][c0 + o] = a;
-        dst[1][r][c0 + o] = b;
-        dst[2][r][c0 + o] = aa;
-        dst[3][r][c0 + o] = bb;
-        dst[4][r][c0 + o] = ab;
-    }
+    filter_segment(A, u, &dst[0][r][c0]);
+    filter_segment(A, w, &dst[1][r][c0]);
+    filter_segment(A, q, &dst[2][r][c0]);
+    filter_segment(A, p, &dst[3][r][c0]);
 }
 
-// Horizontal pass of the backward over NQ staged maps.
-template <int NQ>
-__device__ __forceinline__ void horizontal(const SsimArgs &A, const float (*src)[IH][SW], float (*dst)[IH][HW],
-                                           int item) {
+// Horizontal pass of the backward over the three staged maps.
+__device__ __forceinline__ void horizontal_bwd(const SsimArgs &A, const Box *src, Rows *dst, int item) {
     const int r = item / (TX / HB), c0 = (item % (TX / HB)) * HB;
 #pragma unroll
-    for (int q = 0; q < NQ; ++q) {
+    for (int q = 0; q < 3; ++q) {
         float v[HB + 2 * R];
-#pragma unroll
-        for (int j = 0; j < HB + 2 * R; ++j) v[j] = src[q][r][c0 + j];
-#pragma unroll
-        for (int o = 0; o < HB; ++o) {
-            float acc = 0.f;
-#pragma unroll
-            for (int k = 0; k < K; ++k) acc = __fmaf_rn(A.g[k], v[o + k], acc);
-            dst[q][r][c0 + o] = acc;
-        }
+        load_segment(src[q][r], c0, v);
+        filter_segment(A, v, &dst[q][r][c0]);
     }
 }
 
-// Vertical pass, SSIM, its partials and the tile's sum of 1 - S (shared by
-// both staging paths).
-__device__ __forceinline__ void ssim_epilogue(const SsimArgs &A, const PlaneTile &P, const float (*sh)[IH][HW],
-                                              float cx, float cy, int lx, int ly, double *red) {
+// Vertical pass, SSIM, its partials and the tile's sums (shared by both
+// staging paths).  raw_x, raw_y: the thread's VB pixels (for the L1 term).
+__device__ __forceinline__ void ssim_epilogue(const SsimArgs &A, const PlaneTile &P, const Rows *sh,
+                                              float cx, float cy, const float raw_x[VB], const float raw_y[VB], int lx,
+                                              int ly, double *red) {
     const int gx = P.x0 + lx, oy0 = VB * ly;
-    float m[VB][5];
+    float m[VB][4];
 #pragma unroll
     for (int b = 0; b < VB; ++b)
 #pragma unroll
-        for (int q = 0; q < 5; ++q) m[b][q] = 0.f;
+        for (int q = 0; q < 4; ++q) m[b][q] = 0.f;
 #pragma unroll
-    for (int q = 0; q < 5; ++q) {
+    for (int q = 0; q < 4; ++q) {
         float v[K + VB - 1];
 #pragma unroll
         for (int j = 0; j < K + VB - 1; ++j) v[j] = sh[q][oy0 + j][lx];
@@ -198,28 +213,30 @@ __device__ __forceinline__ void ssim_epilogue(const SsimArgs &A, const PlaneTile
 #pragma unroll
             for (int k = 0; k < K; ++k) m[b][q] = __fmaf_rn(A.g[k], v[b + k], m[b][q]);
     }
-    float dsum = 0.f;  // sum of 1 - S over this thread's pixels
+    float dsum = 0.f, l1 = 0.f;  // sums of 1 - S and |x - y| over this thread's pixels
     const float wx = inside_weight(A, gx, P.W);
 #pragma unroll
     for (int b = 0; b < VB; ++b) {
         const int gy = P.y0 + oy0 + b;
         if (gx >= P.W || gy >= P.H) continue;
+        l1 += fabsf(raw_x[b] - raw_y[b]);
         const float W = wx * inside_weight(A, gy, P.H), cw = 1.f - W;
         const float px = m[b][0], py = m[b][1];  // E[x'], E[y']
         const float mx = __fmaf_rn(cx, W, px), my = __fmaf_rn(cy, W, py);
-        const float sxx = (m[b][2] - px * px) + cw * cx * (2.f * px + cx * W);
-        const float syy = (m[b][3] - py * py) + cw * cy * (2.f * py + cy * W);
-        const float sxy = (m[b][4] - px * py) + cw * (cy * px + cx * py + cx * cy * W);
+        // s_xx + s_yy and s_xy
+        const float sum = (m[b][2] - px * px - py * py) + cw * (cx * (2.f * px + cx * W) + cy * (2.f * py + cy * W));
+        const float sxy = (m[b][3] - px * py) + cw * (cy * px + cx * py + cx * cy * W);
         const float Aa = 2.f * mx * my + C1, B = 2.f * sxy + C2;
-        const float Cc = mx * mx + my * my + C1, D = sxx + syy + C2;
-        const float iC = 1.f / Cc, iD = 1.f / D;
-        const float S = Aa * B * iC * iD;
+        const float Cc = mx * mx + my * my + C1, D = sum + C2;
+        const float inv = 1.f / (Cc * D);
+        const float iC = D * inv, iD = Cc * inv;
+        const float S = Aa * B * inv;
         // 1 - S as (Cc D - A B) / (Cc D): keeps its relative precision near S = 1
-        dsum += __fmaf_rn(Cc, D, -Aa * B) * iC * iD;
+        dsum += __fmaf_rn(Cc, D, -Aa * B) * inv;
         if (A.dmap) {
             const float dsxx = -S * iD;                                      // -A B / (Cc D^2)
-            const float dsxy = 2.f * Aa * iC * iD;                           // 2 A / (Cc D)
-            const float dmu = 2.f * B * iD * (my * Cc - mx * Aa) * iC * iC;  // dS/dmu_x, s fixed
+            const float dsxy = 2.f * Aa * inv;                               // 2 A / (Cc D)
+            const float dmu = 2.f * B * inv * (my * Cc - mx * Aa) * iC;      // dS/dmu_x, s fixed
             const float d1 = dmu - 2.f * mx * dsxx - my * dsxy;
             const int64_t e = P.base + (int64_t)gy * P.W + gx;
             A.dmap[e] = d1;
@@ -227,15 +244,21 @@ __device__ __forceinline__ void ssim_epilogue(const SsimArgs &A, const PlaneTile
             A.dmap[2 * A.n_elem + e] = dsxy;
         }
     }
-    // warp sum in float (at most 64 terms), then the 8 warps in double
+    // warp sums in float (128 terms), then the 8 warps in double
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) dsum += __shfl_xor_sync(0xffffffffu, dsum, o);
-    if (lx == 0) red[ly] = (double)dsum;
+    for (int o = 16; o > 0; o >>= 1) {
+        dsum += __shfl_xor_sync(0xffffffffu, dsum, o);
+        l1 += __shfl_xor_sync(0xffffffffu, l1, o);
+    }
+    if (lx == 0) {
+        red[ly] = (double)dsum;
+        red[NT / 32 + ly] = (double)l1;
+    }
     __syncthreads();
-    if (threadIdx.x == 0) {
+    if (threadIdx.x < 2) {
         double t = 0.0;
-        for (int i = 0; i < NT / 32; ++i) t += red[i];
-        A.part[blockIdx.x] = t;
+        for (int i = 0; i < NT / 32; ++i) t += red[threadIdx.x * (NT / 32) + i];
+        A.part[threadIdx.x * gridDim.x + blockIdx.x] = t;
     }
 }
 
@@ -261,7 +284,7 @@ __device__ __forceinline__ BwdOut ssim_bwd_prefetch(const SsimArgs &A, const Pla
     return o;
 }
 
-__device__ __forceinline__ void ssim_bwd_epilogue(const SsimArgs &A, const PlaneTile &P, const float (*sh)[IH][HW],
+__device__ __forceinline__ void ssim_bwd_epilogue(const SsimArgs &A, const PlaneTile &P, const Rows *sh,
                                                   int lx, int ly, const BwdOut &o) {
     const int gx = P.x0 + lx, oy0 = VB * ly;
     float f[VB][3];
@@ -284,14 +307,17 @@ __device__ __forceinline__ void ssim_bwd_epilogue(const SsimArgs &A, const Plane
         const int gy = P.y0 + oy0 + b;
         if (gx >= P.W || gy >= P.H) continue;
         const int64_t e = P.base + (int64_t)gy * P.W + gx;
-        A.grad[e] = o.g[b] + A.scale * (f[b][0] + 2.f * o.x[b] * f[b][1] + o.y[b] * f[b][2]);
+        // the L1 term's step first, as the L1 kernel adds it
+        const float d = o.x[b] - o.y[b];
+        const float g = o.g[b] + (d > 0.f ? A.l1_step : (d < 0.f ? -A.l1_step : 0.f));
+        A.grad[e] = g + A.scale * (f[b][0] + 2.f * o.x[b] * f[b][1] + o.y[b] * f[b][2]);
     }
 }
 
 __global__ void __launch_bounds__(NT) k_ssim_fwd(SsimArgs A) {
-    __shared__ float st[2][IH][SW];  // staged x', y'
-    __shared__ float sh[5][IH][HW];
-    __shared__ double red[NT / 32];
+    __shared__ __align__(16) Box st[2];  // staged x', y'
+    __shared__ __align__(16) Rows sh[4];
+    __shared__ double red[2 * NT / 32];
     const PlaneTile P = locate(A, blockIdx.x);
     const float *x = A.x + P.base, *y = A.y + P.base;
     const int tid = threadIdx.x, lx = tid & 31, ly = tid >> 5;
@@ -313,20 +339,28 @@ __global__ void __launch_bounds__(NT) k_ssim_fwd(SsimArgs A) {
         for (int k = 0; k < SLOADS; ++k) {
             const int i = tid + k * NT;
             if (i < IH * IW) {
-                st[0][i / IW][i % IW] = vx[k];
-                st[1][i / IW][i % IW] = vy[k];
+                st[0][i / IW][i % IW + BOFF] = vx[k];
+                st[1][i / IW][i % IW + BOFF] = vy[k];
             }
         }
     }
+    float rx[VB], ry[VB];
+#pragma unroll
+    for (int b = 0; b < VB; ++b) {
+        const int gx = P.x0 + lx, gy = P.y0 + VB * ly + b;
+        const bool in = gx < P.W && gy < P.H;
+        rx[b] = in ? x[(int64_t)gy * P.W + gx] : 0.f;
+        ry[b] = in ? y[(int64_t)gy * P.W + gx] : 0.f;
+    }
     __syncthreads();
-    for (int item = tid; item < HITEMS; item += NT) horizontal_fwd(A, st, sh, item);
+    for (int item = tid; item < HITEMS; item += NT) horizontal_fwd<false>(A, P, st[0], st[1], 0.f, 0.f, sh, item);
     __syncthreads();
-    ssim_epilogue(A, P, sh, cx, cy, lx, ly, red);
+    ssim_epilogue(A, P, sh, cx, cy, rx, ry, lx, ly, red);
 }
 
-__global__ void __launch_bounds__(NT) k_ssim_bwd(SsimArgs A) {
-    __shared__ float st[3][IH][SW];
-    __shared__ float sh[3][IH][HW];
+__global__ void __launch_bounds__(NT, 4) k_ssim_bwd(SsimArgs A) {
+    __shared__ __align__(16) Box st[3];
+    __shared__ __align__(16) Rows sh[3];
     const PlaneTile P = locate(A, blockIdx.x);
     const int tid = threadIdx.x, lx = tid & 31, ly = tid >> 5;
     const BwdOut out = ssim_bwd_prefetch(A, P, lx, ly);
@@ -346,12 +380,12 @@ __global__ void __launch_bounds__(NT) k_ssim_bwd(SsimArgs A) {
             const int i = tid + k * NT;
             if (i < IH * IW) {
 #pragma unroll
-                for (int q = 0; q < 3; ++q) st[q][i / IW][i % IW] = v[q][k];
+                for (int q = 0; q < 3; ++q) st[q][i / IW][i % IW + BOFF] = v[q][k];
             }
         }
     }
     __syncthreads();
-    for (int item = tid; item < HITEMS; item += NT) horizontal<3>(A, st, sh, item);
+    for (int item = tid; item < HITEMS; item += NT) horizontal_bwd(A, st, sh, item);
     __syncthreads();
     ssim_bwd_epilogue(A, P, sh, lx, ly, out);
 }
@@ -434,12 +468,12 @@ __global__ void k_wait_selftest(uint32_t *flags, uint64_t limit_ns, int32_t *res
     if (threadIdx.x == 0) *result = done ? 0 : 1;
 }
 
-__global__ void __launch_bounds__(NT) k_ssim_fwd_tma(SsimArgs A, const __grid_constant__ SsimTma T) {
-    __shared__ __align__(128) float tx_[IH][BW];
-    __shared__ __align__(128) float ty_[IH][BW];
-    __shared__ float sh[5][IH][HW];
+__global__ void __launch_bounds__(NT, 5) k_ssim_fwd_tma(SsimArgs A, const __grid_constant__ SsimTma T) {
+    __shared__ __align__(128) Box tx_;
+    __shared__ __align__(128) Box ty_;
+    __shared__ __align__(16) Rows sh[4];
     __shared__ __align__(8) uint64_t bar;
-    __shared__ double red[NT / 32];
+    __shared__ double red[2 * NT / 32];
     const PlaneTile P = locate(A, blockIdx.x);
     const int tid = threadIdx.x, lx = tid & 31, ly = tid >> 5;
     if (tid == 0) {
@@ -452,46 +486,24 @@ __global__ void __launch_bounds__(NT) k_ssim_fwd_tma(SsimArgs A, const __grid_co
     if (!tma_wait(&bar, A.flags, A.wait_ns)) return;
     // shift: the tile's first pixel (halo row R, column R)
     const float cx = tx_[R][R + BOFF], cy = ty_[R][R + BOFF];
-    for (int item = tid; item < HITEMS; item += NT) {
-        const int r = item / (TX / HB), c0 = (item % (TX / HB)) * HB;
-        const int gy = P.y0 - R + r;
-        const bool row_in = gy >= 0 && gy < P.H;
-        float u[HB + 2 * R], w[HB + 2 * R], uu[HB + 2 * R], ww[HB + 2 * R], uw[HB + 2 * R];
+    if (P.x0 >= R && P.y0 >= R && P.x0 + TX + R <= P.W && P.y0 + TY + R <= P.H) {
+        for (int item = tid; item < HITEMS; item += NT) horizontal_fwd<false>(A, P, tx_, ty_, cx, cy, sh, item);
+    } else {
+        for (int item = tid; item < HITEMS; item += NT) horizontal_fwd<true>(A, P, tx_, ty_, cx, cy, sh, item);
+    }
+    float rx[VB], ry[VB];
 #pragma unroll
-        for (int j = 0; j < HB + 2 * R; ++j) {
-            const int gx = P.x0 - R + c0 + j;
-            const bool in = row_in && gx >= 0 && gx < P.W;
-            u[j] = in ? tx_[r][c0 + j + BOFF] - cx : 0.f;
-            w[j] = in ? ty_[r][c0 + j + BOFF] - cy : 0.f;
-            uu[j] = u[j] * u[j];
-            ww[j] = w[j] * w[j];
-            uw[j] = u[j] * w[j];
-        }
-#pragma unroll
-        for (int o = 0; o < HB; ++o) {
-            float a = 0.f, b = 0.f, aa = 0.f, bb = 0.f, ab = 0.f;
-#pragma unroll
-            for (int k = 0; k < K; ++k) {
-                a = __fmaf_rn(A.g[k], u[o + k], a);
-                b = __fmaf_rn(A.g[k], w[o + k], b);
-                aa = __fmaf_rn(A.g[k], uu[o + k], aa);
-                bb = __fmaf_rn(A.g[k], ww[o + k], bb);
-                ab = __fmaf_rn(A.g[k], uw[o + k], ab);
-            }
-            sh[0][r][c0 + o] = a;
-            sh[1][r][c0 + o] = b;
-            sh[2][r][c0 + o] = aa;
-            sh[3][r][c0 + o] = bb;
-            sh[4][r][c0 + o] = ab;
-        }
+    for (int b = 0; b < VB; ++b) {
+        rx[b] = tx_[R + VB * ly + b][lx + R + BOFF];
+        ry[b] = ty_[R + VB * ly + b][lx + R + BOFF];
     }
     __syncthreads();
-    ssim_epilogue(A, P, sh, cx, cy, lx, ly, red);
+    ssim_epilogue(A, P, sh, cx, cy, rx, ry, lx, ly, red);
 }
 
 __global__ void __launch_bounds__(NT) k_ssim_bwd_tma(SsimArgs A, const __grid_constant__ SsimTma T) {
-    __shared__ __align__(128) float sd[3][IH][BW];
-    __shared__ float sh[3][IH][HW];
+    __shared__ __align__(128) Box sd[3];
+    __shared__ __align__(16) Rows sh[3];
     __shared__ __align__(8) uint64_t bar;
     const PlaneTile P = locate(A, blockIdx.x);
     const int tid = threadIdx.x, lx = tid & 31, ly = tid >> 5;
@@ -504,22 +516,7 @@ __global__ void __launch_bounds__(NT) k_ssim_bwd_tma(SsimArgs A, const __grid_co
     __syncthreads();
     const BwdOut out = ssim_bwd_prefetch(A, P, lx, ly);
     if (!tma_wait(&bar, A.flags, A.wait_ns)) return;
-    for (int item = tid; item < HITEMS; item += NT) {
-        const int r = item / (TX / HB), c0 = (item % (TX / HB)) * HB;
-#pragma unroll
-        for (int q = 0; q < 3; ++q) {
-            float v[HB + 2 * R];
-#pragma unroll
-            for (int j = 0; j < HB + 2 * R; ++j) v[j] = sd[q][r][c0 + j + BOFF];
-#pragma unroll
-            for (int o = 0; o < HB; ++o) {
-                float acc = 0.f;
-#pragma unroll
-                for (int k = 0; k < K; ++k) acc = __fmaf_rn(A.g[k], v[o + k], acc);
-                sh[q][r][c0 + o] = acc;
-            }
-        }
-    }
+    for (int item = tid; item < HITEMS; item += NT) horizontal_bwd(A, sd, sh, item);
     __syncthreads();
     ssim_bwd_epilogue(A, P, sh, lx, ly, out);
 }
@@ -572,17 +569,25 @@ bool encode_maps(gs_workspace *ws, const float *rgb, const float *target, SsimTm
 
 }  // namespace
 
-int64_t ssim_tiles(const std::vector<ViewInfo> &views) {
-    int64_t n = 0;
-    for (const ViewInfo &v : views) n += 3 * (int64_t)((v.W + TX - 1) / TX) * ((v.H + TY - 1) / TY);
-    return n;
+std::vector<int4> ssim_tiles(const std::vector<ViewInfo> &views) {
+    std::vector<int4> tiles;  // views in order, channels in order, tiles row-major
+    for (int v = 0; v < (int)views.size(); ++v) {
+        const ViewInfo &vi = views[v];
+        for (int ch = 0; ch < 3; ++ch)
+            for (int y = 0; y < vi.H; y += TY)
+                for (int x = 0; x < vi.W; x += TX)
+                    tiles.push_back(make_int4(x | y << 16, v | ch << 8, vi.W | vi.H << 16,
+                                              3 * vi.pix_off + ch * vi.W * vi.H));
+    }
+    return tiles;
 }
 
-gs_status launch_ssim(gs_workspace *ws, const float *rgb, const float *target, float grad_scale, float *dL_drgb,
+gs_status launch_ssim(gs_workspace *ws, const float *rgb, const float *target, float lambda, float *dL_drgb,
                       cudaStream_t s) {
     SsimArgs A{};
-    A.views = ws->views;
-    A.n_views = ws->n_views;
+    const double n = 3.0 * (double)ws->n_pix;
+    const float grad_scale = (float)(-(double)lambda / n);
+    A.tiles = ws->ssim_tile;
     A.x = rgb;
     A.y = target;
     A.dmap = dL_drgb && grad_scale != 0.f ? ws->ssim_d : nullptr;
@@ -590,6 +595,7 @@ gs_status launch_ssim(gs_workspace *ws, const float *rgb, const float *target, f
     A.part = ws->ssim_part;
     A.n_elem = 3 * ws->n_pix;
     A.scale = grad_scale;
+    A.l1_step = (float)((1.0 - (double)lambda) / n);
     A.flags = &ws->st->flags;
     A.wait_ns = kTmaWaitNs;
     double g[K], sum = 0.0;
