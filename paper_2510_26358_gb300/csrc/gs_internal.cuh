@@ -38,7 +38,8 @@ struct DevState {
     float depth_scale;          // lambda_L / |Omega| of the last gs_depth_loss
     uint32_t depth_valid;
     uint32_t done_l1, done_depth;  // finished blocks of the loss reductions (the last one finishes)
-    uint32_t pad[5];
+    uint32_t done_parts;  // finished blocks of the binning's counting kernels
+    uint32_t pad[4];
     unsigned long long frag_count[4];  // gs_workspace_fragment_counts
 };
 constexpr uint32_t kFlagCapacity = 1u;
@@ -85,10 +86,10 @@ struct gs_workspace {
     float *tfin = nullptr;         // [n_pix]
     float4 *vstat = nullptr;       // [n_pix] depth (mean, var, 1/W, 0) of the variance forward
     // scratch
-    uint32_t *hist = nullptr;      // [256][hist_cols]
+    uint32_t *hist = nullptr;      // [512][hist_cols]
     int32_t hist_cols = 0;         // max(2 sort_blocks, wide_blocks): the most blocks a radix pass may run
     uint32_t *part = nullptr;      // [max(sort_blocks, wide_blocks) + 1]
-    uint32_t *digit_tot = nullptr; // [256] digit totals of the current radix pass
+    uint32_t *digit_tot = nullptr; // [512] digit totals of the current radix pass
     float *pose_part = nullptr;    // [proj_blocks][max_views_per_submap][6]
     double *red_part = nullptr;    // [2][sort_blocks] loss partials
     int64_t n_ssim_tiles = 0;      // 32x32 SSIM tiles over all channel planes

@@ -125,6 +125,16 @@ struct Share {
     __device__ static constexpr int wy(int w) { return (w / NWX) * 8 * QY; }
 };
 
+// The next tile in work order, or -1.  Every CTA draws one number past the
+// tiles; the last of these puts the counter back for the next launch (a clearing
+// launch before each pass cost 1-2 us).
+__device__ __forceinline__ int next_tile(const RasterArgs &A) {
+    const uint32_t w = atomicAdd(A.counter, 1u);
+    if (w < (uint32_t)A.n_tiles) return (int)A.order[w];
+    if (w == (uint32_t)A.n_tiles + gridDim.x - 1u) *A.counter = 0u;
+    return -1;
+}
+
 // Which quadrants a staged Gaussian can reach, bit w * Q + q for quadrant q
 // of warp w: the tile test of the binning on the quadrant's box of pixel
 // centres, with fixed paddings (0.1 % and 0.01 px) that exceed the rounding of
@@ -205,8 +215,7 @@ __global__ void __launch_bounds__(Share<TW, TH, Q>::NT, fwd_blocks(Share<TW, TH,
     for (;;) {
         __syncthreads();
         if (tid == 0) {
-            const uint32_t w = atomicAdd(A.counter, 1u);
-            s_tile = w < (uint32_t)A.n_tiles ? (int)A.order[w] : -1;
+            s_tile = next_tile(A);
         }
         __syncthreads();
         const int tile = s_tile;
@@ -471,8 +480,7 @@ __global__ void __launch_bounds__(TW * TH / PF, VAR ? 640 / (TW * TH / PF) : 0) 
     for (;;) {
         __syncthreads();
         if (tid == 0) {
-            const uint32_t w = atomicAdd(A.counter, 1u);
-            s_tile = w < (uint32_t)A.n_tiles ? (int)A.order[w] : -1;
+            s_tile = next_tile(A);
         }
         __syncthreads();
         const int tile = s_tile;
@@ -669,8 +677,7 @@ __global__ void __launch_bounds__(Share<TW, TH, Q>::NT, bwd_blocks(Share<TW, TH,
     for (;;) {
         __syncthreads();
         if (tid == 0) {
-            const uint32_t w = atomicAdd(A.counter, 1u);
-            s_tile = w < (uint32_t)A.n_tiles ? (int)A.order[w] : -1;
+            s_tile = next_tile(A);
         }
         __syncthreads();
         const int tile = s_tile;
@@ -1026,7 +1033,6 @@ gs_status launch_raster_fwd(gs_workspace *ws, float *rgb, float *depth, float *a
         A.var_out = var;
         A.vstat = ws->vstat;
     }
-    cudaMemsetAsync(A.counter, 0, sizeof(uint32_t), s);
     return run(ws, A, true, mean != nullptr, s);
 }
 
@@ -1054,7 +1060,6 @@ gs_status launch_raster_bwd(gs_workspace *ws, const float *dL_drgb, const float 
         if (r != GS_OK) return r;
     }
     ws->g2d_clear = false;
-    cudaMemsetAsync(A.counter, 0, sizeof(uint32_t), s);
     return run(ws, A, false, var, s);
 }
 

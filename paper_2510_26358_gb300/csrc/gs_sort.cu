@@ -16,7 +16,7 @@
 // kernels run a fixed grid of `sort_blocks` blocks, each owning a contiguous
 // chunk of ceil(n / blocks) rounded to a whole tile.
 //
-// The radix sort is a reduce-then-scan LSD sort with 8-bit digits:
+// The radix sort is a reduce-then-scan LSD sort with 8- or 9-bit digits:
 //   hist     per-block digit counts -> table[digit][block]
 //   scan     exclusive scan of the table (digit-major) -> global offsets
 //   scatter  per block, tile by tile in order: stable in-tile ranks from warp
@@ -73,53 +73,75 @@ __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t *s
 // loads), so that the compaction takes few block-wide scans.
 constexpr int kCompactStep = 8 * T;
 
-__global__ void __launch_bounds__(T) k_count_visible(const uint32_t *pkey, uint32_t n, uint32_t *part,
-                                                    int nb) {
-    __shared__ uint32_t sm[32];
-    uint32_t lo, hi;
-    chunk_range(n, blockIdx.x, nb, kCompactStep, lo, hi);
-    uint32_t c = 0;
-    for (uint32_t i = lo + threadIdx.x; i < hi; i += T) c += pkey[i] != kInvalidKey;
-    uint32_t tot;
-    block_exclusive_scan(c, sm, &tot);
-    if (threadIdx.x == 0) part[blockIdx.x] = tot;
+// What becomes of the scanned total: the visible pairs, or the instances,
+// which are checked against the capacity.  Every binning starts the flags
+// afresh: capacity for this one, no device-wait time-out yet.
+__device__ __forceinline__ void store_instances(DevState *st, unsigned long long total, uint64_t cap) {
+    st->n_inst_needed = total;
+    st->flags = total > cap ? kFlagCapacity : 0u;
+    st->n_inst = total > cap ? 0u : (uint32_t)total;
 }
 
-// exclusive scan of part[0..nb) in place by one block; the total goes to *total
-// and, when cap > 0, is checked against the capacity
-__global__ void k_scan_parts(uint32_t *part, int nb, uint32_t *total, DevState *st, uint64_t cap,
-                             int mode) {
-    __shared__ uint32_t sm[32];
-    __shared__ unsigned long long carry;
-    if (threadIdx.x == 0) carry = 0;
-    __syncthreads();
-    for (int base = 0; base < nb; base += T) {
-        int i = base + threadIdx.x;
-        uint32_t v = i < nb ? part[i] : 0u;
-        uint32_t tot;
-        uint32_t ex = block_exclusive_scan(v, sm, &tot);
-        if (i < nb) part[i] = (uint32_t)(carry + ex);
+// Called by every thread of every block with its count: the last block to
+// finish scans the blocks' sums into part (exclusive) and stores the total.  (A
+// launch of its own took 3 us and the gap to it.)  The sums are 64-bit: a
+// total past 32 bits is past any capacity, and the offsets are then not used.
+template <bool INSTANCES>
+__device__ __forceinline__ void scan_parts(uint32_t count, uint32_t *part, DevState *st, uint64_t cap, uint32_t *sm) {
+    __shared__ unsigned long long s_sum[W];
+    __shared__ bool s_last;
+    const int nb = gridDim.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    auto block_sum = [&](unsigned long long v) {  // in every thread
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
         __syncthreads();
-        if (threadIdx.x == 0) carry += tot;
+        if (lane == 0) s_sum[w] = v;
         __syncthreads();
-    }
+        unsigned long long t = 0;
+#pragma unroll
+        for (int j = 0; j < W; ++j) t += s_sum[j];
+        return t;
+    };
+    const unsigned long long mine = block_sum(count);
     if (threadIdx.x == 0) {
-        unsigned long long t = carry;
-        if (mode == 0) {
-            *total = (uint32_t)t;
-        } else {
-            st->n_inst_needed = t;
-            // every binning starts the flags afresh: capacity for this one,
-            // no device-wait time-out yet
-            if (t > cap) {
-                st->flags = kFlagCapacity;
-                st->n_inst = 0;
-            } else {
-                st->flags = 0u;
-                st->n_inst = (uint32_t)t;
-            }
-        }
+        part[blockIdx.x] = (uint32_t)min(mine, 0xFFFFFFFFull);
+        __threadfence();
+        s_last = atomicAdd(&st->done_parts, 1u) == (uint32_t)nb - 1;
     }
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    uint32_t v[4], sum = 0;  // nb <= 4 T
+    unsigned long long wide = 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int i = 4 * threadIdx.x + k;
+        v[k] = i < nb ? __ldcg(part + i) : 0u;
+        sum += v[k];
+        wide += v[k];
+    }
+    uint32_t tot, ex = block_exclusive_scan(sum, sm, &tot);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int i = 4 * threadIdx.x + k;
+        if (i < nb) part[i] = ex;
+        ex += v[k];
+    }
+    wide = block_sum(wide);
+    if (threadIdx.x == 0) {
+        st->done_parts = 0u;
+        if (INSTANCES) store_instances(st, wide, cap);
+        else st->n_vis = (uint32_t)wide;
+    }
+}
+
+__global__ void __launch_bounds__(T) k_count_visible(const uint32_t *pkey, uint32_t n, uint32_t *part, DevState *st) {
+    __shared__ uint32_t sm[32];
+    uint32_t lo, hi;
+    chunk_range(n, blockIdx.x, gridDim.x, kCompactStep, lo, hi);
+    uint32_t c = 0;
+    for (uint32_t i = lo + threadIdx.x; i < hi; i += T) c += pkey[i] != kInvalidKey;
+    scan_parts<false>(c, part, st, 0, sm);
 }
 
 __global__ void __launch_bounds__(T) k_compact_visible(const uint32_t *pkey, uint32_t n, const uint32_t *part,
@@ -170,23 +192,27 @@ __global__ void __launch_bounds__(T) k_compact_visible(const uint32_t *pkey, uin
 // radix sort passes (count n read from the device)
 // ---------------------------------------------------------------------------
 
+template <int BITS>
 __global__ void __launch_bounds__(T) k_radix_hist(const uint32_t *keys, const uint32_t *n_ptr, int shift,
                                                  uint32_t *hist, int nb, int tile) {
-    __shared__ uint32_t h[W][256];
-    for (int i = threadIdx.x; i < W * 256; i += T) (&h[0][0])[i] = 0;
+    constexpr int D = 1 << BITS;
+    __shared__ uint32_t h[W][D];
+    for (int i = threadIdx.x; i < W * D; i += T) (&h[0][0])[i] = 0;
     __syncthreads();
     uint32_t lo, hi;
     chunk_range(*n_ptr, blockIdx.x, nb, tile, lo, hi);
     int w = threadIdx.x >> 5;
-    for (uint32_t i = lo + threadIdx.x; i < hi; i += T) atomicAdd(&h[w][(keys[i] >> shift) & 255u], 1u);
+    for (uint32_t i = lo + threadIdx.x; i < hi; i += T) atomicAdd(&h[w][(keys[i] >> shift) & (D - 1u)], 1u);
     __syncthreads();
-    uint32_t s = 0;
+    for (int d = threadIdx.x; d < D; d += T) {
+        uint32_t s = 0;
 #pragma unroll
-    for (int j = 0; j < W; ++j) s += h[j][threadIdx.x];
-    hist[threadIdx.x * nb + blockIdx.x] = s;
+        for (int j = 0; j < W; ++j) s += h[j][d];
+        hist[(size_t)d * nb + blockIdx.x] = s;
+    }
 }
 
-// Exclusive scan of each digit's row of the [256][nb] table: block d turns
+// Exclusive scan of each digit's row of the [digits][nb] table: block d turns
 // row d into offsets relative to the digit's first slot and writes the row
 // total to dtot[d].  The digit bases (prefix of dtot) are added by the
 // scatter kernel.  nb <= 4 * T.
@@ -230,12 +256,13 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 template <int R>
 constexpr bool kScatterAhead = R >= 4;
 
-template <int R>
+template <int R, int BITS>
 struct ScatterSmem {
+    static constexpr int D = 1 << BITS;
     uint32_t key[kScatterAhead<R> ? 2 : 1][T * R];
     uint32_t val[kScatterAhead<R> ? 2 : 1][T * R];
-    uint32_t wcnt[W][256];  // per-warp digit counts, then per-warp digit offsets
-    uint32_t base[256], tcnt[256], tstart[256];
+    uint32_t wcnt[W][D];  // per-warp digit counts, then per-warp digit offsets
+    uint32_t base[D], tcnt[D], tstart[D];
     uint32_t scan[32];
 };
 
@@ -249,7 +276,7 @@ struct ScatterSmem {
 // reordered by digit in shared memory and written out in coalesced runs at
 // the global offsets.  Stable: sub-tiles, rounds and lanes follow the input
 // order.
-template <int R>
+template <int R, int BITS>
 __global__ void __launch_bounds__(T) k_radix_scatter(const uint32_t *kin, const uint32_t *vin,
                                                     uint32_t *kout, uint32_t *vout,
                                                     const uint32_t *n_ptr, int shift,
@@ -257,15 +284,22 @@ __global__ void __launch_bounds__(T) k_radix_scatter(const uint32_t *kin, const 
     constexpr int TILE = T * R;
     constexpr int WT = 32 * R;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    ScatterSmem<R> &S = *reinterpret_cast<ScatterSmem<R> *>(smem_raw);
+    ScatterSmem<R, BITS> &S = *reinterpret_cast<ScatterSmem<R, BITS> *>(smem_raw);
+    constexpr int D = 1 << BITS, PER = D / T;  // digits, and digits a thread (consecutive)
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
     uint32_t lo, hi;
     chunk_range(*n_ptr, blockIdx.x, nb, TILE, lo, hi);
     if (lo >= hi) return;
     {
-        uint32_t tot;
-        uint32_t digit_base = block_exclusive_scan(dtot[t], S.scan, &tot);
-        S.base[t] = digit_base + hist[t * nb + blockIdx.x];
+        uint32_t tot, c[PER], sum = 0;
+#pragma unroll
+        for (int k = 0; k < PER; ++k) sum += c[k] = dtot[PER * t + k];
+        uint32_t digit_base = block_exclusive_scan(sum, S.scan, &tot);
+#pragma unroll
+        for (int k = 0; k < PER; ++k) {
+            S.base[PER * t + k] = digit_base + hist[(size_t)(PER * t + k) * nb + blockIdx.x];
+            digit_base += c[k];
+        }
     }
     const uint32_t lt = lanemask_lt();
     // asynchronous copy of the tile at t1 into buffer bi in sixteen-byte
@@ -298,7 +332,7 @@ __global__ void __launch_bounds__(T) k_radix_scatter(const uint32_t *kin, const 
             }
         }
 #pragma unroll
-        for (int j = 0; j < W; ++j) S.wcnt[j][t] = 0;
+        for (int j = 0; j < W * PER; ++j) (&S.wcnt[0][0])[j * T + t] = 0;
         __syncthreads();
         uint32_t key[R], val[R], rank[R];
 #pragma unroll
@@ -310,10 +344,10 @@ __global__ void __launch_bounds__(T) k_radix_scatter(const uint32_t *kin, const 
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             const bool valid = (uint32_t)(w * WT + r * 32 + lane) < tn;
-            const uint32_t d = (key[r] >> shift) & 255u;
+            const uint32_t d = (key[r] >> shift) & (D - 1u);
             uint32_t m = __ballot_sync(0xffffffffu, valid);
 #pragma unroll
-            for (int b = 0; b < 8; ++b) {
+            for (int b = 0; b < BITS; ++b) {
                 const uint32_t bb = __ballot_sync(0xffffffffu, (d >> b) & 1u);
                 m &= ((d >> b) & 1u) ? bb : ~bb;
             }
@@ -325,21 +359,30 @@ __global__ void __launch_bounds__(T) k_radix_scatter(const uint32_t *kin, const 
             __syncwarp();
         }
         __syncthreads();
-        uint32_t run = 0;
+        uint32_t cnt[PER], sum = 0;
 #pragma unroll
-        for (int j = 0; j < W; ++j) {
-            const uint32_t c = S.wcnt[j][t];
-            S.wcnt[j][t] = run;
-            run += c;
+        for (int k = 0; k < PER; ++k) {
+            uint32_t run = 0;
+#pragma unroll
+            for (int j = 0; j < W; ++j) {
+                const uint32_t c = S.wcnt[j][PER * t + k];
+                S.wcnt[j][PER * t + k] = run;
+                run += c;
+            }
+            S.tcnt[PER * t + k] = cnt[k] = run;
+            sum += run;
         }
-        S.tcnt[t] = run;
-        uint32_t tot;
-        S.tstart[t] = block_exclusive_scan(run, S.scan, &tot);
+        uint32_t tot, start = block_exclusive_scan(sum, S.scan, &tot);
+#pragma unroll
+        for (int k = 0; k < PER; ++k) {
+            S.tstart[PER * t + k] = start;
+            start += cnt[k];
+        }
         __syncthreads();
 #pragma unroll
         for (int r = 0; r < R; ++r) {
             if ((uint32_t)(w * WT + r * 32 + lane) < tn) {
-                const uint32_t d = (key[r] >> shift) & 255u;
+                const uint32_t d = (key[r] >> shift) & (D - 1u);
                 const uint32_t lp = S.tstart[d] + S.wcnt[w][d] + rank[r];
                 S.key[bi][lp] = key[r];
                 S.val[bi][lp] = val[r];
@@ -351,14 +394,15 @@ __global__ void __launch_bounds__(T) k_radix_scatter(const uint32_t *kin, const 
             const uint32_t j = t + r * T;
             if (j < tn) {
                 const uint32_t k = S.key[bi][j];
-                const uint32_t d = (k >> shift) & 255u;
+                const uint32_t d = (k >> shift) & (D - 1u);
                 const uint32_t o = S.base[d] + (j - S.tstart[d]);
                 kout[o] = k;
                 vout[o] = S.val[bi][j];
             }
         }
         __syncthreads();
-        S.base[t] += S.tcnt[t];
+#pragma unroll
+        for (int k = 0; k < PER; ++k) S.base[PER * t + k] += S.tcnt[PER * t + k];
     }
 }
 
@@ -379,12 +423,12 @@ constexpr int kOffsetStep = 4 * T;
 
 // instance count of every sorted visible pair (into ioff) and of every block's chunk
 __global__ void __launch_bounds__(T) k_count_instances(const uint32_t *vis_pair, const short4 *rect,
-                                                      const DevState *st, uint32_t *ioff, uint32_t *part,
-                                                      int nb) {
+                                                      DevState *st, uint32_t *ioff, uint32_t *part,
+                                                      uint64_t cap) {
     __shared__ uint32_t sm[32];
     uint32_t n = st->n_vis;
     uint32_t lo, hi;
-    chunk_range(n, blockIdx.x, nb, kOffsetStep, lo, hi);
+    chunk_range(n, blockIdx.x, gridDim.x, kOffsetStep, lo, hi);
     uint32_t c = 0;
     for (uint32_t i0 = lo + 4 * threadIdx.x; i0 < hi; i0 += kOffsetStep) {
         uint32_t pr[4];
@@ -401,14 +445,20 @@ __global__ void __launch_bounds__(T) k_count_instances(const uint32_t *vis_pair,
             c += k;
         }
     }
-    uint32_t tot;
-    block_exclusive_scan(c, sm, &tot);
-    if (threadIdx.x == 0) part[blockIdx.x] = tot;
+    scan_parts<true>(c, part, st, cap, sm);
 }
 
-// ioff[i] <- first output slot of sorted pair i (exclusive scan of the counts);
 // win_pair[w] <- the pair that owns slot w * kEmitWindow (every slot belongs to
 // exactly one pair, so each window start is written once)
+__device__ __forceinline__ void mark_windows(uint32_t pair, uint32_t start, uint32_t count, uint32_t *win_pair,
+                                             uint32_t n_win) {
+    for (uint32_t w = (start + kEmitWindow - 1) / kEmitWindow;
+         count > 0 && w < n_win && w * (uint64_t)kEmitWindow < (uint64_t)start + count; ++w)
+        win_pair[w] = pair;
+}
+
+// ioff[i] <- first output slot of sorted pair i (exclusive scan of the counts),
+// and the owners of the emission windows' first slots
 __global__ void __launch_bounds__(T) k_instance_offsets(const DevState *st, const uint32_t *part, int nb,
                                                        uint32_t *ioff, uint32_t *win_pair, uint32_t n_win) {
     __shared__ uint32_t sm[32];
@@ -431,9 +481,7 @@ __global__ void __launch_bounds__(T) k_instance_offsets(const DevState *st, cons
             const uint32_t i = i0 + u;
             if (i >= hi) break;
             ioff[i] = start;
-            for (uint32_t w = (start + kEmitWindow - 1) / kEmitWindow;
-                 c[u] > 0 && w < n_win && w * (uint64_t)kEmitWindow < (uint64_t)start + c[u]; ++w)
-                win_pair[w] = i;
+            mark_windows(i, start, c[u], win_pair, n_win);
             start += c[u];
         }
         base += tot;
@@ -472,7 +520,7 @@ static_assert(kEmitWindow == T * kEmitPerThread, "a window is a whole number of 
 __global__ void __launch_bounds__(T, kEmitBlocksPerSM) k_emit_instances(
     const uint32_t *vis_pair, const short4 *rect, const float4 *rec, const ViewInfo *views, int n_views,
     const Consts k, const DevState *st, const uint32_t *ioff, const uint32_t *win_pair, uint32_t *inst_tile,
-    uint32_t *inst_val) {
+    uint32_t *inst_val, uint2 *ranges, uint32_t n_tiles) {
     __shared__ uint32_t s_off[kEmitWindow];
     __shared__ uint32_t s_pair[kEmitWindow];
     __shared__ short4 s_rect[kEmitWindow];    // (x0, y0, width, view)
@@ -482,6 +530,8 @@ __global__ void __launch_bounds__(T, kEmitBlocksPerSM) k_emit_instances(
     __shared__ int32_t s_poff[GS_MAX_VIEWS];  // first pair of each view
     __shared__ uint32_t s_range[2];
     __shared__ uint32_t s_wmax[T / 32];
+    // the tiles' ranges start empty (filled after the tile sort)
+    for (uint32_t i = blockIdx.x * T + threadIdx.x; i < n_tiles; i += gridDim.x * T) ranges[i] = make_uint2(0u, 0u);
     if (st->flags & kFlagCapacity) return;
     const uint32_t n = st->n_vis, total = st->n_inst;
     const uint32_t windows = (total + kEmitWindow - 1) / kEmitWindow;
@@ -665,12 +715,233 @@ __global__ void __launch_bounds__(256) k_order_place(const uint2 *ranges, int n_
         order[atomicAdd(&cur[order_bucket(ranges[i])], 1u)] = (uint32_t)i;
 }
 
-// One stable pass over bits [shift, shift+8) by nb blocks; swaps in/out.
+// ---------------------------------------------------------------------------
+// small maps
+// ---------------------------------------------------------------------------
+
+// Up to kSmallPairs (view, Gaussian) pairs: compaction, depth sort, instance
+// counts and offsets in one launch of one block, instead of 17 launches of
+// 2-4 us each, whatever their work.  The sort is the same stable LSD radix sort
+// (ballot ranks, per-warp counts) on keys in shared memory, bound by the
+// instruction issue of its one SM: 9-bit digits of the keys' distance to the
+// smallest, so that 27 bits of range take three passes (10,000 pairs, 8088
+// visible: four passes of 8 bits 41 us, three of 9 38 us).  With what follows a
+// single tile pass it took the forward of a 161x119 view (3001 pairs) from
+// 162 to 85 us.
+constexpr int kSmallPairs = 16384, kSmallThreads = 1024, kSmallWarps = kSmallThreads / 32;
+constexpr int kSmallPer = kSmallPairs / kSmallThreads;
+constexpr int kSmallBits = 9, kSmallDigits = 1 << kSmallBits;
+struct SmallSmem {
+    uint32_t key[kSmallPairs];
+    uint16_t pair[kSmallPairs];
+    uint16_t wcnt[kSmallWarps][kSmallDigits];
+    uint32_t start[kSmallDigits];
+    uint32_t warp[32], lowest, highest;
+};
+
+// exclusive scan of one value a thread over kSmallThreads threads
+__device__ __forceinline__ uint32_t small_scan(uint32_t v, uint32_t *sm, uint32_t &total) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    uint32_t x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    __syncthreads();
+    if (lane == 31) sm[w] = x;
+    __syncthreads();
+    uint32_t s = sm[lane];  // kSmallWarps == 32
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, s, o);
+        if (lane >= o) s += y;
+    }
+    total = __shfl_sync(0xffffffffu, s, 31);
+    const uint32_t before = __shfl_sync(0xffffffffu, s, w > 0 ? w - 1 : 0);
+    return (w > 0 ? before : 0u) + x - v;
+}
+
+__global__ void __launch_bounds__(kSmallThreads) k_bin_small(const uint32_t *pkey, uint32_t n, const short4 *rect,
+                                                             DevState *st, uint64_t cap, uint32_t *vis_pair,
+                                                             uint32_t *ioff, uint32_t *win_pair, uint32_t n_win) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    SmallSmem &S = *reinterpret_cast<SmallSmem *>(smem_raw);
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    const uint32_t lt = lanemask_lt();
+    uint32_t key[kSmallPer], pair[kSmallPer], rank[kSmallPer], tot;
+    // each warp takes a run of `rounds` x 32 consecutive elements
+    uint32_t rounds = (n + kSmallThreads - 1) / kSmallThreads;
+    uint32_t lowest, range;
+    {
+        if (t == 0) {
+            S.lowest = kInvalidKey;
+            S.highest = 0u;
+        }
+        uint32_t c = 0, lo = kInvalidKey, hi = 0u;
+#pragma unroll
+        for (int r = 0; r < kSmallPer; ++r) {
+            const uint32_t i = (w * rounds + r) * 32 + lane;
+            key[r] = r < (int)rounds && i < n ? pkey[i] : kInvalidKey;
+        }
+#pragma unroll
+        for (int r = 0; r < kSmallPer; ++r) {
+            c += __popc(__ballot_sync(0xffffffffu, key[r] != kInvalidKey));
+            lo = min(lo, key[r]);
+            hi = max(hi, key[r] != kInvalidKey ? key[r] : 0u);
+        }
+        lo = __reduce_min_sync(0xffffffffu, lo);
+        hi = __reduce_max_sync(0xffffffffu, hi);
+        __syncthreads();
+        if (lane == 0) {
+            atomicMin(&S.lowest, lo);
+            atomicMax(&S.highest, hi);
+        }
+        uint32_t o = small_scan(lane == 0 ? c : 0u, S.warp, tot);
+        o = __shfl_sync(0xffffffffu, o, 0);
+        lowest = S.lowest;
+        range = tot ? S.highest - lowest : 0u;
+#pragma unroll
+        for (int r = 0; r < kSmallPer; ++r) {
+            const uint32_t m = __ballot_sync(0xffffffffu, key[r] != kInvalidKey);
+            if (key[r] != kInvalidKey) {
+                const uint32_t p = o + __popc(m & lt);
+                S.key[p] = key[r] - lowest;
+                S.pair[p] = (uint16_t)((w * rounds + r) * 32 + lane);
+            }
+            o += __popc(m);
+        }
+    }
+    const uint32_t m = tot;
+    rounds = (m + kSmallThreads - 1) / kSmallThreads;
+    __syncthreads();
+    for (int shift = 0; shift < 32 && range >> shift; shift += kSmallBits) {
+        for (int i = t; i < kSmallWarps * kSmallDigits / 2; i += kSmallThreads) reinterpret_cast<uint32_t *>(S.wcnt)[i] = 0;
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < kSmallPer; ++r) {
+            if (r >= (int)rounds) break;
+            const uint32_t i = (w * rounds + r) * 32 + lane;
+            const bool valid = i < m;
+            key[r] = valid ? S.key[i] : 0u;
+            pair[r] = valid ? S.pair[i] : 0u;
+            const uint32_t d = (key[r] >> shift) & (kSmallDigits - 1u);
+            uint32_t same = __ballot_sync(0xffffffffu, valid);
+#pragma unroll
+            for (int b = 0; b < kSmallBits; ++b) {
+                const uint32_t bb = __ballot_sync(0xffffffffu, (d >> b) & 1u);
+                same &= ((d >> b) & 1u) ? bb : ~bb;
+            }
+            const uint32_t below = same & lt;
+            const uint32_t before = valid ? S.wcnt[w][d] : 0u;
+            rank[r] = before + __popc(below);
+            __syncwarp();
+            if (valid && below == 0) S.wcnt[w][d] = (uint16_t)(before + __popc(same));
+            __syncwarp();
+        }
+        __syncthreads();
+        uint32_t run = 0;
+        if (t < kSmallDigits) {
+#pragma unroll 8
+            for (int j = 0; j < kSmallWarps; ++j) {
+                const uint32_t c = S.wcnt[j][t];
+                S.wcnt[j][t] = (uint16_t)run;
+                run += c;
+            }
+        }
+        uint32_t all;
+        const uint32_t start = small_scan(run, S.warp, all);
+        if (t < kSmallDigits) S.start[t] = start;
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < kSmallPer; ++r) {
+            if (r >= (int)rounds) break;
+            if ((w * rounds + r) * 32 + lane < m) {
+                const uint32_t d = (key[r] >> shift) & (kSmallDigits - 1u);
+                const uint32_t p = S.start[d] + S.wcnt[w][d] + rank[r];
+                S.key[p] = key[r];
+                S.pair[p] = (uint16_t)pair[r];
+            }
+        }
+        __syncthreads();
+    }
+    // instance counts and offsets: `rounds` consecutive sorted pairs a thread
+    uint32_t cnt[kSmallPer], sum = 0;
+#pragma unroll
+    for (int r = 0; r < kSmallPer; ++r) {
+        const uint32_t i = t * rounds + r;
+        const bool in = r < (int)rounds && i < m;
+        const uint32_t p = in ? S.pair[i] : 0u;
+        if (in) vis_pair[i] = p;
+        cnt[r] = in ? rect_tiles(rect[p]) : 0u;
+    }
+#pragma unroll
+    for (int r = 0; r < kSmallPer; ++r) sum += cnt[r];
+    // (at most 16384 pairs of 2^20 tiles: beyond 32 bits only past the capacity)
+    unsigned long long wide = sum;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) wide += __shfl_xor_sync(0xffffffffu, wide, o);
+    __shared__ unsigned long long s_wide[kSmallWarps];
+    if (lane == 0) s_wide[w] = wide;
+    uint32_t low, at = small_scan(sum, S.warp, low);
+    wide = s_wide[lane];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) wide += __shfl_xor_sync(0xffffffffu, wide, o);
+    if (t == 0) {
+        st->n_vis = m;
+        store_instances(st, wide, cap);
+    }
+    if (wide > cap) return;
+#pragma unroll
+    for (int r = 0; r < kSmallPer; ++r) {
+        const uint32_t i = t * rounds + r;
+        if (r >= (int)rounds || i >= m) break;
+        ioff[i] = at;
+        mark_windows(i, at, cnt[r], win_pair, n_win);
+        at += cnt[r];
+    }
+}
+
+// Ranges and raster work order when one pass sorted the instances (at most
+// 512 digits): the digit totals are the lists' lengths.  One block.
+__global__ void __launch_bounds__(512) k_ranges_small(const uint32_t *dtot, const DevState *st, int n_tiles, uint2 *ranges,
+                                                      uint32_t *order) {
+    __shared__ uint32_t sm[16], cnt[kOrderBuckets], first[kOrderBuckets];
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    if (t < kOrderBuckets) cnt[t] = 0;
+    const bool ok = !(st->flags & kFlagCapacity);
+    const uint32_t c = ok && t < n_tiles ? dtot[t] : 0u;
+    uint32_t x = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) sm[w] = x;
+    __syncthreads();
+    for (int j = 0; j < w; ++j) x += sm[j];
+    const uint2 rg = c ? make_uint2(x - c, x) : make_uint2(0u, 0u);
+    uint32_t mine = 0;
+    if (t < n_tiles) {
+        ranges[t] = rg;
+        mine = atomicAdd(&cnt[order_bucket(rg)], 1u);
+    }
+    __syncthreads();
+    if (t < kOrderBuckets) {
+        uint32_t s = 0;
+        for (int j = 0; j < t; ++j) s += cnt[j];
+        first[t] = s;
+    }
+    __syncthreads();
+    if (t < n_tiles) order[first[order_bucket(rg)] + mine] = (uint32_t)t;
+}
+
+// One stable pass over bits [shift, shift + BITS) by nb blocks; swaps in/out.
 // R = 8 rounds (2048-key tiles) on twice the blocks for the instance sort
 // (64 registers: one full wave of four blocks per SM; measured 0.0725 ->
 // 0.068 ms against R = 16 on one block per two SMs' worth), R = 2 or 4 for
 // the smaller sort of the visible pairs (see its launch).
-template <int R>
+template <int R, int BITS>
 gs_status radix_pass(gs_workspace *ws, uint32_t *&k, uint32_t *&v, uint32_t *&k2, uint32_t *&v2,
                      const uint32_t *n_ptr, int shift, int nb, cudaStream_t s) {
     // the digit table has a column per block, and the scan takes at most 4 T
@@ -679,11 +950,11 @@ gs_status radix_pass(gs_workspace *ws, uint32_t *&k, uint32_t *&v, uint32_t *&k2
                        std::to_string(ws->hist_cols) + " columns)");
         return GS_ERR_INVALID_ARG;
     }
-    ++ws->kernel_launches; k_radix_hist<<<nb, T, 0, s>>>(k, n_ptr, shift, ws->hist, nb, T * R);
-    ++ws->kernel_launches; k_radix_scan<<<256, T, 0, s>>>(ws->hist, nb, ws->digit_tot);
+    ++ws->kernel_launches; k_radix_hist<BITS><<<nb, T, 0, s>>>(k, n_ptr, shift, ws->hist, nb, T * R);
+    ++ws->kernel_launches; k_radix_scan<<<1 << BITS, T, 0, s>>>(ws->hist, nb, ws->digit_tot);
     ++ws->kernel_launches;
-    k_radix_scatter<R><<<nb, T, sizeof(ScatterSmem<R>), s>>>(k, v, k2, v2, n_ptr, shift, ws->hist,
-                                                             ws->digit_tot, nb);
+    k_radix_scatter<R, BITS><<<nb, T, sizeof(ScatterSmem<R, BITS>), s>>>(k, v, k2, v2, n_ptr, shift, ws->hist,
+                                                                         ws->digit_tot, nb);
     std::swap(k, k2);
     std::swap(v, v2);
     return check_launch("radix_pass");
@@ -692,12 +963,15 @@ gs_status radix_pass(gs_workspace *ws, uint32_t *&k, uint32_t *&v, uint32_t *&k2
 }  // namespace
 
 gs_status sort_configure() {
-    cudaError_t e = cudaFuncSetAttribute(k_radix_scatter<8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)sizeof(ScatterSmem<8>));
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_radix_scatter<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)sizeof(ScatterSmem<2>));
-
+    cudaError_t e = cudaSuccess;
+    auto allow = [&](const void *fn, size_t bytes) {
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    };
+    allow((const void *)k_radix_scatter<8, 8>, sizeof(ScatterSmem<8, 8>));
+    allow((const void *)k_radix_scatter<8, 9>, sizeof(ScatterSmem<8, 9>));
+    allow((const void *)k_radix_scatter<4, 8>, sizeof(ScatterSmem<4, 8>));
+    allow((const void *)k_radix_scatter<2, 8>, sizeof(ScatterSmem<2, 8>));
+    allow((const void *)k_bin_small, sizeof(SmallSmem));
     if (e != cudaSuccess) {
         set_last_error(std::string("sort_configure: ") + cudaGetErrorString(e));
         return GS_ERR_CUDA;
@@ -706,76 +980,93 @@ gs_status sort_configure() {
 }
 
 gs_status launch_bin_sort(gs_workspace *ws, cudaStream_t s) {
-    int nb = ws->sort_blocks;
-    uint32_t n_pairs = (uint32_t)ws->n_pairs;
+    const int nb = ws->sort_blocks, nw = ws->wide_blocks;
+    const uint32_t n_pairs = (uint32_t)ws->n_pairs, n_tiles = (uint32_t)ws->n_tiles;
+    const uint32_t n_win = (uint32_t)(ws->inst_cap / kEmitWindow + 2);
+    const uint64_t cap = (uint64_t)ws->inst_cap;
     DevState *st = ws->st;
-    cudaMemsetAsync(&st->n_vis, 0, sizeof(uint32_t) * 2 + sizeof(unsigned long long) + sizeof(uint32_t), s);
-    // 1. compaction of visible pairs (more blocks than the other stages: each
-    //    block's chunk is a chain of block-wide scans)
     gs_status r;
-    const int nw = ws->wide_blocks;
-    {
-    StageTimer timer(ws, GS_STAGE_COMPACT, s);
-    ++ws->kernel_launches; k_count_visible<<<nw, T, 0, s>>>(ws->pkey, n_pairs, ws->part, nw);
-    ++ws->kernel_launches; k_scan_parts<<<1, T, 0, s>>>(ws->part, nw, &st->n_vis, st, 0, 0);
-    ++ws->kernel_launches; k_compact_visible<<<nw, T, 0, s>>>(ws->pkey, n_pairs, ws->part, nw, ws->vis_key, ws->vis_pair);
-    r = check_launch("compact");
-    if (r != GS_OK) return r;
+    const uint32_t *v = ws->vis_pair;  // the visible pairs in depth order
+    if (n_pairs <= (uint32_t)kSmallPairs) {
+        // 1-3 (up to the offsets) in one launch
+        StageTimer timer(ws, GS_STAGE_DEPTH_SORT, s);
+        ++ws->kernel_launches;
+        k_bin_small<<<1, kSmallThreads, sizeof(SmallSmem), s>>>(ws->pkey, n_pairs, ws->rect, st, cap, ws->vis_pair,
+                                                                ws->ioff, ws->win_pair, n_win);
+        if ((r = check_launch("bin_small")) != GS_OK) return r;
+    } else {
+        // 1. compaction of visible pairs (more blocks than the other stages: each
+        //    block's chunk is a chain of block-wide scans)
+        {
+            StageTimer timer(ws, GS_STAGE_COMPACT, s);
+            ws->kernel_launches += 2;
+            k_count_visible<<<nw, T, 0, s>>>(ws->pkey, n_pairs, ws->part, st);
+            k_compact_visible<<<nw, T, 0, s>>>(ws->pkey, n_pairs, ws->part, nw, ws->vis_key, ws->vis_pair);
+            if ((r = check_launch("compact")) != GS_OK) return r;
+        }
+        // 2. stable sort of the visible pairs by depth key (32 bits)
+        StageTimer timer(ws, GS_STAGE_DEPTH_SORT, s);
+        uint32_t *k = ws->vis_key, *p = ws->vis_pair, *k2 = ws->vis_key_alt, *p2 = ws->vis_pair_alt;
+        // (blocks grow with the pairs: a tenth of them or so are visible; more
+        // blocks than keys to fill them only lengthen the digit-table scans)
+        const int nd = (int)std::min<int64_t>(nw, std::max<int64_t>(nb, ws->n_pairs / 16384));
+        // four keys a thread once the blocks hold several tiles each (orchard4m,
+        // 3.08 M visible of 24 M pairs: 0.175 -> 0.164 ms), two below (orchard500k,
+        // 148k of 1.5 M: 0.063 ms against 0.065 with four)
+        const bool wide = ws->n_pairs >= (int64_t)8 << 20;
+        for (int sh = 0; sh < 32; sh += 8)
+            if ((r = wide ? radix_pass<4, 8>(ws, k, p, k2, p2, &st->n_vis, sh, nd, s)
+                          : radix_pass<2, 8>(ws, k, p, k2, p2, &st->n_vis, sh, nd, s)) != GS_OK)
+                return r;
+        // after 4 passes the sorted data are back in vis_key / vis_pair
     }
-    // 2. stable sort of the visible pairs by depth key (32 bits)
-    uint32_t *k = ws->vis_key, *v = ws->vis_pair, *k2 = ws->vis_key_alt, *v2 = ws->vis_pair_alt;
-    {
-    StageTimer timer(ws, GS_STAGE_DEPTH_SORT, s);
-    // (blocks grow with the pairs: a tenth of them or so are visible; more
-    // blocks than keys to fill them only lengthen the digit-table scans)
-    const int nd = (int)std::min<int64_t>(nw, std::max<int64_t>(nb, ws->n_pairs / 16384));
-    // four keys a thread once the blocks hold several tiles each (orchard4m,
-    // 3.08 M visible of 24 M pairs: 0.175 -> 0.164 ms), two below (orchard500k,
-    // 148k of 1.5 M: 0.063 ms against 0.065 with four)
-    const bool wide = ws->n_pairs >= (int64_t)8 << 20;
-    for (int sh = 0; sh < 32; sh += 8)
-        if ((r = wide ? radix_pass<4>(ws, k, v, k2, v2, &st->n_vis, sh, nd, s)
-                      : radix_pass<2>(ws, k, v, k2, v2, &st->n_vis, sh, nd, s)) != GS_OK)
-            return r;
-    }
-    // after 4 passes the sorted data are back in vis_key / vis_pair
-    // 3. instance offsets, capacity check, emission in depth order
-    // emit into whichever buffer makes the last tile pass end in inst_tile/inst_val
-    int passes = (ws->tile_bits + 7) / 8;
+    // 3. instance offsets, capacity check, emission in depth order, into
+    //    whichever buffer makes the last tile pass end in inst_tile / inst_val.
+    //    9-bit digits where they save a pass (one up to 511 tiles, two up to
+    //    2^18; 8 submaps in 24 views, 92,160 tiles, 17 bits: 411 -> 355 us), 8-bit
+    //    ones otherwise, which count and rank with less shared memory.
+    const int p8 = (ws->tile_bits + 7) / 8, p9 = (ws->tile_bits + 8) / 9;
+    const bool nine = p9 < p8;
+    const int passes = nine ? p9 : p8;
     uint32_t *tk = (passes & 1) ? ws->inst_tile_alt : ws->inst_tile;
     uint32_t *tv = (passes & 1) ? ws->inst_val_alt : ws->inst_val;
     uint32_t *tk2 = (passes & 1) ? ws->inst_tile : ws->inst_tile_alt;
     uint32_t *tv2 = (passes & 1) ? ws->inst_val : ws->inst_val_alt;
     {
-    StageTimer timer(ws, GS_STAGE_EMIT, s);
-    ++ws->kernel_launches; k_count_instances<<<nw, T, 0, s>>>(v, ws->rect, st, ws->ioff, ws->part, nw);
-    ++ws->kernel_launches; k_scan_parts<<<1, T, 0, s>>>(ws->part, nw, nullptr, st, (uint64_t)ws->inst_cap, 1);
-    ++ws->kernel_launches; k_instance_offsets<<<nw, T, 0, s>>>(st, ws->part, nw, ws->ioff, ws->win_pair,
-                                                                  (uint32_t)(ws->inst_cap / kEmitWindow + 2));
-    ++ws->kernel_launches;
-    k_emit_instances<<<kEmitBlocksPerSM * ws->num_sms, T, 0, s>>>(v, ws->rect, ws->rec, ws->views, ws->n_views,
-                                                                    ws->consts, st, ws->ioff, ws->win_pair, tk, tv);
-    if ((r = check_launch("emit")) != GS_OK) return r;
+        StageTimer timer(ws, GS_STAGE_EMIT, s);
+        if (n_pairs > (uint32_t)kSmallPairs) {
+            ws->kernel_launches += 2;
+            k_count_instances<<<nw, T, 0, s>>>(v, ws->rect, st, ws->ioff, ws->part, cap);
+            k_instance_offsets<<<nw, T, 0, s>>>(st, ws->part, nw, ws->ioff, ws->win_pair, n_win);
+        }
+        ++ws->kernel_launches;
+        k_emit_instances<<<kEmitBlocksPerSM * ws->num_sms, T, 0, s>>>(v, ws->rect, ws->rec, ws->views, ws->n_views,
+                                                                      ws->consts, st, ws->ioff, ws->win_pair, tk, tv,
+                                                                      ws->ranges, n_tiles);
+        if ((r = check_launch("emit")) != GS_OK) return r;
     }
     // 4. stable sort of the instances by tile id
     {
-    StageTimer timer(ws, GS_STAGE_TILE_SORT, s);
-    for (int p = 0; p < passes; ++p)
-        if ((r = radix_pass<8>(ws, tk, tv, tk2, tv2, &st->n_inst, 8 * p, std::min(4 * T, 2 * nb), s)) != GS_OK) return r;
+        StageTimer timer(ws, GS_STAGE_TILE_SORT, s);
+        const int blocks = std::min(4 * T, 2 * nb);
+        for (int p = 0; p < passes; ++p)
+            if ((r = nine ? radix_pass<8, 9>(ws, tk, tv, tk2, tv2, &st->n_inst, 9 * p, blocks, s)
+                          : radix_pass<8, 8>(ws, tk, tv, tk2, tv2, &st->n_inst, 8 * p, blocks, s)) != GS_OK)
+                return r;
     }
-    // 5. ranges
+    // 5. ranges and raster work order
     StageTimer timer(ws, GS_STAGE_RANGES, s);
-    cudaMemsetAsync(ws->ranges, 0, sizeof(uint2) * ws->n_tiles, s);
-    ++ws->kernel_launches;
+    if (passes == 1) {
+        ++ws->kernel_launches;
+        k_ranges_small<<<1, 512, 0, s>>>(ws->digit_tot, st, (int)n_tiles, ws->ranges, ws->tile_order);
+        return check_launch("ranges");
+    }
+    ws->kernel_launches += 3;
     // (eight blocks an SM, every thread resident: 0.054 -> 0.044 ms with the
     // work order on orchard4m's 25.1 M instances, against four)
-    k_ranges<<<ws->num_sms * 8, 256, 0, s>>>(ws->inst_tile, st, (uint32_t)ws->n_tiles, ws->ranges, ws->order_tot);
-    // 6. raster work order
-    ++ws->kernel_launches;
-    k_order_count<<<kOrderBlocks, 256, 0, s>>>(ws->ranges, (int)ws->n_tiles, ws->order_tot, ws->order_base);
-    ++ws->kernel_launches;
-    k_order_place<<<kOrderBlocks, 256, 0, s>>>(ws->ranges, (int)ws->n_tiles, ws->order_tot, ws->order_base,
-                                               ws->tile_order);
+    k_ranges<<<ws->num_sms * 8, 256, 0, s>>>(ws->inst_tile, st, n_tiles, ws->ranges, ws->order_tot);
+    k_order_count<<<kOrderBlocks, 256, 0, s>>>(ws->ranges, (int)n_tiles, ws->order_tot, ws->order_base);
+    k_order_place<<<kOrderBlocks, 256, 0, s>>>(ws->ranges, (int)n_tiles, ws->order_tot, ws->order_base, ws->tile_order);
     return check_launch("ranges");
 }
 
