@@ -16,8 +16,8 @@
 // instructions, T is recovered by division, and with h = gC.c + gD z + gA
 //   dL/dalpha_j = T_j h_j - (sum_{k>j} w_k h_k) / (1 - alpha_j).
 // The 10 image-space gradient components of each Gaussian are summed over the
-// thread's pixels and then over the warp with shuffles before one atomic per
-// component.
+// lane's pixels and then over the warp, through shared memory, before one
+// atomic per two components.
 //
 // In both passes a tile is divided into quadrants of 8x8 pixels, two a lane,
 // and a warp holds one, two or four quadrants.  Of each entry it works only the
