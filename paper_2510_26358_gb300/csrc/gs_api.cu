@@ -139,7 +139,7 @@ void gs_workspace_destroy(gs_workspace *ws) {
                     ws->inst_tile, ws->inst_val, ws->inst_tile_alt, ws->inst_val_alt, ws->ranges,
                     ws->tile_order, ws->order_tot, ws->order_base,
                     ws->last, ws->tfin, ws->vstat, ws->hist, ws->part, ws->digit_tot, ws->pose_part, ws->red_part, ws->ssim_d, ws->ssim_part,
-                    ws->ssim_tile, ws->st};
+                    ws->ssim_tile, ws->pair_state, ws->st};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     for (cudaEvent_t e : ws->ev)
@@ -271,6 +271,7 @@ gs_status gs_workspace_create(const gs_camera *cams, int32_t n_views, const int6
     GS_ALLOC(ws->rect, P);
     GS_ALLOC(ws->g2d, P * kGrad);
     GS_ALLOC(ws->gdir, P);
+    GS_ALLOC(ws->pair_state, P);
     GS_ALLOC(ws->vis_key, P);
     GS_ALLOC(ws->vis_pair, P);
     GS_ALLOC(ws->vis_key_alt, P);

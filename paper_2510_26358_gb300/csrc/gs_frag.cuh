@@ -14,6 +14,9 @@ namespace gs {
 // ---------------------------------------------------------------------------
 
 constexpr uint32_t kInvalidKey = 0xFFFFFFFFu;  // pair depth key of an invisible pair
+// what a (view, Gaussian) pair's state byte says: not visible, visible, and
+// visible with image-space gradients added by the raster backward
+constexpr uint8_t kPairUnseen = 0, kPairVisible = 1, kPairTouched = 2;
 constexpr int kRecF4 = 3;                     // float4 per projected record
 constexpr int kGrad = 10;                     // floats per image-space gradient record
 // image-space gradient components (same order as the oracle's)

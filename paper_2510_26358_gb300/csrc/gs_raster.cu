@@ -107,6 +107,7 @@ struct RasterArgs {
     const float *dL_drgb, *dL_ddepth, *dL_dalpha;
     const float *dL_dmean, *dL_dvar;  // VAR variant
     float *g2d;
+    uint8_t *state;  // pair states: touched pairs are marked
 };
 
 // A tile is divided into quadrants of 8x8 pixels, two a lane: lane l holds
@@ -602,10 +603,32 @@ __device__ __forceinline__ void red_add2(float *p, float a, float b) {
     asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" ::"l"(p), "f"(a), "f"(b) : "memory");
 }
 
-// Adds the n pending entries' sums to their pairs' gradient rows; byte k of
-// `which` is the staged index of slot k.
+// Component pair c of an entry's raw sums (u, v), (qa, qb), (qc, ln o), (r, g) or
+// (b, z) turned into gradients and added to its pair's row.  The raw sums are
+// negated (dpw and the weights are carried negated); dL/dQ = -1/2 sum gpw d
+// d^T; dpw/du = (Q d)_x = l11 t1 / s^2, dpw/dv = (l12 t1 + l22 t2) / s^2 with 1/s^2
+// = 2 ln 2.
+__device__ __forceinline__ void add_gradients(const BwdEntry &e, int c, float x, float y, float *g2d, uint8_t *state) {
+    const uint32_t pair = __float_as_uint(e.z.w);
+    if (c == 0) {
+        state[pair] = kPairTouched;
+        y = -kTwoLn2 * __fmaf_rn(e.l.x, x, e.l.z * y);
+        x = -kTwoLn2 * (e.u.y * x);
+    } else {
+        x *= c <= 2 ? 0.5f : -1.f;
+        y = c == 1 ? y : -y;
+    }
+    red_add2(g2d + (size_t)pair * kGrad + 2 * c, x, y);
+}
+
+// Sums the n pending entries' rows; byte k of `which` is the staged index of
+// slot k.  Where one warp works the tile they go to the pairs' gradient rows;
+// else to the warp's part of tile_sums, from which the CTA adds them once a
+// batch (one atomic a tile and component instead of one a warp, in a fixed
+// order inside the tile).
+template <bool ONE_WARP>
 __device__ __forceinline__ void flush_sums(const float *sum, const BwdEntry *sE, int n, uint32_t which, int lane,
-                                           float *g2d) {
+                                           float *tile_sums, float *g2d, uint8_t *state) {
     __syncwarp();
     // lane = 8 f + 2 slot + half: column f (components 4f .. 4f + 3) of a slot's rows 16 half .. 16 half + 15
     const int f = lane >> 3, turn = lane & 7, slot = turn >> 1, half = lane & 1;
@@ -629,21 +652,11 @@ __device__ __forceinline__ void flush_sums(const float *sum, const BwdEntry *sE,
     t.y += __shfl_xor_sync(0xffffffffu, t.y, 1);
     t.z += __shfl_xor_sync(0xffffffffu, t.z, 1);
     t.w += __shfl_xor_sync(0xffffffffu, t.w, 1);
-    if (active) {
-        // the raw sums are negated (dpw and the weights are carried negated);
-        // dL/dQ = -1/2 sum gpw d d^T; dpw/du = (Q d)_x = l11 t1 / s^2,
-        // dpw/dv = (l12 t1 + l22 t2) / s^2 with 1/s^2 = 2 ln 2
-        const BwdEntry &e = sE[which >> (8 * slot) & 255u];
-        float *gp = g2d + (size_t)__float_as_uint(e.z.w) * kGrad + 4 * f;
-        if (f == 0) {
-            if (half == 0) red_add2(gp, -kTwoLn2 * (e.u.y * t.x), -kTwoLn2 * __fmaf_rn(e.l.x, t.x, e.l.z * t.y));
-            else red_add2(gp + 2, 0.5f * t.z, t.w);
-        } else if (f == 1) {
-            if (half == 0) red_add2(gp, 0.5f * t.x, -t.y);
-            else red_add2(gp + 2, -t.z, -t.w);
-        } else if (half == 0) {
-            red_add2(gp, -t.x, -t.y);
-        }
+    if (active && 2 * f + half < kGrad / 2) {
+        const int j = which >> (8 * slot) & 255u, c = 2 * f + half;
+        const float x = half ? t.z : t.x, y = half ? t.w : t.y;
+        if (ONE_WARP) add_gradients(sE[j], c, x, y, g2d, state);
+        else *reinterpret_cast<float2 *>(tile_sums + j * kGrad + 2 * c) = make_float2(x, y);
     }
     __syncwarp();
 }
@@ -659,7 +672,8 @@ __device__ __forceinline__ void flush_sums(const float *sum, const BwdEntry *sE,
 // both passes take the same decisions bit for bit.
 // (Against one warp a tile, a thread a column of eight pixels and a butterfly
 // of shuffles an entry: 4M orchard, six 1920x1200 views, 1841 -> 1606 us; three
-// 1280x720 views of 500k 322 -> 281; 320x240, 10k 213 -> 99.)
+// 1280x720 views of 500k 322 -> 281; 320x240, 10k 213 -> 99; with several warps'
+// sums added once a tile 1549, 273 and 86.)
 template <int TW, int TH, int Q, bool VAR>
 __global__ void __launch_bounds__(Share<TW, TH, Q>::NT, bwd_blocks(Share<TW, TH, Q>::NW, Q, VAR))
     k_raster_bwd(RasterArgs A) {
@@ -669,6 +683,10 @@ __global__ void __launch_bounds__(Share<TW, TH, Q>::NT, bwd_blocks(Share<TW, TH,
     BwdEntry *sE = reinterpret_cast<BwdEntry *>(smem);
     uint32_t *sM = reinterpret_cast<uint32_t *>(sE + A.depth);
     float *sums = reinterpret_cast<float *>(sM + A.depth) + (NW > 1 ? (threadIdx.x >> 5) * (kSumBytes / 4) : 0);
+    // several warps: their sums of a batch, [warp][entry][component], and the entries each has worked
+    float *all_sums = reinterpret_cast<float *>(sM + A.depth) + NW * (kSumBytes / 4);
+    float *tile_sums = all_sums + (NW > 1 ? (threadIdx.x >> 5) * A.depth * kGrad : 0);
+    __shared__ uint32_t s_worked[NW > 1 ? NW : 1][kBwdDepth / 32];
     __shared__ int s_tile;
     __shared__ uint32_t s_max[NW];
     const int tid = threadIdx.x, lane = tid & 31, wid = NW > 1 ? tid >> 5 : 0;
@@ -765,6 +783,8 @@ __global__ void __launch_bounds__(Share<TW, TH, Q>::NT, bwd_blocks(Share<TW, TH,
             __syncthreads();
             uint32_t which = 0;
             int pending = 0;
+            if (NW > 1 && lane < kBwdDepth / 32) s_worked[wid][lane] = 0u;
+            __syncwarp();
             for (int jb = (nb - 1) & ~31; jb >= 0; jb -= 32) {
                 const uint32_t rel0 = (uint32_t)(lo + jb - rg.x);
                 if (rel0 >= wmax) continue;  // no pixel of this warp reached these entries
@@ -778,6 +798,7 @@ __global__ void __launch_bounds__(Share<TW, TH, Q>::NT, bwd_blocks(Share<TW, TH,
                     todo |= E[q];
                     all &= E[q];
                 }
+                if (NW > 1 && lane == 0) s_worked[wid][jb / 32] = todo;
                 while (todo) {
                     const int j = 31 - __clz(todo);
                     todo ^= 1u << j;
@@ -900,14 +921,34 @@ __global__ void __launch_bounds__(Share<TW, TH, Q>::NT, bwd_blocks(Share<TW, TH,
                         make_float2(f2_lo(sB_) + f2_hi(sB_), f2_lo(sZ) + f2_hi(sZ));
                     which = which << 8 | (uint32_t)(jb + j);
                     if (++pending == kSumSlots) {
-                        flush_sums(sums, sE, kSumSlots, __byte_perm(which, 0, 0x0123), lane, A.g2d);
+                        flush_sums<NW == 1>(sums, sE, kSumSlots, __byte_perm(which, 0, 0x0123), lane, tile_sums, A.g2d,
+                                            A.state);
                         pending = 0;
                     }
                 }
             }
             // (the pending entries' staged records go with this batch)
             if (pending)
-                flush_sums(sums, sE, pending, __byte_perm(which << 8 * (kSumSlots - pending), 0, 0x0123), lane, A.g2d);
+                flush_sums<NW == 1>(sums, sE, pending, __byte_perm(which << 8 * (kSumSlots - pending), 0, 0x0123), lane,
+                                    tile_sums, A.g2d, A.state);
+            if constexpr (NW > 1) {
+                __syncthreads();
+                for (int i = tid; i < nb * (kGrad / 2); i += NT) {
+                    const int j = i / (kGrad / 2), c = i - j * (kGrad / 2);
+                    float2 t = make_float2(0.f, 0.f);
+                    bool any = false;
+#pragma unroll
+                    for (int w = 0; w < NW; ++w)
+                        if (s_worked[w][j >> 5] >> (j & 31) & 1u) {
+                            const float2 x =
+                                *reinterpret_cast<const float2 *>(all_sums + (w * A.depth + j) * kGrad + 2 * c);
+                            t.x += x.x;
+                            t.y += x.y;
+                            any = true;
+                        }
+                    if (any) add_gradients(sE[j], c, t.x, t.y, A.g2d, A.state);
+                }
+            }
         }
     }
 }
@@ -954,7 +995,9 @@ template <int TW, int TH, int Q, bool VAR>
 RasterKernel bwd_variant(int depth) {
     const int d = std::min(depth, kBwdDepth);
     using S = Share<TW, TH, Q>;
-    return {k_raster_bwd<TW, TH, Q, VAR>, S::NT, d, (size_t)d * (sizeof(BwdEntry) + sizeof(uint32_t)) + S::NW * kSumBytes};
+    const size_t batch = S::NW > 1 ? (size_t)S::NW * d * kGrad * sizeof(float) : 0;
+    return {k_raster_bwd<TW, TH, Q, VAR>, S::NT, d,
+            (size_t)d * (sizeof(BwdEntry) + sizeof(uint32_t)) + S::NW * kSumBytes + batch};
 }
 template <int TW, int TH>
 RasterKernel bwd_kernel(const gs_workspace *ws, bool var) {
@@ -1050,6 +1093,7 @@ gs_status launch_raster_bwd(gs_workspace *ws, const float *dL_drgb, const float 
         A.dL_dvar = dL_dvar;
     }
     A.g2d = ws->g2d;
+    A.state = ws->pair_state;
     // the projection clears the rows; a second backward of the same
     // projection clears them itself
     if (!ws->g2d_clear) {
