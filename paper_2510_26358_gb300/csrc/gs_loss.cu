@@ -24,6 +24,7 @@
 #include "gs_scan.cuh"
 
 #include <algorithm>
+#include <cmath>
 
 namespace gs {
 namespace {
@@ -77,6 +78,7 @@ struct DepthArgs {
     const ViewInfo *views;
     int32_t n_views, mode;
     float near_z, sigma_L, sigma_U, lambda;
+    double log_sigma_L;
     const float *depth, *alpha, *lidar;
     const float *var;  // mode 2 (`depth` holds the mean)
     int64_t n_pts;
@@ -92,16 +94,18 @@ struct DepthArgs {
 struct VarTerm {
     double kl, dmu, dvar;
 };
-__device__ __forceinline__ VarTerm var_term(double mu, double var, double z, double sl, double su) {
+// (one division and one logarithm in double: at two operations a clock an SM
+// they are what the 60k returns of a keyframe wait for; log sigma_L comes from
+// the host)
+__device__ __forceinline__ VarTerm var_term(double mu, double var, double z, double sl, double log_sl, double su) {
     VarTerm t;
     const bool clamped = var < 0.0;
     const double v = (clamped ? 0.0 : var) + su * su;
-    const double e = mu - z;
-    t.kl = 0.5 * log(v) - log(sl) + (sl * sl + e * e) / (2.0 * v) - 0.5;
-    const double dmu = e / v;
-    const double dv = clamped ? 0.0 : 0.5 / v - (sl * sl + e * e) / (2.0 * v * v);
-    t.dmu = dmu;
-    t.dvar = dv;
+    const double e = mu - z, iv = 1.0 / v;
+    const double h = 0.5 * (sl * sl + e * e) * iv;
+    t.kl = 0.5 * log(v) - log_sl + h - 0.5;
+    t.dmu = e * iv;
+    t.dvar = clamped ? 0.0 : (0.5 - h) * iv;
     return t;
 }
 
@@ -167,7 +171,7 @@ __global__ void __launch_bounds__(LT) k_depth_partial(DepthArgs A) {
             if (A.mode == 0) {
                 sf.add(fabsf(d));
             } else if (A.mode == 2) {
-                s += var_term(G.dep[u], G.var[u], G.z[u], A.sigma_L, A.sigma_U).kl;
+                s += var_term(G.dep[u], G.var[u], G.z[u], A.sigma_L, A.log_sigma_L, A.sigma_U).kl;
             } else {
                 // the KL's point-independent part (its log and constants) is
                 // added once per valid point at the end: double logs and
@@ -223,7 +227,7 @@ __global__ void __launch_bounds__(LT) k_depth_grad(DepthArgs A) {
             const int64_t pix = G.pix[u];
             if (pix < 0) continue;
             if (A.mode == 2) {
-                const VarTerm t = var_term(G.dep[u], G.var[u], G.z[u], A.sigma_L, A.sigma_U);
+                const VarTerm t = var_term(G.dep[u], G.var[u], G.z[u], A.sigma_L, A.log_sigma_L, A.sigma_U);
                 const double k = scale;
                 if (A.grad) atomicAdd(A.grad + pix, (float)(k * t.dmu));
                 if (A.grad_var) atomicAdd(A.grad_var + pix, (float)(k * t.dvar));
@@ -377,6 +381,7 @@ gs_status launch_depth_loss(gs_workspace *ws, int mode, const float *depth, cons
     A.near_z = ws->cfg.near_z;
     A.sigma_L = ws->cfg.sigma_L;
     A.sigma_U = ws->cfg.sigma_U;
+    A.log_sigma_L = std::log((double)ws->cfg.sigma_L);
     A.lambda = ws->cfg.lambda_L;
     A.depth = depth;
     A.alpha = alpha;

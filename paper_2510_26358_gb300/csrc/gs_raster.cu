@@ -78,14 +78,31 @@ constexpr int fwd_blocks(int warps, int q, bool var) {
 
 constexpr int bwd_blocks(int warps, int q, bool var) { return (q == 1 ? 24 : 16) / warps; }
 
-// One step of the weighted Welford update (the VAR variants).
-__device__ __forceinline__ void welford(float w, float z, bool first, float &W, float &zc, float &m, float &M2) {
-    if (first) zc = z;
+// One step of the weighted Welford update (the VAR variants), for one pixel and
+// for a packed pair; both round alike.  The first fragment (W == 0: every
+// weight is positive) sets zc.  The pair takes its weights and depths negated
+// (as the forward stages them) and keeps zc negated; a pixel with weight 0
+// keeps its values (before its first fragment zc changes, m and M2 stay 0).
+__device__ __forceinline__ void welford(float w, float z, float &W, float &zc, float &m, float &M2) {
+    if (W == 0.f) zc = z;
     W = __fadd_rn(W, w);
     const float y = z - zc;
     const float d = y - m;
-    m = __fmaf_rn(d, __fdividef(w, W), m);
+    m = __fmaf_rn(d, __fmul_rn(w, rcp_approx(fmaxf(W, 1e-30f))), m);
     M2 = __fmaf_rn(__fmul_rn(w, d), y - m, M2);
+}
+__device__ __forceinline__ void welford2(f2 nw, f2 nz, f2 &W, f2 &nzc, f2 &m, f2 &M2) {
+    float w0, w1, c0, c1;
+    f2_unpack(W, w0, w1);
+    f2_unpack(nzc, c0, c1);
+    const float z = f2_lo(nz);
+    nzc = f2_pack(w0 == 0.f ? z : c0, w1 == 0.f ? z : c1);
+    W = f2_sub(W, nw);
+    f2_unpack(W, w0, w1);
+    const f2 r = f2_pack(rcp_approx(fmaxf(w0, 1e-30f)), rcp_approx(fmaxf(w1, 1e-30f)));
+    const f2 y = f2_sub(nzc, nz), nd = f2_sub(m, y);
+    m = f2_fma(nd, f2_mul(nw, r), m);
+    M2 = f2_fma(f2_mul(nw, nd), f2_sub(y, m), M2);
 }
 
 struct RasterArgs {
@@ -230,16 +247,16 @@ __global__ void __launch_bounds__(Share<TW, TH, Q>::NT, fwd_blocks(Share<TW, TH,
         f2 T[Q], Cr[Q], Cg[Q], Cb[Q], D[Q];
         float thr[Q][2];  // -log2 alpha_min while the pixel lives, then -inf
         uint32_t cnt[Q][2];
-        float Wsum[Q][2], zc[Q][2], mr[Q][2], M2[Q][2];
+        f2 Wsum[Q], nzc[Q], mr[Q], M2[Q];  // nzc = -zc
         uint32_t live = 0;  // bit q: quadrant q has a live pixel
 #pragma unroll
         for (int q = 0; q < Q; ++q) {
             T[q] = f2_bcast(1.f);
             Cr[q] = Cg[q] = Cb[q] = D[q] = f2_bcast(0.f);
+            Wsum[q] = nzc[q] = mr[q] = M2[q] = f2_bcast(0.f);
             const int px = px0 + 8 * (q % QX), py = py0 + 8 * (q / QX);
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
-                Wsum[q][h] = zc[q][h] = mr[q][h] = M2[q][h] = 0.f;
                 cnt[q][h] = 0;
                 thr[q][h] = px < vi.W && py + 4 * h < vi.H ? -l2amin : -INFINITY;
             }
@@ -324,15 +341,7 @@ __global__ void __launch_bounds__(Share<TW, TH, Q>::NT, fwd_blocks(Share<TW, TH,
                             Cg[q] = f2_fma(nw, gb.a, Cg[q]);
                             Cb[q] = f2_fma(nw, gb.b, Cb[q]);
                             D[q] = f2_fma(nw, z.a, D[q]);
-                            if (VAR) {
-                                float w[2];
-                                f2_unpack(nw, w[0], w[1]);
-#pragma unroll
-                                for (int h = 0; h < 2; ++h)
-                                    if (in[q][h])
-                                        welford(-w[h], -f2_lo(z.a), cnt[q][h] == 0, Wsum[q][h], zc[q][h], mr[q][h],
-                                                M2[q][h]);
-                            }
+                            if (VAR) welford2(nw, z.a, Wsum[q], nzc[q], mr[q], M2[q]);
 #pragma unroll
                             for (int h = 0; h < 2; ++h)
                                 if (in[q][h]) cnt[q][h] = j1;
@@ -375,6 +384,11 @@ __global__ void __launch_bounds__(Share<TW, TH, Q>::NT, fwd_blocks(Share<TW, TH,
                             f2_unpack(Cg[q], cg[0], cg[1]);
                             f2_unpack(Cb[q], cb[0], cb[1]);
                             f2_unpack(D[q], d[0], d[1]);
+                            float W[2], zc[2], m[2], v[2];
+                            f2_unpack(Wsum[q], W[0], W[1]);
+                            f2_unpack(nzc[q], zc[0], zc[1]);
+                            f2_unpack(mr[q], m[0], m[1]);
+                            f2_unpack(M2[q], v[0], v[1]);
 #pragma unroll
                             for (int h = 0; h < 2; ++h) {
                                 // (an exponent that is not a number is not below the threshold)
@@ -390,7 +404,11 @@ __global__ void __launch_bounds__(Share<TW, TH, Q>::NT, fwd_blocks(Share<TW, TH,
                                 cg[h] = __fmaf_rn(w, -cy, cg[h]);
                                 cb[h] = __fmaf_rn(w, -cz, cb[h]);
                                 d[h] = __fmaf_rn(w, -cw, d[h]);
-                                if (VAR) welford(w, -cw, cnt[q][h] == 0, Wsum[q][h], zc[q][h], mr[q][h], M2[q][h]);
+                                if (VAR) {
+                                    zc[h] = -zc[h];
+                                    welford(w, -cw, W[h], zc[h], m[h], v[h]);
+                                    zc[h] = -zc[h];
+                                }
                                 t[h] = tn;
                                 cnt[q][h] = j1;
                             }
@@ -399,6 +417,10 @@ __global__ void __launch_bounds__(Share<TW, TH, Q>::NT, fwd_blocks(Share<TW, TH,
                             Cg[q] = f2_pack(cg[0], cg[1]);
                             Cb[q] = f2_pack(cb[0], cb[1]);
                             D[q] = f2_pack(d[0], d[1]);
+                            Wsum[q] = f2_pack(W[0], W[1]);
+                            nzc[q] = f2_pack(zc[0], zc[1]);
+                            mr[q] = f2_pack(m[0], m[1]);
+                            M2[q] = f2_pack(v[0], v[1]);
                         }
                     }
                     // quadrants whose pixels have all ended leave the walk
@@ -430,6 +452,11 @@ __global__ void __launch_bounds__(Share<TW, TH, Q>::NT, fwd_blocks(Share<TW, TH,
             f2_unpack(Cg[q], cg[0], cg[1]);
             f2_unpack(Cb[q], cb[0], cb[1]);
             f2_unpack(D[q], d[0], d[1]);
+            float W[2], zc[2], m[2], v[2];
+            f2_unpack(Wsum[q], W[0], W[1]);
+            f2_unpack(nzc[q], zc[0], zc[1]);
+            f2_unpack(mr[q], m[0], m[1]);
+            f2_unpack(M2[q], v[0], v[1]);
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 const int py = py0 + 8 * (q / QX) + 4 * h;
@@ -443,13 +470,14 @@ __global__ void __launch_bounds__(Share<TW, TH, Q>::NT, fwd_blocks(Share<TW, TH,
                 // 1 - T loses the relative precision of a small alpha (T near 1);
                 // the variance variant has the direct sum of the weights at hand,
                 // which keeps it, as the normalised depth D / alpha needs
-                A.alpha_out[pix] = VAR ? Wsum[q][h] : 1.f - t[h];
+                A.alpha_out[pix] = VAR ? W[h] : 1.f - t[h];
                 A.last[pix] = cnt[q][h];
                 A.tfin[pix] = t[h];
                 if (VAR) {
-                    const float mean = zc[q][h] + mr[q][h];
-                    const float iw = Wsum[q][h] > 0.f ? 1.f / Wsum[q][h] : 0.f;
-                    const float var = M2[q][h] * iw;
+                    // (zc stands negated; 0 where nothing blended)
+                    const float mean = W[h] > 0.f ? m[h] - zc[h] : 0.f;
+                    const float iw = W[h] > 0.f ? 1.f / W[h] : 0.f;
+                    const float var = v[h] * iw;
                     A.mean_out[pix] = mean;
                     A.var_out[pix] = var;
                     A.vstat[pix] = make_float4(mean, var, iw, 0.f);
@@ -542,7 +570,7 @@ __global__ void __launch_bounds__(TW * TH / PF, VAR ? 640 / (TW * TH / PF) : 0) 
                     Cg[i] = __fmaf_rn(wgt, c.y, Cg[i]);
                     Cb[i] = __fmaf_rn(wgt, c.z, Cb[i]);
                     D[i] = __fmaf_rn(wgt, c.w, D[i]);
-                    if (VAR) welford(wgt, c.w, cnt[i] == 0, Wsum[i], zc[i], mr[i], M2[i]);
+                    if (VAR) welford(wgt, c.w, Wsum[i], zc[i], mr[i], M2[i]);
                     T[i] = Tn;
                     cnt[i] = b0 + j - rg.x + 1;
                 }
