@@ -69,7 +69,8 @@ typedef struct {
 /* Renderer constants (the paper leaves them to standard 3DGS). */
 typedef struct {
     int32_t tile_w, tile_h; /* tile size in pixels: 8x8, 16x16, 16x32 or 32x16 */
-    int32_t batch_depth;    /* Gaussians staged per shared-memory batch: 32..256, multiple of 32 */
+    int32_t batch_depth;    /* Gaussians staged per shared-memory batch, at most: 32..256, multiple of 32 (the
+                               rasterisers stage fewer where that is faster; no result depends on it) */
     int32_t depth_mode;     /* gs_depth_loss: 0 = L1 |D - z|, 1 = KL of Eq. (7) with fixed sigma_U */
     float near_z;           /* pairs with view-space z <= near_z are culled (0.2 m) */
     float dilation;         /* added to the diagonal of Sigma' (0.3 px^2) */

@@ -52,8 +52,15 @@ namespace {
 constexpr float kQuadRelPad = 1e-3f, kQuadAbsPad = 1e-2f;
 
 // Entries staged at a time, at most (the configuration's batch depth below
-// it): with 64 the staged entries of 20 one-warp CTAs fit an SM.
-constexpr int kFwdDepth = 64, kBwdDepth = 64;
+// it): with 64 the staged entries of 20 one-warp CTAs fit an SM.  The backward of
+// whole tiles a warp: 32 against 64, 4M orchard 1570 -> 1558 us, 500k 277 -> 271.
+// The one in pairs of entries takes all of kPairsDepth where few tiles leave the
+// SMs idle anyway, and less where more CTAs an SM are worth more (128, 64, 32
+// entries, us): 300 tiles of 16x16 54, 68, 71; 3600 127, 118, 120; 8x8: 4270 380, 409,
+// 410; 9900 461, 497, 524; 43,200 584, 472, 439.
+constexpr int kFwdDepth = 64, kPairsDepth = 128;
+template <int Q>
+constexpr int kBwdDepth = Q == 4 ? 32 : 64;
 
 // How many quadrants a warp takes, by the number of 16x16 tiles (or as many
 // pixels).  Whole tiles share the most work between quadrants but make the
@@ -62,11 +69,12 @@ constexpr int kFwdDepth = 64, kBwdDepth = 64;
 // two, four quadrants a warp, us).  Forward, the whole step: 300 tiles (320x240,
 // box of 10k) 288, 298, -; 1200 (orchard of 200k, as below) 247, 258, -; 2400
 // 318, 319, -; 3600 249, 247, -; the kernel: 7200 87, 64, 75; 24,480 (1M) -, 391,
-// 406; 54,000 (4M) -, 971, 936.  Backward, the kernel: 300 tiles 93, 111, 186;
-// 2400 95, 102, 143; 3600 59, 59, 86; 7200 171, 130, 124.  With the variance (one,
-// two; more do not fit the registers) forward, 2400 tiles 73, 97; 7200 139, 107;
-// backward 104, 108; 186, 153.
+// 406; 54,000 (4M) -, 971, 936.  Backward, the kernel (one entry at a time): 2400
+// tiles 89, -, 138; 3600 50, -, 85; 7200 175, 130, 119; 10,800 467, 349, 274.  With
+// the variance (one, two; more do not fit the registers) forward, 2400 tiles 73,
+// 97; 7200 139, 107; backward 104, 108; 192, 147.
 constexpr int kCoarseTiles = 152 * 24;     // backward, and forward with the variance
+constexpr int kDeepTiles = 152 * 3;        // backward in pairs of entries, 16x16 tiles and larger
 constexpr int kFwdHalfTiles = 152 * 16, kFwdWholeTiles = 152 * 256;  // forward
 
 // Resident warps an SM that each variant's registers are bounded for, as CTAs
@@ -76,7 +84,7 @@ constexpr int fwd_blocks(int warps, int q, bool var) {
     return (var ? (q == 4 ? 16 : 20) : (q == 4 ? 20 : q == 2 ? 28 : 40)) / warps;
 }
 
-constexpr int bwd_blocks(int warps, int q, bool var) { return (q == 1 ? 24 : 16) / warps; }
+constexpr int bwd_blocks(int warps) { return 16 / warps; }
 
 // One step of the weighted Welford update (the VAR variants), for one pixel and
 // for a packed pair; both round alike.  The first fragment (W == 0: every
@@ -606,6 +614,13 @@ __global__ void __launch_bounds__(TW * TH / PF, VAR ? 640 / (TW * TH / PF) : 0) 
     }
 }
 
+__device__ __forceinline__ void cp_async16(void *dst, const void *src) {
+    const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 // One staged list entry of the backward (see FwdEntry).
 struct BwdEntry {
     float4 u;    // U, l11, k1, hx
@@ -702,10 +717,9 @@ __device__ __forceinline__ void flush_sums(const float *sum, const BwdEntry *sE,
 // both passes take the same decisions bit for bit.
 // (Against one warp a tile, a thread a column of eight pixels and a butterfly
 // of shuffles an entry: 4M orchard, six 1920x1200 views, 1841 -> 1606 us; three
-// 1280x720 views of 500k 322 -> 281; 320x240, 10k 213 -> 99; with several warps'
-// sums added once a tile 1549, 273 and 86.)
+// 1280x720 views of 500k 322 -> 281; with 32 entries staged 1558 and 271.)
 template <int TW, int TH, int Q, bool VAR>
-__global__ void __launch_bounds__(Share<TW, TH, Q>::NT, bwd_blocks(Share<TW, TH, Q>::NW, Q, VAR))
+__global__ void __launch_bounds__(Share<TW, TH, Q>::NT, bwd_blocks(Share<TW, TH, Q>::NW))
     k_raster_bwd(RasterArgs A) {
     using S = Share<TW, TH, Q>;
     constexpr int QX = S::QX, QY = S::QY, NW = S::NW, NT = S::NT;
@@ -716,7 +730,7 @@ __global__ void __launch_bounds__(Share<TW, TH, Q>::NT, bwd_blocks(Share<TW, TH,
     // several warps: their sums of a batch, [warp][entry][component], and the entries each has worked
     float *all_sums = reinterpret_cast<float *>(sM + A.depth) + NW * (kSumBytes / 4);
     float *tile_sums = all_sums + (NW > 1 ? (threadIdx.x >> 5) * A.depth * kGrad : 0);
-    __shared__ uint32_t s_worked[NW > 1 ? NW : 1][kBwdDepth / 32];
+    __shared__ uint32_t s_worked[NW > 1 ? NW : 1][kBwdDepth<Q> / 32];
     __shared__ int s_tile;
     __shared__ uint32_t s_max[NW];
     const int tid = threadIdx.x, lane = tid & 31, wid = NW > 1 ? tid >> 5 : 0;
@@ -813,7 +827,7 @@ __global__ void __launch_bounds__(Share<TW, TH, Q>::NT, bwd_blocks(Share<TW, TH,
             __syncthreads();
             uint32_t which = 0;
             int pending = 0;
-            if (NW > 1 && lane < kBwdDepth / 32) s_worked[wid][lane] = 0u;
+            if (NW > 1 && lane < kBwdDepth<Q> / 32) s_worked[wid][lane] = 0u;
             __syncwarp();
             for (int jb = (nb - 1) & ~31; jb >= 0; jb -= 32) {
                 const uint32_t rel0 = (uint32_t)(lo + jb - rg.x);
@@ -889,7 +903,7 @@ __global__ void __launch_bounds__(Share<TW, TH, Q>::NT, bwd_blocks(Share<TW, TH,
                         sB_ = f2_fma(nwgt, gB[q], sB_);
                         sZ = f2_fma(nwgt, gz, sZ);
                     };
-                    if (Q > 1 && (all & ~exact) >> j & 1u) {
+                    if ((all & ~exact) >> j & 1u) {
                         // every quadrant, interleaved (1680 -> 1606 us, 4M orchard)
 #pragma unroll
                         for (int q = 0; q < Q; ++q) quad(q, false);
@@ -983,6 +997,272 @@ __global__ void __launch_bounds__(Share<TW, TH, Q>::NT, bwd_blocks(Share<TW, TH,
     }
 }
 
+// The backward with one quadrant a warp, for few tiles (below kCoarseTiles) and
+// for 8x8 ones: a warp's walk along its list is then a chain that little
+// else on the SM hides.  Two entries are worked together (only T and the suffix
+// sum go from one to the next), and the next batch's records are copied in while
+// this one is worked, their pair ids read a batch earlier still.  The
+// arithmetic is k_raster_bwd's with the clamp's two selects always in, which
+// change nothing where alpha stays below its maximum.  Measured against one
+// entry at a time with loads at the head of a batch of 64: 300 tiles of 16x16
+// (box of 10k) 83 -> 55 us; 3600 (orchard of 300k, variance) 129 -> 116; 8x8 tiles:
+// 4270 with long lists (orchard of 1.3M, 481x280) 517 -> 394, 43,200 (500k) 458 ->
+// 448.
+template <int TW, int TH, bool VAR>
+__global__ void __launch_bounds__(Share<TW, TH, 1>::NT, bwd_blocks(Share<TW, TH, 1>::NW))
+    k_raster_bwd_pairs(RasterArgs A) {
+    using S = Share<TW, TH, 1>;
+    constexpr int NW = S::NW, NT = S::NT;
+    constexpr int PT = (kPairsDepth + NT - 1) / NT;  // staged entries a thread
+    extern __shared__ float4 smem[];
+    BwdEntry *sE = reinterpret_cast<BwdEntry *>(smem);
+    float4 *sR = reinterpret_cast<float4 *>(sE + A.depth);  // records copied ahead
+    uint32_t *sM = reinterpret_cast<uint32_t *>(sR + 3 * A.depth);
+    const int tid = threadIdx.x, lane = tid & 31, wid = NW > 1 ? tid >> 5 : 0;
+    float *sums = reinterpret_cast<float *>(sM + A.depth) + wid * (kSumBytes / 4);
+    float *all_sums = reinterpret_cast<float *>(sM + A.depth) + NW * (kSumBytes / 4);
+    float *tile_sums = all_sums + wid * A.depth * kGrad;
+    __shared__ uint32_t s_worked[NW][kPairsDepth / 32];
+    __shared__ int s_tile;
+    __shared__ uint32_t s_max[NW];
+    const float amax = A.c.alpha_max, nl2amin = -A.c.log2_alpha_min;
+    const f2 ONE = f2_bcast(1.f), ZERO = f2_bcast(0.f);
+    for (;;) {
+        __syncthreads();
+        if (tid == 0) s_tile = next_tile(A);
+        __syncthreads();
+        const int tile = s_tile;
+        if (tile < 0) break;
+        const int v = view_of_tile(A.views, A.n_views, tile);
+        const ViewInfo vi = A.views[v];
+        const int lt = tile - vi.tile_off;
+        const int tx0 = (lt % vi.ntx) * TW, ty0 = (lt / vi.ntx) * TH;
+        const int px = tx0 + S::wx(wid) + (lane & 7), py0 = ty0 + S::wy(wid) + (lane >> 3);
+        const uint2 rg = A.ranges[tile];
+        const int64_t hw = (int64_t)vi.W * vi.H;
+        const float *grgb = A.dL_drgb + 3 * (int64_t)vi.pix_off;
+        uint32_t cnt[2];
+        float t_[2], r_[2], g_[2], b_[2], d_[2], a_[2], z_[2], ma_[2], mb_[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int py = py0 + 4 * h;
+            cnt[h] = 0;
+            t_[h] = 1.f;
+            r_[h] = g_[h] = b_[h] = d_[h] = a_[h] = z_[h] = ma_[h] = mb_[h] = 0.f;
+            if (px < vi.W && py < vi.H) {
+                const int64_t pl = (int64_t)py * vi.W + px;
+                const int64_t pix = vi.pix_off + pl;
+                cnt[h] = A.last[pix];
+                t_[h] = A.tfin[pix];
+                r_[h] = grgb[pl];
+                g_[h] = grgb[hw + pl];
+                b_[h] = grgb[2 * hw + pl];
+                d_[h] = A.dL_ddepth ? A.dL_ddepth[pix] : 0.f;
+                a_[h] = A.dL_dalpha ? A.dL_dalpha[pix] : 0.f;
+                if (VAR) {
+                    const float4 vs = A.vstat[pix];
+                    z_[h] = vs.x;
+                    ma_[h] = A.dL_dmean ? A.dL_dmean[pix] * vs.z : 0.f;
+                    mb_[h] = A.dL_dvar ? A.dL_dvar[pix] * vs.z : 0.f;
+                    a_[h] = __fmaf_rn(-mb_[h], vs.y, a_[h]);  // the -b var part of every h
+                }
+            }
+        }
+        const uint32_t wmax = __reduce_max_sync(0xffffffffu, max(cnt[0], cnt[1]));
+        f2 T = f2_pack(t_[0], t_[1]), nacc = ZERO;  // nacc = -acc
+        const f2 gR = f2_pack(r_[0], r_[1]), gG = f2_pack(g_[0], g_[1]), gB = f2_pack(b_[0], b_[1]);
+        const f2 gD = f2_pack(d_[0], d_[1]), gA = f2_pack(a_[0], a_[1]);
+        const f2 zmu = f2_pack(z_[0], z_[1]), ga = f2_pack(ma_[0], ma_[1]), gb = f2_pack(mb_[0], mb_[1]);
+        uint32_t maxcnt = wmax;
+        if constexpr (NW > 1) {
+            if (lane == 0) s_max[wid] = wmax;
+            __syncthreads();
+#pragma unroll
+            for (int w = 0; w < NW; ++w) maxcnt = max(maxcnt, s_max[w]);
+        }
+        struct Work {
+            int j, count;
+            float4 u, ez;
+            F2x2 row, l, o, gbc;
+            float dxi, u1;
+            f2 DY, IN;
+            f2 sR, sG, sB, sZ;  // -wgt dL/dc
+            f2 ng;              // -dL/dpw of each pixel
+        };
+        auto begin = [&](Work &w, const BwdEntry &e) {
+            w.u = e.u;
+            w.row = load_f2x2(e.row);
+            w.l = load_f2x2(e.l);
+            w.o = load_f2x2(e.or_);
+            w.gbc = load_f2x2(e.gb);
+            w.ez = e.z;
+            w.dxi = __fsub_rn((float)px, w.u.x);
+            w.u1 = __fmaf_rn(w.u.y, w.dxi, w.u.z);
+            w.DY = f2_sub(f2_pack((float)py0, (float)(py0 + 4)), w.row.a);
+            const f2 t2 = f2_fma(w.l.b, w.DY, w.row.b);
+            w.IN = f2_fma(t2, t2, w.o.a);
+        };
+        auto work = [&](Work &w, uint32_t rel0) {
+            const f2 CW = load_f2x2(w.ez).a;
+            const f2 t1 = f2_fma(w.l.a, w.DY, f2_bcast(w.u1));
+            float n[2], al[2], ag[2];  // -e, -alpha, the -alpha that has a gradient through pw
+            f2_unpack(f2_fma(t1, t1, w.IN), n[0], n[1]);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const bool in = rel0 + w.j < cnt[h] && n[h] <= nl2amin && w.count;
+                al[h] = in ? -ex2_approx(-n[h]) : 0.f;
+                ag[h] = al[h] >= -amax ? al[h] : 0.f;
+                al[h] = fmaxf(-amax, al[h]);
+            }
+            const f2 nal = f2_pack(al[0], al[1]);
+            float om[2];
+            f2_unpack(f2_add(ONE, nal), om[0], om[1]);
+            const f2 r1m = f2_pack(rcp_approx(om[0]), rcp_approx(om[1]));  // 1 / (1 - alpha)
+            T = f2_mul(T, r1m);  // transmittance before this fragment
+            const f2 nwgt = f2_mul(nal, T);
+            f2 hh = f2_fma(gR, w.o.b, f2_fma(gG, w.gbc.a, f2_fma(gB, w.gbc.b, f2_fma(gD, CW, gA))));
+            f2 gz = gD;
+            if (VAR) {
+                const f2 dz = f2_sub(CW, zmu);
+                const f2 t = f2_fma(gb, dz, ga);  // a + b dz
+                hh = f2_fma(t, dz, hh);
+                gz = f2_add(gz, f2_fma(gb, dz, t));  // a + 2 b dz
+            }
+            // dL/dalpha = T h - acc / (1 - alpha)
+            const f2 dLda = f2_fma(T, hh, f2_mul(nacc, r1m));
+            nacc = f2_fma(nwgt, hh, nacc);
+            w.ng = f2_mul(dLda, f2_pack(ag[0], ag[1]));
+            w.sR = f2_mul(nwgt, gR);
+            w.sG = f2_mul(nwgt, gG);
+            w.sB = f2_mul(nwgt, gB);
+            w.sZ = f2_mul(nwgt, gz);
+        };
+        // the lane's two pixels lie at -2 and 2 from the middle of its rows (see k_raster_bwd)
+        auto finish = [&](const Work &w, float *mine_sum) {
+            const float l12 = f2_lo(w.l.a), l22 = f2_lo(w.l.b);
+            const float dyi = f2_lo(w.DY) + 2.f, dym = dyi + w.ez.z;
+            const float t2_m = __fmaf_rn(l22, dyi, f2_lo(w.row.b)), t1_m = __fmaf_rn(l12, dyi, w.u1);
+            const float dx = w.dxi + w.u.w;
+            float a0, a1;
+            f2_unpack(w.ng, a0, a1);
+            const float S0 = a0 + a1, S1 = 2.f * (a1 - a0), S2 = 4.f * S0;
+            // (u, v, qa, qb), (qc, ln o, r, g), (b, z)
+            *reinterpret_cast<float4 *>(mine_sum) =
+                make_float4(__fmaf_rn(l12, S1, t1_m * S0), __fmaf_rn(t2_m, S0, l22 * S1), dx * dx * S0,
+                            dx * __fmaf_rn(dym, S0, S1));
+            *reinterpret_cast<float4 *>(mine_sum + 4) =
+                make_float4(__fmaf_rn(dym, __fmaf_rn(dym, S0, S1), __fmaf_rn(dym, S1, S2)), S0,
+                            f2_lo(w.sR) + f2_hi(w.sR), f2_lo(w.sG) + f2_hi(w.sG));
+            *reinterpret_cast<float2 *>(mine_sum + 8) =
+                make_float2(f2_lo(w.sB) + f2_hi(w.sB), f2_lo(w.sZ) + f2_hi(w.sZ));
+        };
+        uint32_t id[PT], id1[PT];
+        auto load_ids = [&](int64_t h, uint32_t (&to)[PT]) {  // of the batch that ends at h, if there is one
+            const int64_t l = max((int64_t)rg.x, h - A.depth);
+#pragma unroll
+            for (int k = 0; k < PT; ++k)
+                if (l + tid + k * NT < h && tid + k * NT < A.depth) to[k] = A.vals[l + tid + k * NT];
+        };
+        auto copy_records = [&](int64_t h, const uint32_t (&of)[PT]) {
+            const int64_t l = max((int64_t)rg.x, h - A.depth);
+#pragma unroll
+            for (int k = 0; k < PT; ++k)
+                if (l + tid + k * NT < h && tid + k * NT < A.depth) {
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) cp_async16(sR + 3 * (tid + k * NT) + c, A.rec + 3 * (size_t)of[k] + c);
+                }
+            cp_async_commit();
+        };
+        const int64_t top = (int64_t)rg.x + maxcnt;
+        load_ids(top, id);
+        copy_records(top, id);
+        load_ids(top - A.depth, id1);
+        for (int64_t hi = top; hi > (int64_t)rg.x; hi -= A.depth) {
+            const int64_t lo = max((int64_t)rg.x, hi - A.depth);
+            const int nb = (int)(hi - lo);
+            __syncthreads();
+            cp_async_wait_all();
+#pragma unroll
+            for (int k = 0; k < PT; ++k) {
+                const int j = tid + k * NT;
+                if (j < nb) {
+                    const float4 r0 = sR[3 * j], r1 = sR[3 * j + 1], r2 = sR[3 * j + 2];
+                    float4 a, b;
+                    stage_record(r0, r1, a, b);
+                    sE[j].u = make_float4(a.x, b.x, a.z, r0.z);
+                    sE[j].row = make_float4(a.y, a.y, a.w, a.w);
+                    sE[j].l = make_float4(b.y, b.y, b.z, b.z);
+                    sE[j].or_ = make_float4(-b.w, -b.w, r2.x, r2.x);
+                    sE[j].gb = make_float4(r2.y, r2.y, r2.z, r2.z);
+                    sE[j].z = make_float4(r2.w, r2.w, r0.w, __uint_as_float(id[k]));
+                    sM[j] = quad_mask<TW, TH, 1>(r0, r1, r2, tx0, ty0, A.c);
+                }
+                id[k] = id1[k];
+            }
+            copy_records(hi - A.depth, id);  // (each slot has been read by its own thread)
+            load_ids(hi - 2 * (int64_t)A.depth, id1);
+            __syncthreads();
+            uint32_t which = 0;
+            int pending = 0;
+            if (NW > 1 && lane < kPairsDepth / 32) s_worked[wid][lane] = 0u;
+            __syncwarp();
+            for (int jb = (nb - 1) & ~31; jb >= 0; jb -= 32) {
+                const uint32_t rel0 = (uint32_t)(lo + jb - rg.x);
+                if (rel0 >= wmax) continue;  // no pixel of this warp reached these entries
+                const uint32_t mine = jb + lane < nb ? sM[jb + lane] : 0u;
+                uint32_t todo = __ballot_sync(0xffffffffu, (mine >> wid & 1u) && rel0 + lane < wmax);
+                if (NW > 1 && lane == 0) s_worked[wid][jb / 32] = todo;
+                while (todo) {
+                    Work w[2];
+                    w[0].j = 31 - __clz(todo);
+                    w[0].count = 1;
+                    todo ^= 1u << w[0].j;
+                    // (an odd last one is worked next to itself with alpha = 0)
+                    w[1].count = todo != 0;
+                    w[1].j = todo ? 31 - __clz(todo) : w[0].j;
+                    if (todo) todo ^= 1u << w[1].j;
+                    begin(w[0], sE[jb + w[0].j]);
+                    begin(w[1], sE[jb + w[1].j]);
+                    work(w[0], rel0);
+                    work(w[1], rel0);
+                    finish(w[0], sums + (pending * 32 + lane) * kSumRow);
+                    finish(w[1], sums + ((pending + 1) * 32 + lane) * kSumRow);
+                    which = which << 8 | (uint32_t)(jb + w[0].j);
+                    if (w[1].count) which = which << 8 | (uint32_t)(jb + w[1].j);
+                    pending += 1 + w[1].count;
+                    if (pending > kSumSlots - 2) {
+                        flush_sums<NW == 1>(sums, sE, pending, __byte_perm(which << 8 * (kSumSlots - pending), 0, 0x0123),
+                                            lane, tile_sums, A.g2d, A.state);
+                        pending = 0;
+                    }
+                }
+            }
+            // (the pending entries' staged records go with this batch)
+            if (pending)
+                flush_sums<NW == 1>(sums, sE, pending, __byte_perm(which << 8 * (kSumSlots - pending), 0, 0x0123), lane,
+                                    tile_sums, A.g2d, A.state);
+            if constexpr (NW > 1) {
+                __syncthreads();
+                for (int i = tid; i < nb * (kGrad / 2); i += NT) {
+                    const int j = i / (kGrad / 2), c = i - j * (kGrad / 2);
+                    float2 t = make_float2(0.f, 0.f);
+                    bool any = false;
+#pragma unroll
+                    for (int w = 0; w < NW; ++w)
+                        if (s_worked[w][j >> 5] >> (j & 31) & 1u) {
+                            const float2 x =
+                                *reinterpret_cast<const float2 *>(all_sums + (w * A.depth + j) * kGrad + 2 * c);
+                            t.x += x.x;
+                            t.y += x.y;
+                            any = true;
+                        }
+                    if (any) add_gradients(sE[j], c, t.x, t.y, A.g2d, A.state);
+                }
+            }
+        }
+    }
+}
+
 // zero the image-space gradients of the visible pairs (a backward that does
 // not follow its projection directly)
 __global__ void k_zero_g2d(const uint32_t *vis_pair, const DevState *st, double *g2d) {
@@ -1021,13 +1301,23 @@ RasterKernel fwd_kernel(const gs_workspace *ws, bool var) {
     }
 }
 
+// The backward's: quadrants a warp, or one a warp in pairs of entries.
 template <int TW, int TH, int Q, bool VAR>
 RasterKernel bwd_variant(int depth) {
-    const int d = std::min(depth, kBwdDepth);
+    const int d = std::min(depth, kBwdDepth<Q>);
     using S = Share<TW, TH, Q>;
     const size_t batch = S::NW > 1 ? (size_t)S::NW * d * kGrad * sizeof(float) : 0;
     return {k_raster_bwd<TW, TH, Q, VAR>, S::NT, d,
             (size_t)d * (sizeof(BwdEntry) + sizeof(uint32_t)) + S::NW * kSumBytes + batch};
+}
+template <int TW, int TH, bool VAR>
+RasterKernel bwd_pairs_variant(int depth, int64_t n_tiles) {
+    const bool deep = TW * TH < 256 ? n_tiles < 4 * kCoarseTiles : n_tiles <= kDeepTiles;
+    const int d = std::min(depth, deep ? kPairsDepth : TW * TH < 256 ? kPairsDepth / 4 : kPairsDepth / 2);
+    using S = Share<TW, TH, 1>;
+    const size_t batch = S::NW > 1 ? (size_t)S::NW * d * kGrad * sizeof(float) : 0;
+    return {k_raster_bwd_pairs<TW, TH, VAR>, S::NT, d,
+            (size_t)d * (sizeof(BwdEntry) + 3 * sizeof(float4) + sizeof(uint32_t)) + S::NW * kSumBytes + batch};
 }
 template <int TW, int TH>
 RasterKernel bwd_kernel(const gs_workspace *ws, bool var) {
@@ -1036,7 +1326,7 @@ RasterKernel bwd_kernel(const gs_workspace *ws, bool var) {
         if (ws->n_tiles * (TW * TH / 256) >= kCoarseTiles)
             return var ? bwd_variant<TW, TH, 2, true>(d) : bwd_variant<TW, TH, 4, false>(d);
     }
-    return var ? bwd_variant<TW, TH, 1, true>(d) : bwd_variant<TW, TH, 1, false>(d);
+    return var ? bwd_pairs_variant<TW, TH, true>(d, ws->n_tiles) : bwd_pairs_variant<TW, TH, false>(d, ws->n_tiles);
 }
 
 RasterKernel raster_kernel(const gs_workspace *ws, bool forward, bool var) {

@@ -89,3 +89,32 @@ def test_a_colour_that_is_not_finite_stays_where_it_is_seen(views):
     finally:
         a["renderer"].close()
         b["renderer"].close()
+
+
+# The backward that works entries in pairs stages 32, 64 or 128 of them by the
+# number of tiles and the configuration's depth: 397x401 is 2,550 tiles of 8x8 and
+# 650 of 16x16, 8 views 20,400 of 8x8; 300x241 is 304 of 16x16.
+@pytest.mark.parametrize("size,tile,views", [((397, 401), (8, 8), 1), ((397, 401), (8, 8), 8),
+                                             ((397, 401), (16, 16), 1), ((300, 241), (16, 16), 1),
+                                             ((300, 241), (16, 32), 1)])
+@pytest.mark.parametrize("depth", [32, 128, 256])
+@pytest.mark.parametrize("var", [False, True])
+def test_backward_in_pairs_gives_the_whole_tiles_gradients(size, tile, views, depth, var):
+    sc = S.random_box_scene(5000, *size, 380.0, seed=14, sh_degree=1, log_scale_mu=-2.5)
+    sc.opacity_logits[:] -= 3.0  # lists of several hundred entries, blended far down
+    rng = np.random.default_rng(5)
+    n = size[0] * size[1]
+    up = [rng.normal(size=k).astype(np.float32) for k in (3 * n, n, n)]
+
+    def grads(views, cfg, depth):
+        extra = dict(var=True, gmean=np.tile(up[1], views), gvar=0.1 * np.tile(up[2], views)) if var else {}
+        g = run_gpu(replace(sc, cameras=sc.cameras * views), cfg, *(np.tile(u, views) for u in up), depth=depth,
+                    inst_capacity=1 << 24, **extra)
+        g["renderer"].close()
+        return g
+
+    # 16 views of 16x16 tiles are on the other side of the line: whole tiles a warp
+    want = grads(16, O.Config(tile_w=16, tile_h=16), 256)
+    got = grads(views, O.Config(tile_w=tile[0], tile_h=tile[1]), depth)
+    for k in GRADS:  # either within 1e-5 of 64 bits
+        assert rel_l2(got[k].astype(np.float64) / views, want[k].astype(np.float64) / 16) < 2e-5, k
