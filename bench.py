@@ -264,7 +264,9 @@ def measure_alu_peaks(torch, G, dev, n_sm, reps=5):
 def stage_bytes(u, args):
     """Algorithmic (unique) bytes each library stage must move: every array
     read or written once, repeated reads of a record assumed to hit L2, a
-    radix sort counted at one pass (read and write key + value)."""
+    radix sort counted at one pass (read and write key + value).  An image-space
+    gradient row counts as its ten values in float, although the library sums
+    them in double (80 B)."""
     P = 4 * (3 + 3 + 4 + 1 + 3 * u["sh_coeffs"])
     var = args.depth_loss == "kl-var"
     return {
