@@ -43,12 +43,6 @@ gs_status alloc(gs_workspace *ws, Tp *&p, size_t count) {
     return GS_OK;
 }
 
-// the image-space gradients as gs_workspace_copy gives them
-__global__ void __launch_bounds__(256) k_rows_to_float(const double *rows, int64_t n, float *out) {
-    for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < n; i += (int64_t)gridDim.x * 256)
-        out[i] = (float)rows[i];
-}
-
 gs_status check_config(const gs_config *c) {
     bool tile_ok = (c->tile_w == 8 && c->tile_h == 8) || (c->tile_w == 16 && c->tile_h == 16) ||
                    (c->tile_w == 16 && c->tile_h == 32) || (c->tile_w == 32 && c->tile_h == 16);
@@ -481,7 +475,7 @@ gs_status gs_workspace_copy(gs_workspace *ws, int32_t which, void *dst, int64_t 
         case 5: src = ws->ranges; nb = ws->n_tiles * 8; break;
         case 6: src = ws->last; nb = ws->n_pix * 4; break;
         case 7: src = ws->tfin; nb = ws->n_pix * 4; break;
-        case 8: src = ws->g2d; nb = ws->n_pairs * 40; break;  // (held in double, given in float)
+        case 8: src = ws->g2d; nb = ws->n_pairs * 40; break;
         case 9: src = ws->vstat; nb = ws->n_pix * 16; break;
         default: return fail(GS_ERR_INVALID_ARG, "unknown buffer");
     }
@@ -491,12 +485,6 @@ gs_status gs_workspace_copy(gs_workspace *ws, int32_t which, void *dst, int64_t 
     }
     if (*bytes != nb) return fail(GS_ERR_INVALID_ARG, "byte count mismatch");
     if (nb == 0) return GS_OK;
-    if (which == 8) {
-        const int64_t n = nb / 4;
-        k_rows_to_float<<<(unsigned)std::min<int64_t>((n + 255) / 256, 16 * ws->num_sms), 256, 0, (cudaStream_t)stream>>>(
-            ws->g2d, n, (float *)dst);
-        return check_launch("copy");
-    }
     cudaError_t e = cudaMemcpyAsync(dst, src, (size_t)nb, cudaMemcpyDeviceToDevice, (cudaStream_t)stream);
     if (e != cudaSuccess) return fail(GS_ERR_CUDA, std::string("copy: ") + cudaGetErrorString(e));
     return GS_OK;

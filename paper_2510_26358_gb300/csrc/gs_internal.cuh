@@ -70,7 +70,7 @@ struct gs_workspace {
     float4 *rec = nullptr;         // [n_pairs][3]
     uint32_t *pkey = nullptr;      // [n_pairs]
     short4 *rect = nullptr;        // [n_pairs]
-    double *g2d = nullptr;         // [n_pairs][10]
+    float *g2d = nullptr;          // [n_pairs][10]
     uint8_t *pair_state = nullptr; // [n_pairs] kPairUnseen, kPairVisible, kPairTouched
     float4 *gdir = nullptr;        // [n_pairs] colour gradient w.r.t. the view direction
     uint32_t *vis_key = nullptr, *vis_pair = nullptr, *vis_key_alt = nullptr, *vis_pair_alt = nullptr;

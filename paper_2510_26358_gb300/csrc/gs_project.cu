@@ -287,9 +287,9 @@ struct ProjArgs {
     uint32_t *pkey;
     short4 *rect;
     uint8_t *state;   // [pairs] kPairUnseen, kPairVisible or kPairTouched
-    double *g2d_zero; // forward: the image-space gradient rows of the visible pairs, cleared here
+    float *g2d_zero;  // forward: the image-space gradient rows of the visible pairs, cleared here
     // backward
-    const double *g2d;
+    const float *g2d;
     float *gm, *gls, *gq, *gom, *gsh, *pose_part, *dens_acc;
     float4 *gdir;     // [pairs] dL/d(view direction) of the colour (x, y, z, unused)
     int32_t *dens_cnt;
@@ -544,9 +544,9 @@ __global__ void __launch_bounds__(kProjThreads) k_project_fwd(ProjArgs A) {
             // the backward's atomics add into these rows: cleared next to the
             // record (neighbouring threads, neighbouring rows) instead of by a
             // gather over the sorted visible pairs later
-            double2 *row = reinterpret_cast<double2 *>(A.g2d_zero + pair * kGrad);
+            float2 *row = reinterpret_cast<float2 *>(A.g2d_zero + pair * kGrad);
 #pragma unroll
-            for (int i = 0; i < kGrad / 2; ++i) row[i] = make_double2(0.0, 0.0);
+            for (int i = 0; i < kGrad / 2; ++i) row[i] = make_float2(0.f, 0.f);
             // (read only for visible pairs, like the record: an invisible
             // pair's rectangle is not written)
             A.rect[pair] = rc;
@@ -718,7 +718,7 @@ __global__ void __launch_bounds__(kProjBwdThreads) k_sh_bwd(ProjArgs A) {
                 // the forward marked a clamped channel by the sign of its colour
                 // (both loads issued before the camera's arithmetic)
                 const float cf = reinterpret_cast<const float *>(A.rec + 3 * pair + 2)[ch];
-                const float graw = (float)A.g2d[pair * kGrad + G_R + ch];
+                const float graw = A.g2d[pair * kGrad + G_R + ch];
                 const Cam cam = load_cam(A.cams, v);
                 float w[3], wn;
                 view_dir(cam, mu, w, wn);
@@ -851,10 +851,9 @@ __global__ void __launch_bounds__(kProjBwdThreads, 5) k_project_bwd(ProjArgs A) 
                 int v = A.sub_views[s * A.maxv + kv];
                 const ViewInfo vi = A.views[v];
                 int64_t pair = (int64_t)vi.pair_off + (g - vi.g0);
-                    const double *gg = A.g2d + pair * kGrad;
-                    const float gu = (float)gg[G_U], gv = (float)gg[G_V], gqa = (float)gg[G_QA];
-                    const float gqb = (float)gg[G_QB], gqc = (float)gg[G_QC];
-                    const float glno = (float)gg[G_LNO], gz = (float)gg[G_Z];
+                    const float *gg = A.g2d + pair * kGrad;
+                    float gu = gg[G_U], gv = gg[G_V], gqa = gg[G_QA], gqb = gg[G_QB], gqc = gg[G_QC];
+                    float glno = gg[G_LNO], gz = gg[G_Z];
                     // view-direction gradient of the colour, from the SH adjoint
                     // (loaded with the image-space row, before the pair's geometry)
                     const float4 gd4 = A.gdir[pair];

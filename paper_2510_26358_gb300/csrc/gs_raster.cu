@@ -131,7 +131,7 @@ struct RasterArgs {
     // backward inputs / outputs
     const float *dL_drgb, *dL_ddepth, *dL_dalpha;
     const float *dL_dmean, *dL_dvar;  // VAR variant
-    double *g2d;
+    float *g2d;
     uint8_t *state;  // pair states: touched pairs are marked
 };
 
@@ -642,16 +642,16 @@ struct BwdEntry {
 constexpr int kSumSlots = 4, kSumRow = 12;
 constexpr int kSumBytes = kSumSlots * 32 * kSumRow * (int)sizeof(float);
 
+__device__ __forceinline__ void red_add2(float *p, float a, float b) {
+    asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" ::"l"(p), "f"(a), "f"(b) : "memory");
+}
+
 // Component pair c of an entry's raw sums (u, v), (qa, qb), (qc, ln o), (r, g) or
 // (b, z) turned into gradients and added to its pair's row.  The raw sums are
 // negated (dpw and the weights are carried negated); dL/dQ = -1/2 sum gpw d
 // d^T; dpw/du = (Q d)_x = l11 t1 / s^2, dpw/dv = (l12 t1 + l22 t2) / s^2 with 1/s^2
-// = 2 ln 2.  The rows are in double: a near Gaussian covers thousands of tiles
-// whose sums largely cancel, and a float row lost 1e-6 of its gradients to
-// the order of the additions (against 64 bits, three 1237x701 views: log-scales
-// 8.6e-7 -> 6.0e-7, quaternions 1.4e-6 -> 8.3e-7; 4M orchard 4245 -> 4288 us, most
-// of it the clearing of the wider rows).
-__device__ __forceinline__ void add_gradients(const BwdEntry &e, int c, float x, float y, double *g2d, uint8_t *state) {
+// = 2 ln 2.
+__device__ __forceinline__ void add_gradients(const BwdEntry &e, int c, float x, float y, float *g2d, uint8_t *state) {
     const uint32_t pair = __float_as_uint(e.z.w);
     if (c == 0) {
         state[pair] = kPairTouched;
@@ -661,9 +661,7 @@ __device__ __forceinline__ void add_gradients(const BwdEntry &e, int c, float x,
         x *= c <= 2 ? 0.5f : -1.f;
         y = c == 1 ? y : -y;
     }
-    double *row = g2d + (size_t)pair * kGrad + 2 * c;
-    atomicAdd(row, (double)x);
-    atomicAdd(row + 1, (double)y);
+    red_add2(g2d + (size_t)pair * kGrad + 2 * c, x, y);
 }
 
 // Sums the n pending entries' rows; byte k of `which` is the staged index of
@@ -673,7 +671,7 @@ __device__ __forceinline__ void add_gradients(const BwdEntry &e, int c, float x,
 // order inside the tile).
 template <bool ONE_WARP>
 __device__ __forceinline__ void flush_sums(const float *sum, const BwdEntry *sE, int n, uint32_t which, int lane,
-                                           float *tile_sums, double *g2d, uint8_t *state) {
+                                           float *tile_sums, float *g2d, uint8_t *state) {
     __syncwarp();
     // lane = 8 f + 2 slot + half: column f (components 4f .. 4f + 3) of a slot's rows 16 half .. 16 half + 15
     const int f = lane >> 3, turn = lane & 7, slot = turn >> 1, half = lane & 1;
@@ -1265,10 +1263,10 @@ __global__ void __launch_bounds__(Share<TW, TH, 1>::NT, bwd_blocks(Share<TW, TH,
 
 // zero the image-space gradients of the visible pairs (a backward that does
 // not follow its projection directly)
-__global__ void k_zero_g2d(const uint32_t *vis_pair, const DevState *st, double *g2d) {
+__global__ void k_zero_g2d(const uint32_t *vis_pair, const DevState *st, float *g2d) {
     uint32_t n = st->n_vis;
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n * kGrad; i += gridDim.x * blockDim.x)
-        g2d[(size_t)vis_pair[i / kGrad] * kGrad + i % kGrad] = 0.0;
+        g2d[(size_t)vis_pair[i / kGrad] * kGrad + i % kGrad] = 0.f;
 }
 
 // The kernel of one pass for a tile size, with its launch shape.
