@@ -16,18 +16,20 @@
 // instructions, T is recovered by division, and with h = gC.c + gD z + gA
 //   dL/dalpha_j = T_j h_j - (sum_{k>j} w_k h_k) / (1 - alpha_j).
 // The 10 image-space gradient components of each Gaussian are summed over the
-// lane's pixels and then over the warp, through shared memory, before one
-// atomic per two components.
+// lane's pixels and then over the warp before they are added to its row by
+// float atomics.
 //
-// In both passes a tile is divided into quadrants of 8x8 pixels, two a lane,
-// and a warp holds one, two or four quadrants.  Of each entry it works only the
-// quadrants that the Gaussian's ellipse reaches and that still have a pixel to
-// blend: the passes are bound by instruction issue (FP32, selects and compares),
-// and of the pixel slots of a walk over whole 16x16 tiles only 43 % blend (4M
-// orchard, six 1920x1200 views; of the quadrants an entry meets 2.55 of 4
-// blend, 2.99 are reached).  Pixel updates run without branches: a pixel that a
-// fragment does not reach takes alpha = 0, for which each update is exactly the
-// identity.
+// The forward, and the backward of renders with few tiles, divide a tile into
+// quadrants of 8x8 pixels, two a lane, and a warp holds one, two or four
+// quadrants.  Of each entry it works only the quadrants that the Gaussian's
+// ellipse reaches and that still have a pixel to blend: the passes are bound by
+// instruction issue (FP32, selects and compares), and of the pixel slots of a
+// walk over whole 16x16 tiles only 43 % blend (4M orchard, six 1920x1200 views;
+// of the quadrants an entry meets 2.55 of 4 blend, 2.99 are reached).  The
+// backward of larger renders takes a column of pixels a thread (see
+// k_raster_bwd for why).  Pixel updates run without branches: a pixel
+// that a fragment does not reach takes alpha = 0, for which each update is
+// exactly the identity.
 //
 // The VAR variants also render each pixel's depth distribution under the
 // weights w: its mean mu = sum w z / W and variance var = sum w (z - mu)^2 / W,
@@ -52,15 +54,12 @@ namespace {
 constexpr float kQuadRelPad = 1e-3f, kQuadAbsPad = 1e-2f;
 
 // Entries staged at a time, at most (the configuration's batch depth below
-// it): with 64 the staged entries of 20 one-warp CTAs fit an SM.  The backward of
-// whole tiles a warp: 32 against 64, 4M orchard 1570 -> 1558 us, 500k 277 -> 271.
-// The one in pairs of entries takes all of kPairsDepth where few tiles leave the
-// SMs idle anyway, and less where more CTAs an SM are worth more (128, 64, 32
+// it): with 64 the staged entries of 20 one-warp CTAs of the forward fit an SM.
+// The backward in pairs of entries takes all of kPairsDepth where few tiles leave
+// the SMs idle anyway, and less where more CTAs an SM are worth more (128, 64, 32
 // entries, us): 300 tiles of 16x16 54, 68, 71; 3600 127, 118, 120; 8x8: 4270 380, 409,
-// 410; 9900 461, 497, 524; 43,200 584, 472, 439.
+// 410; 9900 461, 497, 524.  (Its other backward takes the configuration's depth.)
 constexpr int kFwdDepth = 64, kPairsDepth = 128;
-template <int Q>
-constexpr int kBwdDepth = Q == 4 ? 32 : 64;
 
 // How many quadrants a warp takes, by the number of 16x16 tiles (or as many
 // pixels).  Whole tiles share the most work between quadrants but make the
@@ -69,22 +68,22 @@ constexpr int kBwdDepth = Q == 4 ? 32 : 64;
 // two, four quadrants a warp, us).  Forward, the whole step: 300 tiles (320x240,
 // box of 10k) 288, 298, -; 1200 (orchard of 200k, as below) 247, 258, -; 2400
 // 318, 319, -; 3600 249, 247, -; the kernel: 7200 87, 64, 75; 24,480 (1M) -, 391,
-// 406; 54,000 (4M) -, 971, 936.  Backward, the kernel (one entry at a time): 2400
-// tiles 89, -, 138; 3600 50, -, 85; 7200 175, 130, 119; 10,800 467, 349, 274.  With
-// the variance (one, two; more do not fit the registers) forward, 2400 tiles 73,
-// 97; 7200 139, 107; backward 104, 108; 192, 147.
-constexpr int kCoarseTiles = 152 * 24;     // backward, and forward with the variance
-constexpr int kDeepTiles = 152 * 3;        // backward in pairs of entries, 16x16 tiles and larger
-constexpr int kFwdHalfTiles = 152 * 16, kFwdWholeTiles = 152 * 256;  // forward
+// 406; 54,000 (4M) -, 971, 936.  With the variance (one, two; more do not fit the
+// registers) 2400 tiles 73, 97; 7200 139, 107.
+constexpr int kFwdHalfTiles = 152 * 16, kFwdWholeTiles = 152 * 256, kVarHalfTiles = 152 * 24;
+// The backward works pairs of entries below kColumnTiles (16x16 tiles, or as many
+// pixels) and columns of pixels from there on.  kDeepTiles, in tiles of any
+// size (CTAs): see kPairsDepth.
+constexpr int kColumnTiles = 152 * 24, kDeepTiles = 152 * 3;
 
 // Resident warps an SM that each variant's registers are bounded for, as CTAs
 // (forward, 4M orchard: 20 warps of whole tiles 0.94 ms, 24 0.99 ms with spills,
-// 16 1.23 ms; backward: 16 warps 1.61 ms, 12 1.95 ms).
+// 16 1.23 ms).
 constexpr int fwd_blocks(int warps, int q, bool var) {
     return (var ? (q == 4 ? 16 : 20) : (q == 4 ? 20 : q == 2 ? 28 : 40)) / warps;
 }
 
-constexpr int bwd_blocks(int warps) { return 16 / warps; }
+constexpr int bwd_blocks(int warps) { return 16 / warps; }  // 128 registers a thread
 
 // One step of the weighted Welford update (the VAR variants), for one pixel and
 // for a packed pair; both round alike.  The first fragment (W == 0: every
@@ -621,7 +620,7 @@ __device__ __forceinline__ void cp_async16(void *dst, const void *src) {
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-// One staged list entry of the backward (see FwdEntry).
+// One staged list entry of the backward in pairs (see FwdEntry).
 struct BwdEntry {
     float4 u;    // U, l11, k1, hx
     float4 row;  // V, V, k2, k2
@@ -704,308 +703,20 @@ __device__ __forceinline__ void flush_sums(const float *sum, const BwdEntry *sE,
     __syncwarp();
 }
 
-// Back to front over each tile's list, with the forward's division of a tile
-// into quadrants and its masks; a quadrant joins the walk at the last entry
-// that one of its pixels blended.  A pixel that a fragment does not reach
-// takes alpha = 0 and runs the same instructions, which are then exactly the
-// identity (T * 1, acc + 0 * h, sums + 0; the reciprocal approximation
-// returns 1 for 1 on sm_103, measured).  The alpha decision is taken on
-// -e = fma(t1, t1, fma(t2, t2, -log2 o)), which is exactly the negation of
-// e = fma(-t1, t1, fma(-t2, t2, log2 o)) (round to nearest is symmetric), so
-// both passes take the same decisions bit for bit.
-// (Against one warp a tile, a thread a column of eight pixels and a butterfly
-// of shuffles an entry: 4M orchard, six 1920x1200 views, 1841 -> 1606 us; three
-// 1280x720 views of 500k 322 -> 281; with 32 entries staged 1558 and 271.)
-template <int TW, int TH, int Q, bool VAR>
-__global__ void __launch_bounds__(Share<TW, TH, Q>::NT, bwd_blocks(Share<TW, TH, Q>::NW))
-    k_raster_bwd(RasterArgs A) {
-    using S = Share<TW, TH, Q>;
-    constexpr int QX = S::QX, QY = S::QY, NW = S::NW, NT = S::NT;
-    extern __shared__ float4 smem[];
-    BwdEntry *sE = reinterpret_cast<BwdEntry *>(smem);
-    uint32_t *sM = reinterpret_cast<uint32_t *>(sE + A.depth);
-    float *sums = reinterpret_cast<float *>(sM + A.depth) + (NW > 1 ? (threadIdx.x >> 5) * (kSumBytes / 4) : 0);
-    // several warps: their sums of a batch, [warp][entry][component], and the entries each has worked
-    float *all_sums = reinterpret_cast<float *>(sM + A.depth) + NW * (kSumBytes / 4);
-    float *tile_sums = all_sums + (NW > 1 ? (threadIdx.x >> 5) * A.depth * kGrad : 0);
-    __shared__ uint32_t s_worked[NW > 1 ? NW : 1][kBwdDepth<Q> / 32];
-    __shared__ int s_tile;
-    __shared__ uint32_t s_max[NW];
-    const int tid = threadIdx.x, lane = tid & 31, wid = NW > 1 ? tid >> 5 : 0;
-    const float amax = A.c.alpha_max, nl2amin = -A.c.log2_alpha_min;
-    const f2 ONE = f2_bcast(1.f), ZERO = f2_bcast(0.f);
-    for (;;) {
-        __syncthreads();
-        if (tid == 0) {
-            s_tile = next_tile(A);
-        }
-        __syncthreads();
-        const int tile = s_tile;
-        if (tile < 0) break;
-        const int v = view_of_tile(A.views, A.n_views, tile);
-        const ViewInfo vi = A.views[v];
-        const int lt = tile - vi.tile_off;
-        const int tx0 = (lt % vi.ntx) * TW, ty0 = (lt / vi.ntx) * TH;
-        const int px0 = tx0 + S::wx(wid) + (lane & 7), py0 = ty0 + S::wy(wid) + (lane >> 3);
-        const uint2 rg = A.ranges[tile];
-        const int64_t hw = (int64_t)vi.W * vi.H;
-        const float *grgb = A.dL_drgb + 3 * (int64_t)vi.pix_off;
-        uint32_t cnt[Q][2], qmax[Q], wmax = 0;
-        f2 T[Q], gR[Q], gG[Q], gB[Q], gD[Q], gA[Q], nacc[Q];  // nacc = -acc
-        f2 zmu[Q], ga[Q], gb[Q];
-#pragma unroll
-        for (int q = 0; q < Q; ++q) {
-            float t_[2], r_[2], g_[2], b_[2], d_[2], a_[2], z_[2], ma_[2], mb_[2];
-            const int px = px0 + 8 * (q % QX);
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int py = py0 + 8 * (q / QX) + 4 * h;
-                cnt[q][h] = 0;
-                t_[h] = 1.f;
-                r_[h] = g_[h] = b_[h] = d_[h] = a_[h] = z_[h] = ma_[h] = mb_[h] = 0.f;
-                if (px < vi.W && py < vi.H) {
-                    const int64_t pl = (int64_t)py * vi.W + px;
-                    const int64_t pix = vi.pix_off + pl;
-                    cnt[q][h] = A.last[pix];
-                    t_[h] = A.tfin[pix];
-                    r_[h] = grgb[pl];
-                    g_[h] = grgb[hw + pl];
-                    b_[h] = grgb[2 * hw + pl];
-                    d_[h] = A.dL_ddepth ? A.dL_ddepth[pix] : 0.f;
-                    a_[h] = A.dL_dalpha ? A.dL_dalpha[pix] : 0.f;
-                    if (VAR) {
-                        const float4 vs = A.vstat[pix];
-                        z_[h] = vs.x;
-                        ma_[h] = A.dL_dmean ? A.dL_dmean[pix] * vs.z : 0.f;
-                        mb_[h] = A.dL_dvar ? A.dL_dvar[pix] * vs.z : 0.f;
-                        a_[h] = __fmaf_rn(-mb_[h], vs.y, a_[h]);  // the -b var part of every h
-                    }
-                }
-            }
-            qmax[q] = __reduce_max_sync(0xffffffffu, max(cnt[q][0], cnt[q][1]));
-            wmax = max(wmax, qmax[q]);
-            T[q] = f2_pack(t_[0], t_[1]);
-            gR[q] = f2_pack(r_[0], r_[1]);
-            gG[q] = f2_pack(g_[0], g_[1]);
-            gB[q] = f2_pack(b_[0], b_[1]);
-            gD[q] = f2_pack(d_[0], d_[1]);
-            gA[q] = f2_pack(a_[0], a_[1]);
-            nacc[q] = ZERO;
-            if (VAR) {
-                zmu[q] = f2_pack(z_[0], z_[1]);
-                ga[q] = f2_pack(ma_[0], ma_[1]);
-                gb[q] = f2_pack(mb_[0], mb_[1]);
-            }
-        }
-        uint32_t maxcnt = wmax;
-        if constexpr (NW > 1) {
-            if (lane == 0) s_max[wid] = wmax;
-            __syncthreads();
-#pragma unroll
-            for (int w = 0; w < NW; ++w) maxcnt = max(maxcnt, s_max[w]);
-        }
-        for (int64_t hi = (int64_t)rg.x + maxcnt; hi > (int64_t)rg.x; hi -= A.depth) {
-            const int64_t lo = max((int64_t)rg.x, hi - A.depth);
-            const int nb = (int)(hi - lo);
-            __syncthreads();
-            for (int j = tid; j < nb; j += NT) {
-                const uint32_t pair = A.vals[lo + j];
-                const float4 r0 = A.rec[3 * (size_t)pair], r1 = A.rec[3 * (size_t)pair + 1];
-                const float4 r2 = A.rec[3 * (size_t)pair + 2];
-                float4 a, b;
-                stage_record(r0, r1, a, b);
-                sE[j].u = make_float4(a.x, b.x, a.z, r0.z);
-                sE[j].row = make_float4(a.y, a.y, a.w, a.w);
-                sE[j].l = make_float4(b.y, b.y, b.z, b.z);
-                sE[j].or_ = make_float4(-b.w, -b.w, r2.x, r2.x);
-                sE[j].gb = make_float4(r2.y, r2.y, r2.z, r2.z);
-                sE[j].z = make_float4(r2.w, r2.w, r0.w, __uint_as_float(pair));
-                sM[j] = quad_mask<TW, TH, Q>(r0, r1, r2, tx0, ty0, A.c);
-            }
-            __syncthreads();
-            uint32_t which = 0;
-            int pending = 0;
-            if (NW > 1 && lane < kBwdDepth<Q> / 32) s_worked[wid][lane] = 0u;
-            __syncwarp();
-            for (int jb = (nb - 1) & ~31; jb >= 0; jb -= 32) {
-                const uint32_t rel0 = (uint32_t)(lo + jb - rg.x);
-                if (rel0 >= wmax) continue;  // no pixel of this warp reached these entries
-                const uint32_t mine = jb + lane < nb ? sM[jb + lane] : 0u;
-                const uint32_t exact = __ballot_sync(0xffffffffu, mine & kExactPath);
-                uint32_t E[Q], todo = 0, all = ~0u;
-#pragma unroll
-                for (int q = 0; q < Q; ++q) {
-                    const bool hit = (mine >> (wid * Q + q) & 1u) && rel0 + lane < qmax[q];
-                    E[q] = __ballot_sync(0xffffffffu, hit);
-                    todo |= E[q];
-                    all &= E[q];
-                }
-                if (NW > 1 && lane == 0) s_worked[wid][jb / 32] = todo;
-                while (todo) {
-                    const int j = 31 - __clz(todo);
-                    todo ^= 1u << j;
-                    const uint32_t rel = rel0 + j;
-                    const BwdEntry &e = sE[jb + j];
-                    const float4 u = e.u;
-                    const F2x2 row = load_f2x2(e.row), l = load_f2x2(e.l), o = load_f2x2(e.or_), gbc = load_f2x2(e.gb);
-                    const float4 ez = e.z;
-                    const f2 CW = load_f2x2(ez).a;
-                    float dxi[QX], u1[QX];
-                    f2 DY[QY], IN[QY];
-#pragma unroll
-                    for (int x = 0; x < QX; ++x) {
-                        dxi[x] = __fsub_rn((float)(px0 + 8 * x), u.x);
-                        u1[x] = __fmaf_rn(u.y, dxi[x], u.z);
-                    }
-#pragma unroll
-                    for (int y = 0; y < QY; ++y) {
-                        DY[y] = f2_sub(f2_pack((float)(py0 + 8 * y), (float)(py0 + 8 * y + 4)), row.a);
-                        const f2 t2 = f2_fma(l.b, DY[y], row.b);
-                        IN[y] = f2_fma(t2, t2, o.a);
-                    }
-                    f2 sR = ZERO, sG = ZERO, sB_ = ZERO, sZ = ZERO;  // sums of -wgt dL/dc
-                    f2 ng[Q];                                        // -dL/dpw of each pixel
-                    auto quad = [&](int q, const bool clamp) {
-                        const f2 t1 = f2_fma(l.a, DY[q / QX], f2_bcast(u1[q % QX]));
-                        float n[2], al[2], ag[2];  // -e, -alpha, the -alpha that has a gradient through pw
-                        f2_unpack(f2_fma(t1, t1, IN[q / QX]), n[0], n[1]);
-#pragma unroll
-                        for (int h = 0; h < 2; ++h) {
-                            const bool in = rel < cnt[q][h] && n[h] <= nl2amin;
-                            al[h] = ag[h] = in ? -ex2_approx(-n[h]) : 0.f;
-                            if (clamp) {
-                                ag[h] = al[h] >= -amax ? al[h] : 0.f;
-                                al[h] = fmaxf(-amax, al[h]);
-                            }
-                        }
-                        const f2 nal = f2_pack(al[0], al[1]);
-                        float om[2];
-                        f2_unpack(f2_add(ONE, nal), om[0], om[1]);
-                        const f2 r1m = f2_pack(rcp_approx(om[0]), rcp_approx(om[1]));  // 1 / (1 - alpha)
-                        T[q] = f2_mul(T[q], r1m);  // transmittance before this fragment
-                        const f2 nwgt = f2_mul(nal, T[q]);
-                        f2 hh = f2_fma(gR[q], o.b, f2_fma(gG[q], gbc.a, f2_fma(gB[q], gbc.b, f2_fma(gD[q], CW, gA[q]))));
-                        f2 gz = gD[q];
-                        if (VAR) {
-                            const f2 dz = f2_sub(CW, zmu[q]);
-                            const f2 t = f2_fma(gb[q], dz, ga[q]);  // a + b dz
-                            hh = f2_fma(t, dz, hh);
-                            gz = f2_add(gz, f2_fma(gb[q], dz, t));  // a + 2 b dz
-                        }
-                        // dL/dalpha = T h - acc / (1 - alpha)
-                        const f2 dLda = f2_fma(T[q], hh, f2_mul(nacc[q], r1m));
-                        nacc[q] = f2_fma(nwgt, hh, nacc[q]);
-                        ng[q] = f2_mul(dLda, clamp ? f2_pack(ag[0], ag[1]) : nal);
-                        sR = f2_fma(nwgt, gR[q], sR);
-                        sG = f2_fma(nwgt, gG[q], sG);
-                        sB_ = f2_fma(nwgt, gB[q], sB_);
-                        sZ = f2_fma(nwgt, gz, sZ);
-                    };
-                    if ((all & ~exact) >> j & 1u) {
-                        // every quadrant, interleaved (1680 -> 1606 us, 4M orchard)
-#pragma unroll
-                        for (int q = 0; q < Q; ++q) quad(q, false);
-                    } else {
-#pragma unroll
-                        for (int q = 0; q < Q; ++q) ng[q] = ZERO;
-                        if (!(exact >> j & 1u)) {
-#pragma unroll
-                            for (int q = 0; q < Q; ++q)
-                                if (E[q] >> j & 1u) quad(q, false);
-                        } else {
-#pragma unroll
-                            for (int q = 0; q < Q; ++q)
-                                if (E[q] >> j & 1u) quad(q, true);
-                        }
-                    }
-                    // Moments of the lane's pixels about the middle of its rows,
-                    // which lie at -6, -2, 2 and 6 (-2, 2) from there: with S_k = sum
-                    // over a column of row^k (-gpw), t1 and t2 affine in the row,
-                    // dy = dym + row.  (About the first row the terms are up to
-                    // twice as large and cancel.)
-                    constexpr float MID = QY == 2 ? 6.f : 2.f;
-                    const float dyi = f2_lo(DY[0]) + MID, dym = dyi + ez.z;
-                    const float t2_m = __fmaf_rn(e.l.z, dyi, e.row.z);
-                    float S0 = 0.f, S1 = 0.f, S2 = 0.f, mU = 0.f, mA = 0.f, mB = 0.f;
-#pragma unroll
-                    for (int x = 0; x < QX; ++x) {
-                        float a0, a1, s0, s1, s2;
-                        f2_unpack(ng[x], a0, a1);
-                        if (QY == 2) {
-                            float b0, b1;
-                            f2_unpack(ng[(QY - 1) * QX + x], b0, b1);
-                            const float outer = a0 + b1, inner = a1 + b0;
-                            s0 = outer + inner;
-                            s1 = __fmaf_rn(6.f, b1 - a0, 2.f * (b0 - a1));
-                            s2 = __fmaf_rn(36.f, outer, 4.f * inner);
-                        } else {
-                            s0 = a0 + a1;
-                            s1 = 2.f * (a1 - a0);
-                            s2 = 4.f * s0;
-                        }
-                        const float dx = dxi[x] + u.w;
-                        const float t1_m = __fmaf_rn(e.l.x, dyi, u1[x]);
-                        S0 += s0;
-                        S1 += s1;
-                        S2 += s2;
-                        mU = __fmaf_rn(t1_m, s0, mU);
-                        mA = __fmaf_rn(dx * dx, s0, mA);
-                        mB = __fmaf_rn(dx, __fmaf_rn(dym, s0, s1), mB);
-                    }
-                    float *mine_sum = sums + (pending * 32 + lane) * kSumRow;
-                    // (u, v, qa, qb), (qc, ln o, r, g), (b, z)
-                    *reinterpret_cast<float4 *>(mine_sum) =
-                        make_float4(__fmaf_rn(e.l.x, S1, mU), __fmaf_rn(t2_m, S0, e.l.z * S1), mA, mB);
-                    *reinterpret_cast<float4 *>(mine_sum + 4) =
-                        make_float4(__fmaf_rn(dym, __fmaf_rn(dym, S0, S1), __fmaf_rn(dym, S1, S2)), S0,
-                                    f2_lo(sR) + f2_hi(sR), f2_lo(sG) + f2_hi(sG));
-                    *reinterpret_cast<float2 *>(mine_sum + 8) =
-                        make_float2(f2_lo(sB_) + f2_hi(sB_), f2_lo(sZ) + f2_hi(sZ));
-                    which = which << 8 | (uint32_t)(jb + j);
-                    if (++pending == kSumSlots) {
-                        flush_sums<NW == 1>(sums, sE, kSumSlots, __byte_perm(which, 0, 0x0123), lane, tile_sums, A.g2d,
-                                            A.state);
-                        pending = 0;
-                    }
-                }
-            }
-            // (the pending entries' staged records go with this batch)
-            if (pending)
-                flush_sums<NW == 1>(sums, sE, pending, __byte_perm(which << 8 * (kSumSlots - pending), 0, 0x0123), lane,
-                                    tile_sums, A.g2d, A.state);
-            if constexpr (NW > 1) {
-                __syncthreads();
-                for (int i = tid; i < nb * (kGrad / 2); i += NT) {
-                    const int j = i / (kGrad / 2), c = i - j * (kGrad / 2);
-                    float2 t = make_float2(0.f, 0.f);
-                    bool any = false;
-#pragma unroll
-                    for (int w = 0; w < NW; ++w)
-                        if (s_worked[w][j >> 5] >> (j & 31) & 1u) {
-                            const float2 x =
-                                *reinterpret_cast<const float2 *>(all_sums + (w * A.depth + j) * kGrad + 2 * c);
-                            t.x += x.x;
-                            t.y += x.y;
-                            any = true;
-                        }
-                    if (any) add_gradients(sE[j], c, t.x, t.y, A.g2d, A.state);
-                }
-            }
-        }
-    }
-}
-
-// The backward with one quadrant a warp, for few tiles (below kCoarseTiles) and
-// for 8x8 ones: a warp's walk along its list is then a chain that little
-// else on the SM hides.  Two entries are worked together (only T and the suffix
-// sum go from one to the next), and the next batch's records are copied in while
-// this one is worked, their pair ids read a batch earlier still.  The
-// arithmetic is k_raster_bwd's with the clamp's two selects always in, which
-// change nothing where alpha stays below its maximum.  Measured against one
-// entry at a time with loads at the head of a batch of 64: 300 tiles of 16x16
-// (box of 10k) 83 -> 55 us; 3600 (orchard of 300k, variance) 129 -> 116; 8x8 tiles:
-// 4270 with long lists (orchard of 1.3M, 481x280) 517 -> 394, 43,200 (500k) 458 ->
-// 448.
+// The backward with few tiles (below kColumnTiles): one quadrant a warp, back to
+// front over the tile's list with the forward's masks.  A warp's walk is then
+// a chain that little else on the SM hides.  Two entries are worked together
+// (only T and the suffix sum go from one to the next), and the next batch's
+// records are copied in while this one is worked, their pair ids read a batch
+// earlier still.  A pixel that a fragment does not reach takes alpha = 0 and runs
+// the same instructions, which are then exactly the identity (T * 1, acc + 0 * h,
+// sums + 0; the reciprocal approximation returns 1 for 1 on sm_103, measured).
+// The alpha decision is taken on -e = fma(t1, t1, fma(t2, t2, -log2 o)), which is
+// exactly the negation of e = fma(-t1, t1, fma(-t2, t2, log2 o)) (round to nearest
+// is symmetric), so both passes take the same decisions bit for bit.  Measured
+// against one entry at a time with loads at the head of a batch of 64: 300 tiles
+// of 16x16 (box of 10k) 83 -> 55 us; 3600 (orchard of 300k, variance) 129 -> 116; 8x8
+// tiles: 4270 with long lists (orchard of 1.3M, 481x280) 517 -> 394.
 template <int TW, int TH, bool VAR>
 __global__ void __launch_bounds__(Share<TW, TH, 1>::NT, bwd_blocks(Share<TW, TH, 1>::NW))
     k_raster_bwd_pairs(RasterArgs A) {
@@ -1135,7 +846,10 @@ __global__ void __launch_bounds__(Share<TW, TH, 1>::NT, bwd_blocks(Share<TW, TH,
             w.sB = f2_mul(nwgt, gB);
             w.sZ = f2_mul(nwgt, gz);
         };
-        // the lane's two pixels lie at -2 and 2 from the middle of its rows (see k_raster_bwd)
+        // Moments of the lane's two pixels about the middle of its rows, which lie
+        // at -2 and 2 from there: with S_k = sum of row^k (-gpw), t1 and t2 affine in
+        // the row, dy = dym + row.  (About the first row the terms are up to twice
+        // as large and cancel.)
         auto finish = [&](const Work &w, float *mine_sum) {
             const float l12 = f2_lo(w.l.a), l22 = f2_lo(w.l.b);
             const float dyi = f2_lo(w.DY) + 2.f, dym = dyi + w.ez.z;
@@ -1261,6 +975,325 @@ __global__ void __launch_bounds__(Share<TW, TH, 1>::NT, bwd_blocks(Share<TW, TH,
     }
 }
 
+// Sums ten per-lane values over the warp by recursive halving: at each of the
+// five butterfly levels a lane keeps half of its remaining components and
+// sends the other half to its partner, so 12 shuffles replace 50.  Afterwards
+// lane l holds the warp total of component
+//   comp(l) = 5*b4 + 3*b3 + 2*b2 + b1      (bK = bit K of l),
+// valid when (b3 == 0 and not (b2 and b1)) or (b3 == 1 and b2 == 0); lanes l
+// and l^1 hold the same total.  reduce10_component gives comp(l) or -1.
+__device__ __forceinline__ float warp_reduce_scatter10(const float v[10], int lane) {
+    const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4, b1 = lane & 2;
+    float a[5];
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+        float send = b4 ? v[i] : v[i + 5];
+        float keep = b4 ? v[i + 5] : v[i];
+        a[i] = keep + __shfl_xor_sync(0xffffffffu, send, 16);
+    }
+    float c[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        float hiv = i + 3 < 5 ? a[i + 3] : 0.f;
+        float send = b3 ? a[i] : hiv;
+        float keep = b3 ? hiv : a[i];
+        c[i] = keep + __shfl_xor_sync(0xffffffffu, send, 8);
+    }
+    float d[2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        float hiv = i + 2 < 3 ? c[i + 2] : 0.f;
+        float send = b2 ? c[i] : hiv;
+        float keep = b2 ? hiv : c[i];
+        d[i] = keep + __shfl_xor_sync(0xffffffffu, send, 4);
+    }
+    float send = b1 ? d[0] : d[1];
+    float keep = b1 ? d[1] : d[0];
+    float e = keep + __shfl_xor_sync(0xffffffffu, send, 2);
+    return e + __shfl_xor_sync(0xffffffffu, e, 1);
+}
+
+__device__ __forceinline__ int reduce10_component(int lane) {
+    const int b4 = (lane >> 4) & 1, b3 = (lane >> 3) & 1, b2 = (lane >> 2) & 1, b1 = (lane >> 1) & 1;
+    const bool ok = b3 == 0 ? !(b2 && b1) : b2 == 0;
+    return ok ? 5 * b4 + 3 * b3 + 2 * b2 + b1 : -1;
+}
+
+// The backward of renders of kColumnTiles and more: a thread works PPT pixels of
+// a column, a warp's sums go to the rows by one butterfly an entry.  Quadrants
+// and sums about their middle, added to rows in double, took 1558 us where this
+// takes 1841 (4M orchard, six 1920x1200 views) and come nearer to 64 bits, but
+// move results that must stay where they are: the gradients of a long thin
+// Gaussian near a camera are sums over thousands of tiles that largely cancel, and
+// in another order of the terms the quaternion gradients of that step changed by
+// up to 1.6e-4 in norm (240 random maps; repeating the same order changes them by
+// 1e-6, and one map in eight passed 2e-5 in norm or 8e-4 at an element).  Below
+// kColumnTiles no Gaussian covers that many tiles, and the other order stays inside.
+// The terms, their order inside a warp, and the float rows are therefore fixed.
+//
+// At least 512 resident threads per SM (16 warps, 128 registers a thread):
+// with eight pixels a thread, measured best on the 500k orchard (16 one-warp
+// blocks: 0.435 ms; 14: 0.441 ms).
+//
+// A thread's PPT pixels are worked in Q = PPT/2 packed pairs (pixel p in the
+// low half, pixel p + Q in the high half), so that one f32x2 instruction does
+// the arithmetic of two pixels.  The alpha decision is taken on
+// -e = fma(t1, t1, fma(t2, t2, -log2 o)), which is exactly the negation of
+// the forward's e = fma(-t1, t1, fma(-t2, t2, log2 o)) (round to nearest is
+// symmetric), so both passes take the same decisions bit for bit.
+template <int TW, int TH, int PPT, bool VAR>
+__global__ void __launch_bounds__(TW * TH / PPT, 512 / (TW * TH / PPT)) k_raster_bwd(RasterArgs A) {
+    constexpr int NT = TW * TH / PPT;
+    static_assert(NT % 32 == 0, "the backward needs whole warps");
+    static_assert(PPT % 2 == 0, "the backward works pixels in pairs");
+    constexpr int NW = (NT + 31) / 32;
+    constexpr int Q = PPT / 2;
+    extern __shared__ float4 smem[];
+    float4 *sA = smem, *sB = smem + A.depth, *sC = smem + 2 * A.depth;
+    float2 *sH = reinterpret_cast<float2 *>(smem + 3 * A.depth);
+    uint32_t *sP = reinterpret_cast<uint32_t *>(sH + A.depth);
+    __shared__ int s_tile;
+    __shared__ uint32_t s_max[NW];
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const float amax = A.c.alpha_max, nl2amin = -A.c.log2_alpha_min;
+    const f2 ONE = f2_bcast(1.f);
+    // component this lane adds after the reduction (even lanes only), and the
+    // factors c0 + c11 l11 + c22 l22 that turn its raw sum into the gradient
+    // (the colour and depth sums come out negated, see below)
+    const int my_comp = (lane & 1) ? -1 : reduce10_component(lane);
+    const float sc0 = my_comp == G_QA || my_comp == G_QC ? -0.5f
+                      : my_comp == G_QB                  ? -1.f
+                      : my_comp == G_U || my_comp == G_V ? 0.f
+                      : my_comp == G_LNO                 ? 1.f
+                                                         : -1.f;
+    const float sc11 = my_comp == G_U ? kTwoLn2 : 0.f;
+    const float sc22 = my_comp == G_V ? kTwoLn2 : 0.f;
+    for (;;) {
+        __syncthreads();
+        if (tid == 0) {
+            s_tile = next_tile(A);
+        }
+        __syncthreads();
+        const int tile = s_tile;
+        if (tile < 0) break;
+        const int v = view_of_tile(A.views, A.n_views, tile);
+        const ViewInfo vi = A.views[v];
+        const int lt = tile - vi.tile_off;
+        const int px = (lt % vi.ntx) * TW + tid % TW;
+        const int py0 = (lt / vi.ntx) * TH + (tid / TW) * PPT;
+        const float pxf = (float)px;
+        const f2 PY0 = f2_pack((float)py0, (float)(py0 + Q));
+        const uint2 rg = A.ranges[tile];
+        const int64_t hw = (int64_t)vi.W * vi.H;
+        const float *grgb = A.dL_drgb + 3 * (int64_t)vi.pix_off;
+        uint32_t cnt[PPT], mycnt = 0;
+        f2 T[Q], gR[Q], gG[Q], gB[Q], gD[Q], gA[Q], nacc[Q];  // nacc = -acc
+        f2 zmu[Q], ga[Q], gb[Q];
+#pragma unroll
+        for (int p = 0; p < Q; ++p) {
+            float t_[2], r_[2], g_[2], b_[2], d_[2], a_[2], z_[2], ma_[2], mb_[2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int i = p + h * Q, py = py0 + i;
+                cnt[i] = 0;
+                t_[h] = 1.f;
+                r_[h] = g_[h] = b_[h] = d_[h] = a_[h] = z_[h] = ma_[h] = mb_[h] = 0.f;
+                if (px < vi.W && py < vi.H) {
+                    const int64_t pl = (int64_t)py * vi.W + px;
+                    const int64_t pix = vi.pix_off + pl;
+                    cnt[i] = A.last[pix];
+                    t_[h] = A.tfin[pix];
+                    r_[h] = grgb[pl];
+                    g_[h] = grgb[hw + pl];
+                    b_[h] = grgb[2 * hw + pl];
+                    d_[h] = A.dL_ddepth ? A.dL_ddepth[pix] : 0.f;
+                    a_[h] = A.dL_dalpha ? A.dL_dalpha[pix] : 0.f;
+                    if (VAR) {
+                        const float4 vs = A.vstat[pix];
+                        z_[h] = vs.x;
+                        ma_[h] = A.dL_dmean ? A.dL_dmean[pix] * vs.z : 0.f;
+                        mb_[h] = A.dL_dvar ? A.dL_dvar[pix] * vs.z : 0.f;
+                        a_[h] = __fmaf_rn(-mb_[h], vs.y, a_[h]);  // the -b var part of every h
+                    }
+                }
+                mycnt = max(mycnt, cnt[i]);
+            }
+            T[p] = f2_pack(t_[0], t_[1]);
+            gR[p] = f2_pack(r_[0], r_[1]);
+            gG[p] = f2_pack(g_[0], g_[1]);
+            gB[p] = f2_pack(b_[0], b_[1]);
+            gD[p] = f2_pack(d_[0], d_[1]);
+            gA[p] = f2_pack(a_[0], a_[1]);
+            nacc[p] = f2_bcast(0.f);
+            if (VAR) {
+                zmu[p] = f2_pack(z_[0], z_[1]);
+                ga[p] = f2_pack(ma_[0], ma_[1]);
+                gb[p] = f2_pack(mb_[0], mb_[1]);
+            }
+        }
+        uint32_t wmax = mycnt;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) wmax = max(wmax, __shfl_xor_sync(0xffffffffu, wmax, o));
+        if (lane == 0) s_max[wid] = wmax;
+        __syncthreads();
+        uint32_t maxcnt = 0;
+#pragma unroll
+        for (int w = 0; w < NW; ++w) maxcnt = max(maxcnt, s_max[w]);
+        for (int64_t hi = (int64_t)rg.x + maxcnt; hi > (int64_t)rg.x; hi -= A.depth) {
+            const int64_t lo = max((int64_t)rg.x, hi - A.depth);
+            const int nb = (int)(hi - lo);
+            __syncthreads();
+            for (int j = tid; j < nb; j += NT) {
+                uint32_t pair = A.vals[lo + j];
+                float4 r0 = A.rec[3 * (size_t)pair], r1 = A.rec[3 * (size_t)pair + 1];
+                float4 a, bb;
+                stage_record(r0, r1, a, bb);
+                sA[j] = a;
+                sB[j] = bb;
+                sC[j] = A.rec[3 * (size_t)pair + 2];
+                sH[j] = make_float2(r0.z, r0.w);
+                sP[j] = pair;
+            }
+            __syncthreads();
+            for (int j = nb - 1; j >= 0; --j) {
+                const uint32_t rel = (uint32_t)(lo + j - rg.x);
+                if (rel >= wmax) continue;  // no pixel of this warp reached this entry
+                const float4 a = sA[j], b = sB[j];
+                float dxi, u1;
+                frag_column(a, b, pxf, dxi, u1);
+                // the forward's alpha decision for each of the thread's pixels:
+                // ar = the unclamped alpha of a pixel the fragment reaches, else 0
+                float ar[PPT], t1_0 = 0.f, t2_0 = 0.f, dyi_0 = 0.f;
+                bool any = false;
+                {
+                    const f2 AY = f2_bcast(a.y), L12 = f2_bcast(b.y), L22 = f2_bcast(b.z);
+                    const f2 U1 = f2_bcast(u1), K2 = f2_bcast(a.w), NBW = f2_bcast(-b.w);
+                    f2 PY = PY0;
+#pragma unroll
+                    for (int p = 0; p < Q; ++p) {
+                        const f2 dy = f2_sub(PY, AY);  // dyi = py - V, exact as in the forward
+                        if (p + 1 < Q) PY = f2_add(PY, ONE);
+                        const f2 t1 = f2_fma(L12, dy, U1);
+                        const f2 t2 = f2_fma(L22, dy, K2);
+                        const f2 ne = f2_fma(t1, t1, f2_fma(t2, t2, NBW));  // -e
+                        if (p == 0) {
+                            t1_0 = f2_lo(t1);
+                            t2_0 = f2_lo(t2);
+                            dyi_0 = f2_lo(dy);
+                        }
+                        float n_[2];
+                        f2_unpack(ne, n_[0], n_[1]);
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            const int i = p + h * Q;
+                            const bool in = rel < cnt[i] && n_[h] <= nl2amin;
+                            ar[i] = in ? ex2_approx(-n_[h]) : 0.f;
+                            any |= in;
+                        }
+                    }
+                }
+                if (!__any_sync(0xffffffffu, any)) continue;
+                // Every pixel runs the same instructions: a pixel this fragment
+                // does not reach takes alpha = 0, for which each update below is
+                // exactly the identity (T * 1, acc + 0 * h, sums + 0; the
+                // reciprocal approximation returns 1 for 1 on sm_103, measured).
+                // The blended sums are carried negated (nwgt = -wgt), which
+                // saves the negations the packed instructions cannot fold.
+                const float4 c = sC[j];
+                const f2 CX = f2_bcast(c.x), CY = f2_bcast(c.y), CZ = f2_bcast(c.z), CW = f2_bcast(c.w);
+                f2 sR, sG, sB_, sZ;  // sums of -wgt dL/dc
+                // R_k = sum over pairs p of p^k gpw (k = 0, 1, 2), gpw = dL/dpw
+                f2 R0, R1, R2;
+#pragma unroll
+                for (int p = 0; p < Q; ++p) {
+                    const float a0 = ar[p], a1 = ar[p + Q];
+                    const f2 nal = f2_pack(fmaxf(-amax, -a0), fmaxf(-amax, -a1));  // -alpha
+                    // alpha of an unclamped pixel, else 0: a clamped alpha has no
+                    // gradient through pw
+                    const f2 ag = f2_pack(a0 <= amax ? a0 : 0.f, a1 <= amax ? a1 : 0.f);
+                    float o_[2];
+                    f2_unpack(f2_add(ONE, nal), o_[0], o_[1]);
+                    const f2 r1m = f2_pack(rcp_approx(o_[0]), rcp_approx(o_[1]));  // 1 / (1 - alpha)
+                    T[p] = f2_mul(T[p], r1m);  // transmittance before this fragment
+                    const f2 nwgt = f2_mul(nal, T[p]);
+                    f2 h = f2_fma(gR[p], CX, f2_fma(gG[p], CY, f2_fma(gB[p], CZ, f2_fma(gD[p], CW, gA[p]))));
+                    f2 gz = gD[p];
+                    if (VAR) {
+                        const f2 dz = f2_sub(CW, zmu[p]);
+                        const f2 t = f2_fma(gb[p], dz, ga[p]);  // a + b dz
+                        h = f2_fma(t, dz, h);
+                        gz = f2_add(gz, f2_fma(gb[p], dz, t));  // a + 2 b dz
+                    }
+                    // dL/dalpha = T h - acc / (1 - alpha)
+                    const f2 dLda = f2_fma(T[p], h, f2_mul(nacc[p], r1m));
+                    nacc[p] = f2_fma(nwgt, h, nacc[p]);
+                    const f2 gpw = f2_mul(dLda, ag);
+                    if (p == 0) {
+                        sR = f2_mul(nwgt, gR[p]);
+                        sG = f2_mul(nwgt, gG[p]);
+                        sB_ = f2_mul(nwgt, gB[p]);
+                        sZ = f2_mul(nwgt, gz);
+                        R0 = gpw;
+                    } else {
+                        sR = f2_fma(nwgt, gR[p], sR);
+                        sG = f2_fma(nwgt, gG[p], sG);
+                        sB_ = f2_fma(nwgt, gB[p], sB_);
+                        sZ = f2_fma(nwgt, gz, sZ);
+                        R0 = f2_add(R0, gpw);
+                    }
+                    if (p == 1) {
+                        R1 = gpw;
+                        R2 = gpw;
+                    } else if (p > 1) {
+                        R1 = f2_fma(gpw, f2_bcast((float)p), R1);
+                        R2 = f2_fma(gpw, f2_bcast((float)(p * p)), R2);
+                    }
+                }
+                if (Q == 1) R1 = R2 = f2_bcast(0.f);
+                // S_k = sum over the column's pixels i of i^k gpw: pixel p + Q
+                // sits in the high half of pair p
+                float r0l, r0h, r1l, r1h, r2l, r2h;
+                f2_unpack(R0, r0l, r0h);
+                f2_unpack(R1, r1l, r1h);
+                f2_unpack(R2, r2l, r2h);
+                const float S0 = r0l + r0h;
+                const float S1 = __fmaf_rn((float)Q, r0h, r1l + r1h);
+                const float S2 = __fmaf_rn((float)(Q * Q), r0h, __fmaf_rn((float)(2 * Q), r1h, r2l + r2h));
+                // per-lane raw moments: the pixel offsets are dx (one per column)
+                // and dy_i = dy_0 + i, and t1, t2 are affine in i; the
+                // per-Gaussian factors are applied once after the warp reduction
+                const float2 hh = sH[j];
+                const float dx = dxi + hh.x, dy0 = dyi_0 + hh.y;
+                const float sy = __fmaf_rn(dy0, S0, S1);  // sum gpw dy
+                float g[kGrad];
+                g[G_LNO] = S0;
+                g[G_U] = __fmaf_rn(t1_0, S0, b.y * S1);  // sum gpw t1, t1_i = t1_0 + l12 i
+                g[G_V] = __fmaf_rn(t2_0, S0, b.z * S1);  // sum gpw t2, t2_i = t2_0 + l22 i
+                g[G_QA] = dx * dx * S0;                     // sum gpw dx^2
+                g[G_QB] = dx * sy;                          // sum gpw dx dy
+                g[G_QC] = __fmaf_rn(dy0, sy, __fmaf_rn(dy0, S1, S2));  // sum gpw dy^2
+                g[G_R] = f2_lo(sR) + f2_hi(sR);
+                g[G_G] = f2_lo(sG) + f2_hi(sG);
+                g[G_B] = f2_lo(sB_) + f2_hi(sB_);
+                g[G_Z] = f2_lo(sZ) + f2_hi(sZ);
+                const float tot = warp_reduce_scatter10(g, lane);
+                if (my_comp >= 0) {
+                    // dL/dQ = -1/2 sum gpw d d^T; dpw/du = (Q d)_x = l11 t1 / s^2,
+                    // dpw/dv = (l12 t1 + l22 t2) / s^2 with 1/s^2 = 2 ln 2: each lane
+                    // scales its sum by c0 + c11 l11 + c22 l22 (constants per lane;
+                    // c0 = -1 undoes the negation of the colour and depth sums)
+                    float *gp = A.g2d + (size_t)sP[j] * kGrad;
+                    atomicAdd(gp + my_comp, tot * __fmaf_rn(sc11, b.x, __fmaf_rn(sc22, b.z, sc0)));
+                    if (my_comp == G_U) {
+                        atomicAdd(gp + G_V, kTwoLn2 * b.y * tot);
+                        A.state[sP[j]] = kPairTouched;
+                    }
+                }
+            }
+        }
+    }
+}
+
 // zero the image-space gradients of the visible pairs (a backward that does
 // not follow its projection directly)
 __global__ void k_zero_g2d(const uint32_t *vis_pair, const DevState *st, float *g2d) {
@@ -1291,7 +1324,7 @@ RasterKernel fwd_kernel(const gs_workspace *ws, bool var) {
         if (!var)
             return tiles >= kFwdWholeTiles ? fwd_variant<TW, TH, 4, false>(d)
                    : tiles >= kFwdHalfTiles ? fwd_variant<TW, TH, 2, false>(d) : fwd_variant<TW, TH, 1, false>(d);
-        return tiles >= kCoarseTiles ? fwd_variant<TW, TH, 2, true>(d) : fwd_variant<TW, TH, 1, true>(d);
+        return tiles >= kVarHalfTiles ? fwd_variant<TW, TH, 2, true>(d) : fwd_variant<TW, TH, 1, true>(d);
     }
     else {
         const size_t smem = (size_t)d * 3 * sizeof(float4);
@@ -1299,31 +1332,30 @@ RasterKernel fwd_kernel(const gs_workspace *ws, bool var) {
     }
 }
 
-// The backward's: quadrants a warp, or one a warp in pairs of entries.
-template <int TW, int TH, int Q, bool VAR>
-RasterKernel bwd_variant(int depth) {
-    const int d = std::min(depth, kBwdDepth<Q>);
-    using S = Share<TW, TH, Q>;
-    const size_t batch = S::NW > 1 ? (size_t)S::NW * d * kGrad * sizeof(float) : 0;
-    return {k_raster_bwd<TW, TH, Q, VAR>, S::NT, d,
-            (size_t)d * (sizeof(BwdEntry) + sizeof(uint32_t)) + S::NW * kSumBytes + batch};
-}
+// The backward's.
 template <int TW, int TH, bool VAR>
 RasterKernel bwd_pairs_variant(int depth, int64_t n_tiles) {
-    const bool deep = TW * TH < 256 ? n_tiles < 4 * kCoarseTiles : n_tiles <= kDeepTiles;
-    const int d = std::min(depth, deep ? kPairsDepth : TW * TH < 256 ? kPairsDepth / 4 : kPairsDepth / 2);
+    const int d = std::min(depth, TW * TH < 256 || n_tiles <= kDeepTiles ? kPairsDepth : kPairsDepth / 2);
     using S = Share<TW, TH, 1>;
     const size_t batch = S::NW > 1 ? (size_t)S::NW * d * kGrad * sizeof(float) : 0;
     return {k_raster_bwd_pairs<TW, TH, VAR>, S::NT, d,
             (size_t)d * (sizeof(BwdEntry) + 3 * sizeof(float4) + sizeof(uint32_t)) + S::NW * kSumBytes + batch};
 }
+// Pixels a thread of the column variant.  More amortise the reduction and the
+// shared-memory reads (500k orchard, 16x16 tiles: 4 -> 0.467 ms, 8, one warp a
+// tile, 0.435); the VAR variant holds three more values a pixel and keeps 4 (8
+// spills); an 8x8 tile keeps 2 so that its CTA is a whole warp.
+template <int TW, int TH, bool VAR>
+RasterKernel bwd_columns_variant(int depth) {
+    constexpr int PPT = TW * TH >= 256 ? (VAR ? 4 : 8) : 2;
+    return {k_raster_bwd<TW, TH, PPT, VAR>, TW * TH / PPT, depth,
+            (size_t)depth * (3 * sizeof(float4) + sizeof(float2) + sizeof(uint32_t))};
+}
 template <int TW, int TH>
 RasterKernel bwd_kernel(const gs_workspace *ws, bool var) {
     const int d = ws->cfg.batch_depth;
-    if constexpr (TW * TH >= 256) {
-        if (ws->n_tiles * (TW * TH / 256) >= kCoarseTiles)
-            return var ? bwd_variant<TW, TH, 2, true>(d) : bwd_variant<TW, TH, 4, false>(d);
-    }
+    if (ws->n_tiles * (TW * TH) / 256 >= kColumnTiles)
+        return var ? bwd_columns_variant<TW, TH, true>(d) : bwd_columns_variant<TW, TH, false>(d);
     return var ? bwd_pairs_variant<TW, TH, true>(d, ws->n_tiles) : bwd_pairs_variant<TW, TH, false>(d, ws->n_tiles);
 }
 
