@@ -1302,19 +1302,23 @@ __global__ void k_zero_g2d(const uint32_t *vis_pair, const DevState *st, float *
         g2d[(size_t)vis_pair[i / kGrad] * kGrad + i % kGrad] = 0.f;
 }
 
-// The kernel of one pass for a tile size, with its launch shape.
+// The kernel of one pass for a tile size, with its launch shape.  The limit on
+// a kernel's dynamic shared memory belongs to the function, not to a
+// workspace: smem_most is what its largest depth takes, the same for every
+// workspace, so that opening one never lowers the limit under another.
 struct RasterKernel {
     void (*fn)(RasterArgs);
     int threads, depth;  // depth: entries staged at a time
-    size_t smem;
+    size_t smem, smem_most;
 };
+constexpr int kMostDepth = 256;  // of the configuration (see check_config)
 
 // The forward's quadrants a warp.
 template <int TW, int TH, int Q, bool VAR>
 RasterKernel fwd_variant(int depth) {
     const int d = std::min(depth, kFwdDepth);
-    return {k_raster_fwd<TW, TH, Q, VAR>, Share<TW, TH, Q>::NT, d,
-            (size_t)d * (sizeof(FwdEntry) + sizeof(uint32_t))};
+    constexpr size_t entry = sizeof(FwdEntry) + sizeof(uint32_t);
+    return {k_raster_fwd<TW, TH, Q, VAR>, Share<TW, TH, Q>::NT, d, d * entry, kFwdDepth * entry};
 }
 template <int TW, int TH>
 RasterKernel fwd_kernel(const gs_workspace *ws, bool var) {
@@ -1327,8 +1331,9 @@ RasterKernel fwd_kernel(const gs_workspace *ws, bool var) {
         return tiles >= kVarHalfTiles ? fwd_variant<TW, TH, 2, true>(d) : fwd_variant<TW, TH, 1, true>(d);
     }
     else {
-        const size_t smem = (size_t)d * 3 * sizeof(float4);
-        return {var ? k_raster_fwd_columns<TW, TH, 2, true> : k_raster_fwd_columns<TW, TH, 2, false>, TW * TH / 2, d, smem};
+        constexpr size_t entry = 3 * sizeof(float4);
+        return {var ? k_raster_fwd_columns<TW, TH, 2, true> : k_raster_fwd_columns<TW, TH, 2, false>, TW * TH / 2, d,
+                d * entry, kMostDepth * entry};
     }
 }
 
@@ -1337,9 +1342,10 @@ template <int TW, int TH, bool VAR>
 RasterKernel bwd_pairs_variant(int depth, int64_t n_tiles) {
     const int d = std::min(depth, TW * TH < 256 || n_tiles <= kDeepTiles ? kPairsDepth : kPairsDepth / 2);
     using S = Share<TW, TH, 1>;
-    const size_t batch = S::NW > 1 ? (size_t)S::NW * d * kGrad * sizeof(float) : 0;
-    return {k_raster_bwd_pairs<TW, TH, VAR>, S::NT, d,
-            (size_t)d * (sizeof(BwdEntry) + 3 * sizeof(float4) + sizeof(uint32_t)) + S::NW * kSumBytes + batch};
+    constexpr size_t entry = sizeof(BwdEntry) + 3 * sizeof(float4) + sizeof(uint32_t) +
+                             (S::NW > 1 ? S::NW * kGrad * sizeof(float) : 0);
+    constexpr size_t sums = S::NW * kSumBytes;
+    return {k_raster_bwd_pairs<TW, TH, VAR>, S::NT, d, d * entry + sums, kPairsDepth * entry + sums};
 }
 // Pixels a thread of the column variant.  More amortise the reduction and the
 // shared-memory reads (500k orchard, 16x16 tiles: 4 -> 0.467 ms, 8, one warp a
@@ -1348,8 +1354,8 @@ RasterKernel bwd_pairs_variant(int depth, int64_t n_tiles) {
 template <int TW, int TH, bool VAR>
 RasterKernel bwd_columns_variant(int depth) {
     constexpr int PPT = TW * TH >= 256 ? (VAR ? 4 : 8) : 2;
-    return {k_raster_bwd<TW, TH, PPT, VAR>, TW * TH / PPT, depth,
-            (size_t)depth * (3 * sizeof(float4) + sizeof(float2) + sizeof(uint32_t))};
+    constexpr size_t entry = 3 * sizeof(float4) + sizeof(float2) + sizeof(uint32_t);
+    return {k_raster_bwd<TW, TH, PPT, VAR>, TW * TH / PPT, depth, depth * entry, kMostDepth * entry};
 }
 template <int TW, int TH>
 RasterKernel bwd_kernel(const gs_workspace *ws, bool var) {
@@ -1400,7 +1406,7 @@ gs_status raster_configure(gs_workspace *ws) {
     for (int i = 0; i < 4 && e == cudaSuccess; ++i) {
         const bool forward = i < 2, var = i & 1;
         const RasterKernel k = raster_kernel(ws, forward, var);
-        e = cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem);
+        e = cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem_most);
         int occ = 0;
         if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k.fn, k.threads, k.smem);
         int32_t &grid = forward ? (var ? ws->raster_grid_fwd_var : ws->raster_grid_fwd)
