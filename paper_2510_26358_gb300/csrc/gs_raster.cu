@@ -269,6 +269,9 @@ __global__ void __launch_bounds__(Share<TW, TH, Q>::NT, fwd_blocks(Share<TW, TH,
             }
             if (__any_sync(0xffffffffu, fmaxf(thr[q][0], thr[q][1]) > -INFINITY)) live |= 1u << q;
         }
+        // entries worked since the quadrants were last looked at: counted across
+        // batches, so that a warp which few entries of each reach leaves too
+        int since = 0;
         for (uint32_t b0 = rg.x; b0 < rg.y; b0 += A.depth) {
             if (__syncthreads_and(live == 0)) break;
             const int nb = min((int)(rg.y - b0), A.depth);
@@ -298,7 +301,6 @@ __global__ void __launch_bounds__(Share<TW, TH, Q>::NT, fwd_blocks(Share<TW, TH,
                     todo |= E[q];
                     all &= E[q];
                 }
-                int since = 0;
                 while (todo) {
                     const int j = __ffs(todo) - 1;
                     todo &= todo - 1;
@@ -430,7 +432,7 @@ __global__ void __launch_bounds__(Share<TW, TH, Q>::NT, fwd_blocks(Share<TW, TH,
                             M2[q] = f2_pack(v[0], v[1]);
                         }
                     }
-                    // quadrants whose pixels have all ended leave the walk
+                    // every eight entries, quadrants whose pixels have all ended leave the walk
                     if (++since == 8) {
                         since = 0;
                         uint32_t left = 0;
