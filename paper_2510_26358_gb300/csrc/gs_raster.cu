@@ -72,9 +72,13 @@ constexpr int kFwdDepth = 64, kPairsDepth = 128;
 // registers) 2400 tiles 73, 97; 7200 139, 107.
 constexpr int kFwdHalfTiles = 152 * 16, kFwdWholeTiles = 152 * 256, kVarHalfTiles = 152 * 24;
 // The backward works pairs of entries below kColumnTiles (16x16 tiles, or as many
-// pixels) and columns of pixels from there on.  kDeepTiles, in tiles of any
+// pixels) and columns of pixels from there on; 8x8 tiles, whose lists are short
+// and whose pairs have fewest entries to share a flush, take columns from
+// kColumnTiles8 of them on (pairs, columns, us, orchard of 200k, 640x480 views: 4800
+// tiles 39, 66; 9600 104, 96; 14,400 203, 178; with the variance 41, 66; 113, 100; 219,
+// 188).  16x16: 2400 tiles 84, 184; 3600 172, 354.  kDeepTiles, in tiles of any
 // size (CTAs): see kPairsDepth.
-constexpr int kColumnTiles = 152 * 24, kDeepTiles = 152 * 3;
+constexpr int kColumnTiles = 152 * 24, kColumnTiles8 = 152 * 48, kDeepTiles = 152 * 3;
 
 // Resident warps an SM that each variant's registers are bounded for, as CTAs
 // (forward, 4M orchard: 20 warps of whole tiles 0.94 ms, 24 0.99 ms with spills,
@@ -1362,7 +1366,7 @@ RasterKernel bwd_columns_variant(int depth) {
 template <int TW, int TH>
 RasterKernel bwd_kernel(const gs_workspace *ws, bool var) {
     const int d = ws->cfg.batch_depth;
-    if (ws->n_tiles * (TW * TH) / 256 >= kColumnTiles)
+    if (TW * TH < 256 ? ws->n_tiles >= kColumnTiles8 : ws->n_tiles * (TW * TH / 256) >= kColumnTiles)
         return var ? bwd_columns_variant<TW, TH, true>(d) : bwd_columns_variant<TW, TH, false>(d);
     return var ? bwd_pairs_variant<TW, TH, true>(d, ws->n_tiles) : bwd_pairs_variant<TW, TH, false>(d, ws->n_tiles);
 }
