@@ -295,7 +295,7 @@ gs_status gs_workspace_create(const gs_camera *cams, int32_t n_views, const int6
     GS_ALLOC(ws->part, (size_t)std::max(ws->sort_blocks, ws->wide_blocks) + 1);
     GS_ALLOC(ws->digit_tot, (size_t)512);
     GS_ALLOC(ws->pose_part, (size_t)std::max(1, blocks) * maxv * 6);
-    GS_ALLOC(ws->red_part, (size_t)2 * ws->sort_blocks);
+    GS_ALLOC(ws->red_part, (size_t)red_part_count(ws->sort_blocks));
     const std::vector<int4> tiles = ssim_tiles(ws->views_h);
     ws->n_ssim_tiles = (int64_t)tiles.size();
     GS_ALLOC(ws->ssim_tile, tiles.size());

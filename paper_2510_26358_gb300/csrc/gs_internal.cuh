@@ -42,6 +42,13 @@ struct DevState {
     uint32_t pad[4];
     unsigned long long frag_count[4];  // gs_workspace_fragment_counts
 };
+// Doubles of gs_workspace::red_part: two partials a block of the loss kernels
+// (sort_blocks of them: few on a GPU with few SMs), or one a block and then the
+// image loss's last sums, two a slice.
+constexpr int kImageLossSlices = 32;
+constexpr int64_t red_part_count(int64_t sort_blocks) {
+    return sort_blocks + (sort_blocks > 2 * kImageLossSlices ? sort_blocks : 2 * kImageLossSlices);
+}
 constexpr uint32_t kFlagCapacity = 1u;
 constexpr int kEmitWindow = 1024;      // output slots per emission window
 constexpr uint32_t kFlagTimeout = 2u;  // a bounded device wait (TMA) gave up
@@ -92,7 +99,7 @@ struct gs_workspace {
     uint32_t *part = nullptr;      // [max(sort_blocks, wide_blocks) + 1]
     uint32_t *digit_tot = nullptr; // [512] digit totals of the current radix pass
     float *pose_part = nullptr;    // [proj_blocks][max_views_per_submap][6]
-    double *red_part = nullptr;    // [2][sort_blocks] loss partials
+    double *red_part = nullptr;    // [red_part_count(sort_blocks)] loss partials
     int64_t n_ssim_tiles = 0;      // 32x32 SSIM tiles over all channel planes
     int4 *ssim_tile = nullptr;     // [n_ssim_tiles] where each lies
     float *ssim_d = nullptr;       // [3][3 n_pix] SSIM partials for the backward

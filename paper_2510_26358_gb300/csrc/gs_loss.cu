@@ -324,7 +324,7 @@ __global__ void __launch_bounds__(LT) k_l1_partial(const float *rgb, const TT *t
 // FP64 adds, two a clock an SM: one block for the 2 x 8280 partials of three
 // 1280x720 views took 10 us, 7 this way.  The last CTA of the SSIM kernel doing
 // it instead cost every CTA a fence and an atomic: 100 -> 124 us.)
-constexpr int kFinalBlocks = 32;
+constexpr int kFinalBlocks = kImageLossSlices;
 __global__ void __launch_bounds__(LT) k_image_loss_final(const double *l1part, int64_t nl, const double *spart,
                                                         int64_t ns, int64_t n, float lambda, double *slice,
                                                         uint32_t *done, float *loss) {
@@ -449,7 +449,7 @@ gs_status launch_image_loss(gs_workspace *ws, const float *rgb, const float *tar
     if (r == GS_OK) r = launch_ssim(ws, rgb, target, lambda, fused ? dL_drgb : nullptr, s);
     if (r != GS_OK) return r;
     ++ws->kernel_launches;
-    // (the slices' sums after the L1 kernel's partials: 2 sort_blocks doubles)
+    // (the slices' sums after the L1 kernel's partials)
     k_image_loss_final<<<kFinalBlocks, LT, 0, s>>>(l1part, nl, ws->ssim_part, ns, n, lambda,
                                                    ws->red_part + ws->sort_blocks, &ws->st->done_l1, loss);
     return check_launch("image_loss");
