@@ -431,7 +431,10 @@ gs_status gs_zero_buffers(void *const *ptrs, const int64_t *bytes, int32_t count
  * events on its stream around every stage below (do not enable it while
  * capturing a CUDA graph); gs_workspace_stage_ms synchronises on the events
  * and writes the last duration of each stage in milliseconds (-1 if the
- * stage has not run since profiling was enabled). */
+ * stage has not run since profiling was enabled).  A stage whose work another
+ * stage's kernel takes along reads the time between its two events: compaction
+ * up to 16,384 (view, Gaussian) pairs (the depth sort's launch does it), the L1
+ * term of gs_image_loss where SSIM is in the gradient (the SSIM kernels do). */
 enum {
     GS_STAGE_PROJECT = 0,    /* gs_project */
     GS_STAGE_COMPACT = 1,    /* visible-pair compaction */
@@ -440,7 +443,7 @@ enum {
     GS_STAGE_TILE_SORT = 4,  /* radix sort of instances by tile */
     GS_STAGE_RANGES = 5,     /* per-tile ranges */
     GS_STAGE_RASTER_FWD = 6, /* forward compositing */
-    GS_STAGE_IMAGE_L1 = 7,   /* gs_image_l1 */
+    GS_STAGE_IMAGE_L1 = 7,   /* gs_image_l1, L1 term of gs_image_loss */
     GS_STAGE_DEPTH_LOSS = 8, /* gs_depth_loss */
     GS_STAGE_ZERO_GRAD = 9,  /* clearing the image-space gradients */
     GS_STAGE_RASTER_BWD = 10, /* backward compositing */

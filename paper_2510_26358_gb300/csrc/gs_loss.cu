@@ -437,14 +437,16 @@ gs_status launch_image_loss(gs_workspace *ws, const float *rgb, const float *tar
     const double *l1part = ws->ssim_part + ns;
     int64_t nl = ns;
     gs_status r = GS_OK;
-    if (!fused) {
-        StageTimer timer(ws, GS_STAGE_IMAGE_L1, s);
-        ++ws->kernel_launches;
-        l1part = ws->red_part;
-        nl = ws->sort_blocks;
-        k_l1_partial<float><<<(int)nl, LT, 0, s>>>(rgb, target, n, dL_drgb, ws->red_part,
-                                                   (float)((1.0 - (double)lambda) / (double)n), nullptr, nullptr);
-        r = check_launch("image_loss");
+    {
+        StageTimer timer(ws, GS_STAGE_IMAGE_L1, s);  // (a stage that ran reads a time, however short)
+        if (!fused) {
+            ++ws->kernel_launches;
+            l1part = ws->red_part;
+            nl = ws->sort_blocks;
+            k_l1_partial<float><<<(int)nl, LT, 0, s>>>(rgb, target, n, dL_drgb, ws->red_part,
+                                                       (float)((1.0 - (double)lambda) / (double)n), nullptr, nullptr);
+            r = check_launch("image_loss");
+        }
     }
     if (r == GS_OK) r = launch_ssim(ws, rgb, target, lambda, fused ? dL_drgb : nullptr, s);
     if (r != GS_OK) return r;

@@ -1000,6 +1000,7 @@ gs_status launch_bin_sort(gs_workspace *ws, cudaStream_t s) {
     const uint32_t *v = ws->vis_pair;  // the visible pairs in depth order
     if (n_pairs <= (uint32_t)kSmallPairs) {
         // 1-3 (up to the offsets) in one launch
+        { StageTimer none(ws, GS_STAGE_COMPACT, s); }  // (a stage that ran reads a time)
         StageTimer timer(ws, GS_STAGE_DEPTH_SORT, s);
         ++ws->kernel_launches;
         k_bin_small<<<1, kSmallThreads, sizeof(SmallSmem), s>>>(ws->pkey, n_pairs, ws->rect, st, cap, ws->vis_pair,
