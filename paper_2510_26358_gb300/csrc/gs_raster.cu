@@ -58,31 +58,32 @@ constexpr float kQuadRelPad = 1e-3f, kQuadAbsPad = 1e-2f;
 // The backward in pairs of entries takes all of kPairsDepth where few tiles leave
 // the SMs idle anyway, and less where more CTAs an SM are worth more (128, 64, 32
 // entries, us): 300 tiles of 16x16 54, 68, 71; 3600 127, 118, 120; 8x8: 4270 380, 409,
-// 410; 9900 461, 497, 524.  (Its other backward takes the configuration's depth.)
+// 410.  (The backward by columns takes the configuration's depth.)
 constexpr int kFwdDepth = 64, kPairsDepth = 128;
 
-// How many quadrants a warp takes, by the number of 16x16 tiles (or as many
-// pixels).  Whole tiles share the most work between quadrants but make the
+// How many quadrants a warp of the forward takes, by the number of 16x16 tiles
+// (or as many pixels), in multiples of the measured GPU's 152 SMs.  Whole tiles share the most work between quadrants but make the
 // fewest warps: with few tiles the time is the longest list's chain of
 // entries, which is shorter the less a warp does for each.  Measured (one,
-// two, four quadrants a warp, us).  Forward, the whole step: 300 tiles (320x240,
+// two, four quadrants a warp, us).  The whole step: 300 tiles (320x240,
 // box of 10k) 288, 298, -; 1200 (orchard of 200k, as below) 247, 258, -; 2400
 // 318, 319, -; 3600 249, 247, -; the kernel: 7200 87, 64, 75; 24,480 (1M) -, 391,
 // 406; 54,000 (4M) -, 971, 936.  With the variance (one, two; more do not fit the
 // registers) 2400 tiles 73, 97; 7200 139, 107.
 constexpr int kFwdHalfTiles = 152 * 16, kFwdWholeTiles = 152 * 256, kVarHalfTiles = 152 * 24;
 // The backward works pairs of entries below kColumnTiles (16x16 tiles, or as many
-// pixels) and columns of pixels from there on; 8x8 tiles, whose lists are short
-// and whose pairs have fewest entries to share a flush, take columns from
-// kColumnTiles8 of them on (pairs, columns, us, orchard of 200k, 640x480 views: 4800
-// tiles 39, 66; 9600 104, 96; 14,400 203, 178; with the variance 41, 66; 113, 100; 219,
-// 188).  16x16: 2400 tiles 84, 184; 3600 172, 354.  kDeepTiles, in tiles of any
-// size (CTAs): see kPairsDepth.
+// pixels), where that takes half of the time, and columns of pixels from there
+// on, where the sums' order must stay (see k_raster_bwd).  8x8 tiles take columns
+// from kColumnTiles8 of them on, where those are the faster ones.  Pairs, columns,
+// us, orchard of 200k, one to three 640x480 views, without and with the variance:
+// 16x16 1200 tiles 55, 145 and 57, 102; 2400 84, 184 and 88, 139; 3600 172, 354 and 184, 276;
+// 8x8 4800 39, 66 and 41, 66; 9600 104, 96 and 113, 100; 14,400 203, 178 and 219, 188.
+// kDeepTiles counts tiles of any size, as CTAs: see kPairsDepth.
 constexpr int kColumnTiles = 152 * 24, kColumnTiles8 = 152 * 48, kDeepTiles = 152 * 3;
 
 // Resident warps an SM that each variant's registers are bounded for, as CTAs
-// (forward, 4M orchard: 20 warps of whole tiles 0.94 ms, 24 0.99 ms with spills,
-// 16 1.23 ms).
+// (4M orchard: 20 warps of whole tiles 0.94 ms, with 24 bytes spilled, 24 0.99 ms
+// with more, 16 1.23 ms; 32-pixel tiles spill up to 28 bytes with one or two).
 constexpr int fwd_blocks(int warps, int q, bool var) {
     return (var ? (q == 4 ? 16 : 20) : (q == 4 ? 20 : q == 2 ? 28 : 40)) / warps;
 }
@@ -1034,7 +1035,8 @@ __device__ __forceinline__ int reduce10_component(int lane) {
 // in another order of the terms the quaternion gradients of that step changed by
 // up to 1.6e-4 in norm (240 random maps; repeating the same order changes them by
 // 1e-6, and one map in eight passed 2e-5 in norm or 8e-4 at an element).  Below
-// kColumnTiles no Gaussian covers that many tiles, and the other order stays inside.
+// kColumnTiles a Gaussian covers fewer tiles, and some 360 gradients in the other
+// order stayed inside.
 // The terms, their order inside a warp, and the float rows are therefore fixed.
 //
 // At least 512 resident threads per SM (16 warps, 128 registers a thread):

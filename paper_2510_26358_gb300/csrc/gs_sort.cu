@@ -12,8 +12,10 @@
 // Per-tile ranges come from key changes.
 //
 // Every count lives on the device (capacity overflow sets a flag), so the
-// sequence needs no host round trip and can be captured in a CUDA graph.  All
-// kernels run a fixed grid of `sort_blocks` blocks, each owning a contiguous
+// sequence needs no host round trip and can be captured in a CUDA graph.  Every
+// kernel runs a grid fixed with the workspace (up to wide_blocks for compaction,
+// depth sort and offsets, 2 x sort_blocks for the instance sort, some blocks an
+// SM for emission and ranges); a counting or scatter block owns a contiguous
 // chunk of ceil(n / blocks) rounded to a whole tile.
 //
 // The radix sort is a reduce-then-scan LSD sort with 8- or 9-bit digits:
@@ -510,9 +512,9 @@ __global__ void __launch_bounds__(T) k_instance_offsets(const DevState *st, cons
 // A rectangle tile that the Gaussian's padded alpha >= alpha_min ellipse
 // misses (about a fifth of them on wide scenes: the corners of the rectangles
 // of large or tilted ellipses) is written with tile id kInvalidKey.  The tile
-// sort puts these after every real tile (the sort covers whole bytes above
-// the highest tile id), the ranges skip them, and the rasterisers never walk
-// them.
+// sort puts these after every real tile (its digits cover at least tile_bits,
+// the bits of the value n_tiles, and those of the all-ones id exceed every
+// real one's), the ranges skip them, and the rasterisers never walk them.
 
 // Blocks of the emission an SM keeps resident: a window's staging is a short
 // chain of dependent loads (slot owners, pair ids, rectangles) that every
@@ -1007,8 +1009,8 @@ gs_status launch_bin_sort(gs_workspace *ws, cudaStream_t s) {
                                                                 ws->ioff, ws->win_pair, n_win);
         if ((r = check_launch("bin_small")) != GS_OK) return r;
     } else {
-        // 1. compaction of visible pairs (more blocks than the other stages: each
-        //    block's chunk is a chain of block-wide scans)
+        // 1. compaction of visible pairs (more blocks than the instance sort: a
+        //    block's chunk is a chain of steps with a barrier each)
         {
             StageTimer timer(ws, GS_STAGE_COMPACT, s);
             ws->kernel_launches += 2;

@@ -6,14 +6,15 @@
 // s_xy = E[xy] - mu_x mu_y,
 //   S = (2 mu_x mu_y + C1)(2 s_xy + C2) / ((mu_x^2 + mu_y^2 + C1)(s_xx + s_yy + C2)).
 //
-// Forward: one CTA per 32x16 output tile of one channel plane stages the tile
+// Forward: one CTA per 32x32 output tile of one channel plane stages the tile
 // and its 5-pixel halo of x and y in shared memory, filters x, y, x^2 + y^2 and xy
 // horizontally, then vertically, and writes S's partial derivatives w.r.t.
 // the three window sums that depend on x,
 //   d1 = dS/dE[x],  d2 = dS/dE[x^2],  d12 = dS/dE[xy],
-// plus a per-CTA sum of 1 - S (double).  Backward: the same tiling filters
-// (d1, d2, d12) with the same window (the adjoint of a zero-padded symmetric
-// filter is itself) and adds scale * (G*d1 + 2 x G*d2 + y G*d12) to dL/dx.
+// plus per-CTA sums of 1 - S and |x - y| (double).  Backward: the same tiling
+// filters (d1, d2, d12) with the same window (the adjoint of a zero-padded
+// symmetric filter is itself) and adds scale * (G*d1 + 2 x G*d2 + y G*d12) and the
+// L1 term's step to dL/dx.
 //
 // Precision: E[x^2] - mu_x^2 cancels in float where the image is smooth
 // (variances of 1e-5 against E[x^2] ~ 0.3, which cost 1e-4 of 1 - SSIM near
@@ -52,7 +53,7 @@ constexpr int BOFF = 3;       // halo column c lives at staged column c + BOFF
 constexpr int HW = TX + 4;    // filtered row stride (16-byte pieces)
 constexpr int NT = 256;
 constexpr int HB = 4;                     // horizontal outputs per thread
-constexpr int HITEMS = IH * (TX / HB);    // 208 row segments per tile
+constexpr int HITEMS = IH * (TX / HB);    // 336 row segments per tile
 constexpr int VB = 4;                     // vertical outputs per thread (consecutive rows)
 constexpr int SLOADS = (IH * IW + NT - 1) / NT;  // staged values per thread and map
 static_assert(TY == VB * (NT / TX), "one vertical pass covers the tile");

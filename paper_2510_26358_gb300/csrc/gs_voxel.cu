@@ -18,7 +18,7 @@
 //      (rgb - 1/2) / Y00, higher coefficients 0.
 // LRU selection: with n > tau splats, the (n - tau) smallest (last_used,
 // index) pairs are flagged, by an exact radix select of the last_used value
-// (four 8-bit passes) and an ordered count of the ties.
+// (three passes of 11, 11 and 10 bits) and an ordered count of the ties.
 // Partition: a stable split of the splat rows by a flag array into a kept and
 // a moved set; either side may live in host-mapped memory (offload, reload).
 #include "gs_internal.cuh"
