@@ -1028,8 +1028,8 @@ __device__ __forceinline__ int reduce10_component(int lane) {
 
 // The backward of renders of kColumnTiles and more: a thread works PPT pixels of
 // a column, a warp's sums go to the rows by one butterfly an entry.  Quadrants
-// and sums about their middle, added to rows in double, took 1558 us where this
-// takes 1841 (4M orchard, six 1920x1200 views) and come nearer to 64 bits, but
+// and sums about their middle, added to rows in double, took 1559 us where this
+// takes 1870 (4M orchard, six 1920x1200 views) and come nearer to 64 bits, but
 // move results that must stay where they are: the gradients of a long thin
 // Gaussian near a camera are sums over thousands of tiles that largely cancel, and
 // in another order of the terms the quaternion gradients of that step changed by
