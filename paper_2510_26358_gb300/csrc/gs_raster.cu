@@ -1034,10 +1034,10 @@ __device__ __forceinline__ int reduce10_component(int lane) {
 // Gaussian near a camera are sums over thousands of tiles that largely cancel, and
 // in another order of the terms the quaternion gradients of that step changed by
 // up to 1.6e-4 in norm (240 random maps; repeating the same order changes them by
-// 1e-6, and one map in eight passed 2e-5 in norm or 8e-4 at an element).  Below
-// kColumnTiles a Gaussian covers fewer tiles, and some 360 gradients in the other
-// order stayed inside.
-// The terms, their order inside a warp, and the float rows are therefore fixed.
+// 1e-6, 3e-5 at most, and one map in eight passed 2e-5 in norm or 8e-4 at an
+// element by more than that).  Below kColumnTiles a Gaussian covers fewer tiles,
+// and some 360 gradients in the other order stayed inside.  The terms, their order
+// inside a warp, and the float rows are therefore fixed.
 //
 // At least 512 resident threads per SM (16 warps, 128 registers a thread):
 // with eight pixels a thread, measured best on the 500k orchard (16 one-warp
