@@ -78,6 +78,8 @@ constexpr int kFwdHalfTiles = 152 * 16, kFwdWholeTiles = 152 * 256, kVarHalfTile
 // us, orchard of 200k, one to three 640x480 views, without and with the variance:
 // 16x16 1200 tiles 55, 145 and 57, 102; 2400 84, 184 and 88, 139; 3600 172, 354 and 184, 276;
 // 8x8 4800 39, 66 and 41, 66; 9600 104, 96 and 113, 100; 14,400 203, 178 and 219, 188.
+// (8x8 with long lists: 800k, 4800 tiles 164, 209; 6300 154, 183; of 1.3M in 2135 to 6405
+// tiles one list's walk sets the time, 395 to 420 either way.)
 // kDeepTiles counts tiles of any size, as CTAs: see kPairsDepth.
 constexpr int kColumnTiles = 152 * 24, kColumnTiles8 = 152 * 48, kDeepTiles = 152 * 3;
 
